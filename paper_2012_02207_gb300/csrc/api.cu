@@ -534,7 +534,7 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
         (rc = ensure(ctx, ctx->M, 8 * K)) || (rc = ensure(ctx, ctx->S, 24 * K)) ||
         (rc = ensure(ctx, ctx->zc, 24 * K)) || (rc = ensure(ctx, ctx->r, 8 * K)) || (rc = ensure(ctx, ctx->hs, 8 * K)) ||
         (rc = ensure(ctx, ctx->Pk, 8 * K * (p + 1))) || (rc = ensure(ctx, ctx->mult, 8 * K * nr)) ||
-        (rc = ensure(ctx, ctx->fmin, 4 * K)) || (rc = ensure(ctx, ctx->fscratch, 4 * (2 * K + N))) ||
+        (rc = ensure(ctx, ctx->fmin, 4 * K)) || (rc = ensure(ctx, ctx->fscratch, 4 * 2 * K)) ||
         (rc = ensure(ctx, ctx->zhi, 16 * K)) || (rc = ensure(ctx, ctx->zlo, 16 * K)) ||
         (rc = ensure(ctx, ctx->contrib, 8 * K * nr)) || (rc = ensure(ctx, ctx->Phat, 4 * K * (p + 1))) ||
         (rc = ensure(ctx, ctx->r32, 4 * K)) || (rc = ensure(ctx, ctx->geo, sizeof(double) * kShiftGeo * K)) ||
