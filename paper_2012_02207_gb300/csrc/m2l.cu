@@ -17,11 +17,9 @@
 //
 // One warp per target cell gathers over the target's sources (sorted by
 // index); lane l takes sources l, l+32, ... and accumulates its own partial
-// local expansion; the 32 partials are summed by a fixed butterfly (FP32 in
-// the FP32 kernel, FP64 in the FP64 one), so the result does not depend on
-// scheduling.
+// local expansion; the 32 partials are summed by a fixed butterfly, so the
+// result does not depend on scheduling. This file holds the FP32 kernel; m2l64.cu the FP64 one.
 #include "gbfmm_internal.cuh"
-#include "swap_tables.cuh"
 
 namespace gbfmm {
 
@@ -173,132 +171,6 @@ __global__ void __launch_bounds__(128, m2l_min_blocks(P)) k_m2l32(const int* __r
     }
 }
 
-// ------------------------------------------------------------------------
-// FP64, runtime order p <= 30: coefficients in per-thread local arrays.
-
-__device__ void rotz64(double* a, int p, double c, double s) {
-    double pr = 1.0, pi = 0.0;
-    for (int m = 1; m <= p; ++m) {
-        const double t = pr * c - pi * s;
-        pi = pr * s + pi * c;
-        pr = t;
-        for (int n = m; n <= p; ++n) {
-            const double re = a[hre(n, m)], im = a[him(n, m)];
-            a[hre(n, m)] = re * pr - im * pi;
-            a[him(n, m)] = re * pi + im * pr;
-        }
-    }
-}
-
-// after_z: the swap right after the z-translation, whose output F'_n^m
-// vanishes for m > p - n, so those inputs are skipped
-template <int PM>
-__device__ void swap64(double* a, int p, const Swap64& sw, bool after_z = false) {
-    double tc[PM + 1], ts[PM + 1];
-    for (int n = 1; n <= p; ++n) {
-        const double* A = sw.cosb + cos_off(n);
-        const double* B = sw.sinb + sin_off(n);
-        const int jmax = after_z && p - n < n ? p - n : n;
-        for (int m = 0; m <= n; ++m) {
-            double acc = 0.0;
-            for (int j = (m + n) & 1; j <= jmax; j += 2) acc += __ldg(A + m * (n + 1) + j) * a[hre(n, j)];
-            tc[m] = acc;
-        }
-        for (int m = 1; m <= n; ++m) {
-            double acc = 0.0;
-            for (int j = ((m + n + 1) & 1) ? 1 : 2; j <= jmax; j += 2)
-                acc += __ldg(B + (m - 1) * n + (j - 1)) * a[him(n, j)];
-            ts[m] = acc;
-        }
-        for (int m = 0; m <= n; ++m) a[hre(n, m)] = tc[m];
-        for (int m = 1; m <= n; ++m) a[him(n, m)] = ts[m];
-    }
-}
-
-template <int PM>
-__device__ void ztrans64(double* a, int p, double u, double v, double irho, const double* fact,
-                         const double* iw) {
-    double up[PM + 1], vp[PM + 1], tr[PM + 1], ti[PM + 1];
-    up[0] = 1.0;
-    vp[0] = irho;
-    for (int k = 1; k <= p; ++k) { up[k] = up[k - 1] * u; vp[k] = vp[k - 1] * v; }
-    for (int m = 0; m <= p; ++m) {
-        for (int k = m; k <= p; ++k) {
-            const double sg = ((k + m) & 1) ? -up[k] : up[k];
-            tr[k] = sg * a[hre(k, m)];
-            ti[k] = m ? sg * a[him(k, m)] : 0.0;
-        }
-        for (int n = m; n <= p; ++n) {
-            double sr = 0.0, si = 0.0;
-            const double iwn = __ldg(iw + n * (kMaxP + 2) + m);
-            for (int k = m; k <= p - n; ++k) {
-                const double cz = __ldg(fact + n + k) * iwn * __ldg(iw + k * (kMaxP + 2) + m);
-                sr += cz * tr[k];
-                si += cz * ti[k];
-            }
-            a[hre(n, m)] = vp[n] * sr;
-            if (m) a[him(n, m)] = vp[n] * si;
-        }
-    }
-}
-
-// PM bounds the per-thread arrays: p <= PM.
-template <int PM>
-__global__ void __launch_bounds__(64) k_m2l64(const int* __restrict__ dnn, int p, const uint32_t* __restrict__ src,
-                                               const uint32_t* __restrict__ off,
-                                               const double* __restrict__ mult,
-                                               const double* __restrict__ zc,
-                                               const double* __restrict__ hs,
-                                               double* __restrict__ loc, Swap64 sw,
-                                               const double* __restrict__ fact,
-                                               const double* __restrict__ iw, unsigned* __restrict__ queue) {
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int nr = ncoef_real(p);
-    double c[ncoef_real(PM)], acc[ncoef_real(PM)];
-    (void)wib;
-    for (;;) {
-        int b = 0;
-        if (lane == 0) b = (int)atomicAdd(queue, 1u);
-        b = __shfl_sync(0xffffffffu, b, 0);
-        if (b >= *dnn) break;
-        for (int j = 0; j < nr; ++j) acc[j] = 0.0;
-        const uint32_t q0 = off[b], q1 = off[b + 1];
-        const double bx = zc[3 * b], by = zc[3 * b + 1], bz = zc[3 * b + 2];
-        const double sb = hs[b];
-        for (uint32_t q = q0 + lane; q < q1; q += 32) {
-            const int a = (int)src[q];
-            const double rx = zc[3 * a] - bx, ry = zc[3 * a + 1] - by, rz = zc[3 * a + 2] - bz;
-            const double sa = hs[a];
-            const double* mv = mult + (size_t)nr * a;
-            for (int j = 0; j < nr; ++j) c[j] = mv[j];
-            const double rxy2 = rx * rx + ry * ry;
-            const double rho = sqrt(rxy2 + rz * rz);
-            const double rxy = sqrt(rxy2);
-            double cp = 1.0, sp = 0.0;
-            if (rxy > 0.0) { cp = rx / rxy; sp = ry / rxy; }
-            const double ct = rz / rho, st = rxy / rho;
-            const double irho = 1.0 / rho;
-            rotz64(c, p, sp, cp);
-            swap64<PM>(c, p, sw);
-            rotz64(c, p, ct, -st);
-            swap64<PM>(c, p, sw);
-            ztrans64<PM>(c, p, sa * irho, sb * irho, irho, fact, iw);
-            swap64<PM>(c, p, sw, true);
-            rotz64(c, p, ct, st);
-            swap64<PM>(c, p, sw);
-            rotz64(c, p, sp, -cp);
-            for (int j = 0; j < nr; ++j) acc[j] += c[j];
-        }
-        double* out = loc + (size_t)nr * b;
-        for (int j = 0; j < nr; ++j) {
-            double v = acc[j];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) out[j] = v;
-        }
-    }
-}
-
 template <int P>
 void launch_m2l32(const int* dnn, const uint32_t* src, const uint32_t* off, const float* mult,
                   int stride, const float4* zhi, const float4* zlo, float* loc, unsigned* queue,
@@ -309,23 +181,6 @@ void launch_m2l32(const int* dnn, const uint32_t* src, const uint32_t* off, cons
      note_launch());
 }
 }  // namespace
-
-void m2l_f64(const int* dnn, int p, const uint32_t* src, const uint32_t* off,
-             const double* mult, const double* zc, const double* hs, double* loc,
-             const DevTables& tb, unsigned* queue, cudaStream_t st) {
-    const Swap64 sw{tb.swap_cos, tb.swap_sin};
-    cudaMemsetAsync(queue, 0, sizeof(unsigned), st);
-    if (p <= 8) {
-        (k_m2l64<8><<<device_sm_count() * 16, 64, 0, st>>>(dnn, p, src, off, mult, zc, hs, loc, sw, tb.fact, tb.iw, queue), note_launch());
-    } else if (p <= 16) {
-        (k_m2l64<16><<<device_sm_count() * 16, 64, 0, st>>>(dnn, p, src, off, mult, zc, hs, loc, sw, tb.fact, tb.iw, queue), note_launch());
-    } else {
-        // ~17 KB of local arrays per thread: a 48 KB shared-memory request caps
-        // residency at 4 blocks (256 threads) per SM to bound the local-memory reservation
-        ensure_dyn_smem((const void*)k_m2l64<kMaxP>, 48 * 1024);
-        (k_m2l64<kMaxP><<<device_sm_count() * 4, 64, 48 * 1024, st>>>(dnn, p, src, off, mult, zc, hs, loc, sw, tb.fact, tb.iw, queue), note_launch());
-    }
-}
 
 void m2l_f32(const int* dnn, int p, const uint32_t* src, const uint32_t* off,
              const float* mult, const float4* zhi, const float4* zlo, float* loc, unsigned* queue,
