@@ -375,9 +375,11 @@ void jerk_leaves(const LeafArgs& a, bool fp32, const void* locj, const double* v
                  const int* item_leaf, const uint32_t* item_first, const uint32_t* slot_first, const uint32_t* nitems,
                  unsigned* work, const int* leaf_of, double* jx, double* jy, double* jz, cudaStream_t st);
 // ------------------------------------------------------------- timestep.cu
-// HOLD step sizes: tau_i = min over j != i of the pair step (Appendix A)
+// HOLD step sizes: tau_i = min over j != i of the pair step (Appendix A);
+// upper: n words of scratch
 void timesteps_f64(int n, const double* x, const double* y, const double* z, const double* vx, const double* vy,
-                   const double* vz, const double* m, double G, double eta, bool sym, double* tau, cudaStream_t st);
+                   const double* vz, const double* m, double G, double eta, bool sym, double* tau,
+                   unsigned* upper, cudaStream_t st);
 // ----------------------------------------------------------------- hold.cu
 constexpr int kHoldMaxDepth = 60;                  // no set is split below this level
 constexpr int kHoldMaxLevels = kHoldMaxDepth + 1;  // frames of the device-resident recursion
