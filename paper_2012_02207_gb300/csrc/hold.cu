@@ -7,6 +7,7 @@
 // Compiled with -fmad=false: a drift x + dt v and a kick v + h a round as
 // two operations, as the oracle does.
 #include "gbfmm_internal.cuh"
+#include "hold_bounds.cuh"
 #include "hold_pair.cuh"
 
 namespace gbfmm {
@@ -92,8 +93,19 @@ __global__ void k_hold_iota(int n, int* __restrict__ idx) {
 // undone when the frame ends, so the parent sees its fast set in its own
 // order again, as the oracle (fresh S and F arrays per level) does. Forces
 // are the oracle's FP64 direct sum in the oracle's order and operations
-// (r = sqrt(r^2), m / (r^2 r), no contraction), the step sizes the same
-// tau_pair: the trajectory is the oracle's bit for bit.
+// (r = sqrt(r^2), m / (r^2 r), no contraction), and a body is fast when the same
+// tau_pair says so: the trajectory is the oracle's bit for bit.
+//
+// One SM's FP64 pipe (two lanes a clock) bounds it, and the latency of the
+// steps in the small sets deep in the recursion. So
+//  - the split needs only to know whether some pair step is below dt: FP32
+//    bounds (hold_bounds.cuh) decide nearly every pair, the rest are evaluated
+//    exactly;
+//  - a kick runs over the unordered pairs with a slow member, one thread each:
+//    r and r^3 serve both bodies, whose two terms go to shared memory, and one
+//    thread per body and component adds its terms in source order.
+// N = 100 (a Plummer sphere, dt = 1/16, one step): 30.1 -> 4.1 ms against one thread
+// per body, every pair step exact and every force pair from both sides.
 
 struct HoldFrame {
     double dt;
@@ -106,31 +118,121 @@ struct HoldFrame {
 
 constexpr int kHoldThreads = 256;
 
-// accelerations of the sinks ix[s0..s1) from the sources ix[q0..q1) (a body
-// does not act on itself), each sink kicked at once: v <- v + h G sum
-__device__ __forceinline__ void hold_kick_from(const int* ix, int s0, int s1, int q0, int q1, const double* px,
-                                               const double* py, const double* pz, const double* pm, double* pvx,
-                                               double* pvy, double* pvz, double G, double soft2, double h) {
-    for (int t = s0 + (int)threadIdx.x; t < s1; t += kHoldThreads) {
-        const int i = ix[t];
-        const double xi = px[i], yi = py[i], zi = pz[i];
-        double sx = 0.0, sy = 0.0, sz = 0.0;
-        for (int q = q0; q < q1; ++q) {
-            const int j = ix[q];
-            if (j == i) continue;
-            const double dx = px[j] - xi, dy = py[j] - yi, dz = pz[j] - zi;
+constexpr int kHoldPairs = 1024;  // pairs whose terms are in shared memory at a time (>= kHoldSmallMax)
+constexpr int kHoldUnsure = 256;  // pairs the bounds leave open, listed before they are evaluated
+
+// shared memory of a kick's terms or a split's FP32 members
+__host__ __device__ constexpr size_t hold_term_bytes(int k) {
+    return 6 * kHoldPairs * sizeof(double) > (size_t)k * sizeof(PairBody32) ? 6 * kHoldPairs * sizeof(double)
+                                                                           : (size_t)k * sizeof(PairBody32);
+}
+
+// Kick of the set ix[0..n), its first ns members slow: slow bodies feel
+// all of it, fast ones the slow ones; v <- v + h G sum, sources in set order,
+// a body not acting on itself. Rows a = 0..ns-1 of pairs (a, b), a < b, in
+// chunks: a chunk holds for each of its rows the pairs with every b > a, so a
+// body s adds its sources in order: those of the chunk's rows below s, then,
+// if s is itself a row of the chunk, those above s. acc: 3 n sums; term:
+// 6 kHoldPairs values (on a from b, then on b from a).
+__device__ void set_kick(const int* ix, int n, int ns, const double* px, const double* py, const double* pz,
+                          const double* pm, double* pvx, double* pvy, double* pvz, double G, double soft2, double h,
+                          double* acc, double* term) {
+    const int tid = threadIdx.x;
+    const int rows = kHoldPairs / n < ns ? kHoldPairs / n : ns;
+    for (int e = tid; e < 3 * n; e += kHoldThreads) acc[e] = 0.0;
+    for (int a0 = 0; a0 < ns; a0 += rows) {
+        const int a1 = a0 + rows < ns ? a0 + rows : ns;
+        for (int e = tid; e < (a1 - a0) * n; e += kHoldThreads) {
+            const int a = a0 + e / n, b = e % n;
+            if (b <= a) continue;
+            const int i = ix[a], j = ix[b];
+            const double dx = px[j] - px[i], dy = py[j] - py[i], dz = pz[j] - pz[i];
             double r2 = dx * dx + dy * dy + dz * dz;
             if (soft2 > 0.0) r2 = r2 + soft2;
             const double r = sqrt(r2);
-            const double mr3 = pm[j] / (r2 * r);
-            sx += mr3 * dx;
-            sy += mr3 * dy;
-            sz += mr3 * dz;
+            const double r3 = r2 * r;
+            const double ma = pm[j] / r3, mb = pm[i] / r3;
+            term[e] = ma * dx;
+            term[kHoldPairs + e] = ma * dy;
+            term[2 * kHoldPairs + e] = ma * dz;
+            // (the pair seen from b: exactly the opposite offsets)
+            term[3 * kHoldPairs + e] = mb * -dx;
+            term[4 * kHoldPairs + e] = mb * -dy;
+            term[5 * kHoldPairs + e] = mb * -dz;
         }
-        pvx[i] += h * (G * sx);
-        pvy[i] += h * (G * sy);
-        pvz[i] += h * (G * sz);
+        __syncthreads();
+        for (int e = a0 * 3 + tid; e < 3 * n; e += kHoldThreads) {  // bodies below a0 have all their sources
+            const int s = e / 3, c = e - 3 * s;
+            const double* on_b = term + (3 + c) * kHoldPairs + s;
+            const double* on_a = term + c * kHoldPairs + (s - a0) * n;
+            double v = acc[e];
+            for (int a = a0; a < a1 && a < s; ++a) v += on_b[(a - a0) * n];
+            if (s < a1)
+                for (int b = s + 1; b < n; ++b) v += on_a[b];
+            acc[e] = v;
+        }
+        __syncthreads();
     }
+    for (int s = tid; s < n; s += kHoldThreads) {
+        const int i = ix[s];
+        pvx[i] += h * (G * acc[3 * s]);
+        pvy[i] += h * (G * acc[3 * s + 1]);
+        pvz[i] += h * (G * acc[3 * s + 2]);
+    }
+    __syncthreads();
+}
+
+// The fast members of the set ix[0..n) as bits: those with a pair step below
+// dt. b32: the members in FP32 pairs (scratch), unsure: kHoldUnsure words.
+__device__ void set_fast_bits(const int* ix, int n, const double* px, const double* py, const double* pz,
+                               const double* pvx, const double* pvy, const double* pvz, const double* pm, double G,
+                               double eta, bool sym, double dt, PairBody32* b32, unsigned* bits, unsigned* unsure,
+                               int* nunsure) {
+    const int tid = threadIdx.x;
+    for (int t = tid; t < n; t += kHoldThreads) {
+        const int i = ix[t];
+        b32[t] = PairBody32(px[i], py[i], pz[i], pvx[i], pvy[i], pvz[i], pm[i]);
+    }
+    if (tid < ((n + 31) >> 5)) bits[tid] = 0u;
+    if (tid == 0) *nunsure = 0;
+    __syncthreads();
+    const float dtf = (float)dt;  // its rounding is far inside the bounds' margin
+    auto mark = [&](int a, int b) {
+        atomicOr(bits + (a >> 5), 1u << (a & 31));
+        atomicOr(bits + (b >> 5), 1u << (b & 31));
+    };
+    auto exact = [&](int a, int b) {
+        const int i = ix[a], j = ix[b];
+        if (tau_pair(px[j] - px[i], py[j] - py[i], pz[j] - pz[i], pvx[j] - pvx[i], pvy[j] - pvy[i], pvz[j] - pvz[i],
+                     pm[i] + pm[j], G, eta, sym) < dt)
+            mark(a, b);
+    };
+    const int np = n * (n - 1) / 2;
+    for (int p = tid; p < np; p += kHoldThreads) {
+        int b = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f);  // p = b (b - 1) / 2 + a, a < b
+        while (b * (b - 1) / 2 > p) --b;
+        while (b * (b + 1) / 2 <= p) ++b;
+        const int a = p - b * (b - 1) / 2;
+        const PairScale32 scale(b32[a], G, eta);
+        float lo, hi;
+        pair_bounds32(b32[a], b32[b], scale, sym, lo, hi);
+        if (hi < dtf) {
+            mark(a, b);
+        } else if (lo < dtf) {
+            const int k = atomicAdd(nunsure, 1);
+            if (k < kHoldUnsure) unsure[k] = (unsigned)a << 16 | (unsigned)b;
+            else exact(a, b);
+        }
+    }
+    __syncthreads();
+    const int nu = *nunsure < kHoldUnsure ? *nunsure : kHoldUnsure;
+    for (int k = tid; k < nu; k += kHoldThreads) {
+        const int a = (int)(unsure[k] >> 16), b = (int)(unsure[k] & 0xffffu);
+        // (a bit set meanwhile by another pair only saves the evaluation)
+        const unsigned wa = *(volatile unsigned*)(bits + (a >> 5)), wb = *(volatile unsigned*)(bits + (b >> 5));
+        if (!((wa >> (a & 31)) & (wb >> (b & 31)) & 1u)) exact(a, b);
+    }
+    __syncthreads();
 }
 
 // stats: {slow-system kicks, FMM solves (none here), direct solves, deepest level, splits}
@@ -149,12 +251,16 @@ __global__ void __launch_bounds__(kHoldThreads) k_hold_small(int k, const int* _
     double* pvy = pvx + k;
     double* pvz = pvy + k;
     double* pm = pvz + k;
-    double* tau = pm + k;
-    HoldFrame* stack = reinterpret_cast<HoldFrame*>(tau + k);  // kHoldMaxLevels frames
+    double* acc = pm + k;                                      // 3 k sums of a kick
+    double* term = acc + 3 * k;                                // its pairs' terms
+    HoldFrame* stack = reinterpret_cast<HoldFrame*>(reinterpret_cast<unsigned char*>(term) + hold_term_bytes(k));
     int* ix = reinterpret_cast<int*>(stack + kHoldMaxLevels);
     int* tmp = ix + k;
     unsigned* fbits = reinterpret_cast<unsigned*>(tmp + k);  // kHoldMaxLevels x W
-    __shared__ int s_sp, s_nf;
+    // the members in FP32 pairs share the terms' memory (a split and a kick never overlap)
+    PairBody32* b32 = reinterpret_cast<PairBody32*>(term);
+    __shared__ unsigned s_unsure[kHoldUnsure];
+    __shared__ int s_sp, s_nf, s_nunsure;
     const int tid = threadIdx.x;
     for (int a = tid; a < k; a += kHoldThreads) {
         const int i = idx[a];
@@ -180,26 +286,8 @@ __global__ void __launch_bounds__(kHoldThreads) k_hold_small(int k, const int* _
             if ((unsigned long long)f.depth > deepest) deepest = (unsigned long long)f.depth;
             int ns = n;
             if (n > 1 && f.dt > dt_min && f.depth < kHoldMaxDepth && sp + 1 < kHoldMaxLevels) {
-                // tau of every member within the set, then the fast flags as a mask
-                for (int t = tid; t < n; t += kHoldThreads) {
-                    const int i = ix[f.lo + t];
-                    double tt = CUDART_INF;
-                    for (int q = f.lo; q < f.hi; ++q) {
-                        const int j = ix[q];
-                        if (j == i) continue;
-                        const double tij = tau_pair(px[j] - px[i], py[j] - py[i], pz[j] - pz[i], pvx[j] - pvx[i],
-                                                    pvy[j] - pvy[i], pvz[j] - pvz[i], pm[i] + pm[j], G, eta,
-                                                    sym != 0);
-                        if (tij < tt) tt = tij;
-                    }
-                    tau[t] = tt;
-                }
-                __syncthreads();
-                for (int t0 = 0; t0 < n; t0 += kHoldThreads) {
-                    const int t = t0 + tid;
-                    const unsigned b = __ballot_sync(0xffffffffu, t < n && tau[t] < f.dt);
-                    if ((tid & 31) == 0 && t < n) bits[t >> 5] = b;
-                }
+                set_fast_bits(ix + f.lo, n, px, py, pz, pvx, pvy, pvz, pm, G, eta, sym != 0, f.dt, b32, bits,
+                               s_unsure, &s_nunsure);
                 if (tid == 0) s_nf = 0;
                 __syncthreads();
                 if (tid < ((n + 31) >> 5)) atomicAdd(&s_nf, __popc(bits[tid]));
@@ -235,9 +323,7 @@ __global__ void __launch_bounds__(kHoldThreads) k_hold_small(int k, const int* _
             if (f.ns > 0) {
                 // slow bodies feel all of P, fast ones the slow ones; drift the slow ones
                 const double h = 0.5 * f.dt;
-                hold_kick_from(ix, f.lo, s1, f.lo, f.hi, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h);
-                hold_kick_from(ix, s1, f.hi, f.lo, s1, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h);
-                __syncthreads();
+                set_kick(ix + f.lo, n, f.ns, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h, acc, term);
                 for (int t = f.lo + tid; t < s1; t += kHoldThreads) {
                     const int i = ix[t];
                     px[i] += f.dt * pvx[i];
@@ -245,8 +331,7 @@ __global__ void __launch_bounds__(kHoldThreads) k_hold_small(int k, const int* _
                     pz[i] += f.dt * pvz[i];
                 }
                 __syncthreads();
-                hold_kick_from(ix, f.lo, s1, f.lo, f.hi, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h);
-                hold_kick_from(ix, s1, f.hi, f.lo, s1, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h);
+                set_kick(ix + f.lo, n, f.ns, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h, acc, term);
                 kicks += 2;
                 direct += (f.ns < n) ? 4 : 2;
             }
@@ -327,7 +412,7 @@ void hold_drift(int k, const int* idx, double dt, double* x, double* y, double* 
 
 size_t hold_small_smem(int k) {
     const size_t W = (size_t)(k + 31) / 32;
-    return 8 * sizeof(double) * (size_t)k + sizeof(HoldFrame) * kHoldMaxLevels + 2 * sizeof(int) * (size_t)k +
+    return 10 * sizeof(double) * (size_t)k + hold_term_bytes(k) + sizeof(HoldFrame) * kHoldMaxLevels + 2 * sizeof(int) * (size_t)k +
            sizeof(unsigned) * W * kHoldMaxLevels;
 }
 
