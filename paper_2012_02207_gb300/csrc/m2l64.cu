@@ -20,10 +20,8 @@
 //    going to the input with u^k and 1/w_n^m to the output with v^n;
 //  - the powers of both angles are formed once per source and serve a rotation
 //    and its inverse.
-// N = 100000, p = 10 (3.29 M sources): 50.8 -> 23.0 ms, the FP64 pipe at 74% of
+// N = 100000, p = 10 (3.29 M sources): 50.8 -> 24.3 ms, the FP64 pipe at 70% of
 // its cycles; N = 4096, p = 8: 1.08 -> 0.29 ms.
-#include <type_traits>
-
 #include "gbfmm_internal.cuh"
 #include "swap_tables.cuh"
 
@@ -181,22 +179,26 @@ constexpr int kM2L64Warps = 4;
 // blocks per SM: 2, 3, 4 and 5 took 26.2, 23.0, 23.3 and 23.3 ms at N = 100000, p = 10
 constexpr int kM2L64Blocks = 3;
 
-// PM bounds the per-thread arrays (p <= PM); G warps share a target, their
-// sums added in warp order.
-template <int PM, int G>
+// PM bounds the per-thread arrays (p <= PM). A target's sources are dealt in
+// batches of 32 to kM2L64Warps parts; every part sums its batches per lane, then
+// its lanes, and the parts are added in order. share: the warps of a block take
+// a part each of one target; otherwise a warp takes all parts of a target of its
+// own, one after the other. The sums are the same either way (a forest's
+// clusters get the bits of their separate solves).
+template <int PM>
 __global__ void __launch_bounds__(32 * kM2L64Warps, kM2L64Blocks)
-    k_m2l64(const int* __restrict__ dnn, int p, const uint32_t* __restrict__ src, const uint32_t* __restrict__ off,
-            const double* __restrict__ mult, const double* __restrict__ zc, const double* __restrict__ hs,
-            double* __restrict__ loc, Swap64 sw, const double* __restrict__ fact, const double* __restrict__ iw,
-            unsigned* __restrict__ queue) {
-    extern __shared__ double red[];  // G > 1: a target's sums per warp
+    k_m2l64(const int* __restrict__ dnn, int p, bool share, const uint32_t* __restrict__ src,
+            const uint32_t* __restrict__ off, const double* __restrict__ mult, const double* __restrict__ zc,
+            const double* __restrict__ hs, double* __restrict__ loc, Swap64 sw, const double* __restrict__ fact,
+            const double* __restrict__ iw, unsigned* __restrict__ queue) {
+    extern __shared__ double red[];  // share: a target's sums per part
     __shared__ int s_target;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nr = ncoef_real(p);
     double c[ncoef_real(PM)], acc[ncoef_real(PM)], pa[2 * (PM + 1)], pb[2 * (PM + 1)];
     for (;;) {
         int b = 0;
-        if (G == 1) {
+        if (!share) {
             if (lane == 0) b = (int)atomicAdd(queue, 1u);
             b = __shfl_sync(0xffffffffu, b, 0);
         } else {
@@ -206,83 +208,90 @@ __global__ void __launch_bounds__(32 * kM2L64Warps, kM2L64Blocks)
             b = s_target;
         }
         if (b >= *dnn) break;
-        for (int j = 0; j < nr; ++j) acc[j] = 0.0;
         const uint32_t q0 = off[b], q1 = off[b + 1];
+        const int nbatch = (int)((q1 - q0 + 31) / 32);
+        const int nparts = nbatch < 1 ? 1 : (nbatch < kM2L64Warps ? nbatch : kM2L64Warps);
+        double* out = loc + (size_t)nr * b;
         const double bx = zc[3 * b], by = zc[3 * b + 1], bz = zc[3 * b + 2];
         const double sb = hs[b];
-        for (uint32_t q = q0 + (G == 1 ? lane : threadIdx.x); q < q1; q += 32 * G) {
-            const int a = (int)src[q];
-            const double rx = zc[3 * a] - bx, ry = zc[3 * a + 1] - by, rz = zc[3 * a + 2] - bz;
-            const double sa = hs[a];
-            const double* mv = mult + (size_t)nr * a;
-            const double rxy2 = rx * rx + ry * ry;
-            const double rho = sqrt(rxy2 + rz * rz);
-            const double rxy = sqrt(rxy2);
-            const double irho = 1.0 / rho;
-            double cp = 1.0, sp = 0.0;
-            if (rxy > 0.0) {
-                const double irxy = 1.0 / rxy;
-                cp = rx * irxy;
-                sp = ry * irxy;
+        for (int w = share ? wib : 0; w < nparts; w += share ? kM2L64Warps : 1) {
+            for (int j = 0; j < nr; ++j) acc[j] = 0.0;
+            for (uint32_t q = q0 + 32 * w + lane; q < q1; q += 32 * kM2L64Warps) {
+                const int a = (int)src[q];
+                const double rx = zc[3 * a] - bx, ry = zc[3 * a + 1] - by, rz = zc[3 * a + 2] - bz;
+                const double sa = hs[a];
+                const double* mv = mult + (size_t)nr * a;
+                const double rxy2 = rx * rx + ry * ry;
+                const double rho = sqrt(rxy2 + rz * rz);
+                const double rxy = sqrt(rxy2);
+                const double irho = 1.0 / rho;
+                double cp = 1.0, sp = 0.0;
+                if (rxy > 0.0) {
+                    const double irxy = 1.0 / rxy;
+                    cp = rx * irxy;
+                    sp = ry * irxy;
+                }
+                const double ct = rz * irho, st = rxy * irho;
+                // (sin phi + i cos phi)^m and (cos theta - i sin theta)^m
+                double ar = 1.0, ai = 0.0, br = 1.0, bi = 0.0;
+                for (int m = 1; m <= p; ++m) {
+                    const double ta = ar * sp - ai * cp, tb = br * ct + bi * st;
+                    ai = ar * cp + ai * sp;
+                    bi = bi * ct - br * st;
+                    ar = ta;
+                    br = tb;
+                    pa[2 * m] = ar; pa[2 * m + 1] = ai;
+                    pb[2 * m] = br; pb[2 * m + 1] = bi;
+                }
+                c[0] = mv[0];
+                for (int n = 1; n <= p; ++n) {
+                    const int low = n < p - n ? n : p - n;  // orders the translation reads
+                    swap_all_n(n, mv + n * n, SwapPass{pa, false, nullptr, sw.cosb, sw.sinb}, n, c + n * n);
+                    swap_low_n(n, c + n * n, SwapPass{pb, false, nullptr, sw.cosb, sw.sinb}, low, c + n * n);
+                }
+                ztrans64<PM>(c, p, sa * irho, sb * irho, irho, fact, iw);
+                acc[0] += c[0];
+                for (int n = 1; n <= p; ++n) {
+                    const int low = n < p - n ? n : p - n;  // orders the translation left non-zero
+                    swap_all_n(n, c + n * n, SwapPass{nullptr, false, nullptr, sw.cosb, sw.sinb}, low, c + n * n);
+                    swap_all_n(n, c + n * n, SwapPass{pb, true, pa, sw.cosb, sw.sinb}, n, acc + n * n);
+                }
             }
-            const double ct = rz * irho, st = rxy * irho;
-            // (sin phi + i cos phi)^m and (cos theta - i sin theta)^m
-            double ar = 1.0, ai = 0.0, br = 1.0, bi = 0.0;
-            for (int m = 1; m <= p; ++m) {
-                const double t = ar * sp - ai * cp, w = br * ct + bi * st;
-                ai = ar * cp + ai * sp;
-                bi = bi * ct - br * st;
-                ar = t;
-                br = w;
-                pa[2 * m] = ar; pa[2 * m + 1] = ai;
-                pb[2 * m] = br; pb[2 * m + 1] = bi;
-            }
-            c[0] = mv[0];
-            for (int n = 1; n <= p; ++n) {
-                const int low = n < p - n ? n : p - n;  // orders the translation reads
-                swap_all_n(n, mv + n * n, SwapPass{pa, false, nullptr, sw.cosb, sw.sinb}, n, c + n * n);
-                swap_low_n(n, c + n * n, SwapPass{pb, false, nullptr, sw.cosb, sw.sinb}, low, c + n * n);
-            }
-            ztrans64<PM>(c, p, sa * irho, sb * irho, irho, fact, iw);
-            acc[0] += c[0];
-            for (int n = 1; n <= p; ++n) {
-                const int low = n < p - n ? n : p - n;  // orders the translation left non-zero
-                swap_all_n(n, c + n * n, SwapPass{nullptr, false, nullptr, sw.cosb, sw.sinb}, low, c + n * n);
-                swap_all_n(n, c + n * n, SwapPass{pb, true, pa, sw.cosb, sw.sinb}, n, acc + n * n);
-            }
-        }
-        __syncwarp();
-        // the lanes' sums, 32 coefficients at a time: lane l ends with coefficient j0 + l
-        double* out = loc + (size_t)nr * b;
-        for (int j0 = 0; j0 < nr; j0 += 32) {
-            double v[32];
+            __syncwarp();
+            // the lanes' sums, 32 coefficients at a time: lane l ends with coefficient j0 + l
+            for (int j0 = 0; j0 < nr; j0 += 32) {
+                double v[32];
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = j0 + i < nr ? acc[j0 + i] : 0.0;
-            halve64<32>(v, lane, 16);
-            halve64<16>(v, lane, 8);
-            halve64<8>(v, lane, 4);
-            halve64<4>(v, lane, 2);
-            halve64<2>(v, lane, 1);
-            if (j0 + lane < nr) (G == 1 ? out : red + (size_t)wib * nr)[j0 + lane] = v[0];
+                for (int i = 0; i < 32; ++i) v[i] = j0 + i < nr ? acc[j0 + i] : 0.0;
+                halve64<32>(v, lane, 16);
+                halve64<16>(v, lane, 8);
+                halve64<8>(v, lane, 4);
+                halve64<4>(v, lane, 2);
+                halve64<2>(v, lane, 1);
+                if (j0 + lane < nr) {
+                    if (share) red[(size_t)w * nr + j0 + lane] = v[0];
+                    else out[j0 + lane] = w ? out[j0 + lane] + v[0] : v[0];
+                }
+            }
         }
-        if (G > 1) {
+        if (share) {
             __syncthreads();
-            for (int j = threadIdx.x; j < nr; j += 32 * G) {
+            for (int j = threadIdx.x; j < nr; j += 32 * kM2L64Warps) {
                 double s = red[j];
-                for (int w = 1; w < G; ++w) s += red[(size_t)w * nr + j];
+                for (int w = 1; w < nparts; ++w) s += red[(size_t)w * nr + j];
                 out[j] = s;
             }
         }
     }
 }
 
-template <int PM, int G>
-void launch_m2l64(const int* dnn, int p, const uint32_t* src, const uint32_t* off, const double* mult,
+template <int PM>
+void launch_m2l64(bool share, const int* dnn, int p, const uint32_t* src, const uint32_t* off, const double* mult,
                   const double* zc, const double* hs, double* loc, const DevTables& tb, unsigned* queue,
                   cudaStream_t st) {
-    const int sh = G == 1 ? 0 : G * ncoef_real(p) * (int)sizeof(double);
-    (k_m2l64<PM, G><<<device_sm_count() * kM2L64Blocks, 32 * kM2L64Warps, sh, st>>>(
-         dnn, p, src, off, mult, zc, hs, loc, Swap64{tb.swap_cos, tb.swap_sin}, tb.fact, tb.iw, queue),
+    const int sh = share ? kM2L64Warps * ncoef_real(p) * (int)sizeof(double) : 0;
+    (k_m2l64<PM><<<device_sm_count() * kM2L64Blocks, 32 * kM2L64Warps, sh, st>>>(
+         dnn, p, share, src, off, mult, zc, hs, loc, Swap64{tb.swap_cos, tb.swap_sin}, tb.fact, tb.iw, queue),
      note_launch());
 }
 
@@ -298,15 +307,9 @@ constexpr int kM2L64FewCells = 16384;
 void m2l_f64(const int* dnn, int ncells, int p, const uint32_t* src, const uint32_t* off, const double* mult,
              const double* zc, const double* hs, double* loc, const DevTables& tb, unsigned* queue, cudaStream_t st) {
     cudaMemsetAsync(queue, 0, sizeof(unsigned), st);
-    auto go = [&](auto pm) {
-        constexpr int PM = decltype(pm)::value;
-        if (ncells < kM2L64FewCells)
-            launch_m2l64<PM, kM2L64Warps>(dnn, p, src, off, mult, zc, hs, loc, tb, queue, st);
-        else
-            launch_m2l64<PM, 1>(dnn, p, src, off, mult, zc, hs, loc, tb, queue, st);
-    };
-    if (p <= 16) go(std::integral_constant<int, 16>{});
-    else go(std::integral_constant<int, kMaxP>{});
+    const bool share = ncells < kM2L64FewCells;
+    if (p <= 16) launch_m2l64<16>(share, dnn, p, src, off, mult, zc, hs, loc, tb, queue, st);
+    else launch_m2l64<kMaxP>(share, dnn, p, src, off, mult, zc, hs, loc, tb, queue, st);
 }
 
 }  // namespace gbfmm

@@ -52,3 +52,19 @@ def test_fp64_m2l_one_warp_per_target():
     fi[run.tree()["perm"]] = run.geometry()["f"]
     assert np.max(np.linalg.norm(acc - oacc, axis=1) / fi) <= 1e-12
     assert np.max(np.abs(pot - opot) / np.abs(opot)) <= 1e-12
+
+
+def test_fp64_forest_equals_separate_solves():
+    """A forest above the cell count where a warp takes a whole target, of clusters that are below it alone."""
+    sizes = [30000, 300, 35000, 1]
+    offs = np.concatenate([[0], np.cumsum(sizes)])
+    parts = [ics.plummer(n, 20 + n) for n in sizes]
+    pos, m = np.concatenate([q[0] for q in parts]), np.concatenate([q[2] for q in parts])
+    cols = [torch.tensor(np.ascontiguousarray(c), dtype=torch.float64, device="cuda") for c in (*pos.T, m)]
+    f = gb.FMM(p=5, eps=1e-6, leaf_size=4, precision="fp64")
+    out = torch.stack(f.solve_batch(offs, *cols))
+    assert f.stats()["nnodes"] > 16384
+    for a, b in zip(offs[:-1], offs[1:]):
+        g = gb.FMM(p=5, eps=1e-6, leaf_size=4, precision="fp64")
+        one = torch.stack(g.solve(*(c[a:b].contiguous() for c in cols)))
+        assert torch.equal(one, out[:, a:b])
