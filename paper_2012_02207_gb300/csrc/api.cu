@@ -164,6 +164,7 @@ struct fmm_ctx {
     cudaStream_t gstream = nullptr;       // stream of the captured solve (capture needs a non-default one)
     int walk_steps[2] = {0, 0};           // steps of the last ordinary solve's walks
     uint32_t items_total[2] = {0, 0};     // and its P2P work items and partial slots
+    int tslice = kMaxLeaf;                // and their targets per item
     cudaEvent_t gev[2] = {nullptr, nullptr};
 };
 
@@ -636,7 +637,10 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
     uint32_t* item_first = as<uint32_t>(ctx->item_first);
     uint32_t* slot_first = as<uint32_t>(ctx->slot_first);
     uint32_t* totals = as<uint32_t>(ctx->work) + 4;
-    leaf_items_plan(t, as<uint32_t>(ctx->doff[3]), item_first, slot_first, totals, st);
+    // (in graph form t.nnodes is the planned capacity)
+    const int tslice = leaf_target_slice(t.nnodes, mixed);
+    ctx->tslice = tslice;
+    leaf_items_plan(t, tslice, as<uint32_t>(ctx->doff[3]), item_first, slot_first, totals, st);
     uint32_t htot[2] = {0, 0};
     if (gp) {
         htot[0] = gp->items_cap;
@@ -670,6 +674,7 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
     la.bulk = (ctx->cfg.flags & FMM_FLAG_P2P_LOADS) == 0;
     la.tx_extra = (ctx->cfg.fault_inject & 2u) ? 16u : 0u;
     la.slots_cap = htot[1];
+    la.tslice = tslice;
     if (mixed) {
         leaf_relative_f32(t, la.xs, la.ys, la.zs, la.ms, la.zc, as<float4>(ctx->prel), st);
         la.prel = as<float4>(ctx->prel);
@@ -771,6 +776,7 @@ int jerk_pass(fmm_ctx* ctx, const double* vx, const double* vy, const double* vz
     la.loc = mixed ? ctx->loc32.ptr : ctx->loc.ptr;
     la.part_hi = as<double2>(ctx->part_hi); la.part_lo = as<double2>(ctx->part_lo);
     la.slots_cap = ctx->items_total[1];
+    la.tslice = ctx->tslice;
     jerk_leaves(la, mixed, mixed ? ctx->jloc32.ptr : ctx->jloc.ptr, as<double>(ctx->jv), as<float4>(ctx->jv32),
                 as<int>(ctx->item_leaf), as<uint32_t>(ctx->item_first), as<uint32_t>(ctx->slot_first),
                 as<uint32_t>(ctx->work) + 4, as<unsigned>(ctx->work), as<int>(ctx->leaf_of), jx, jy, jz, st);

@@ -348,9 +348,14 @@ struct LeafArgs {
     float soft2f;  // the same, rounded to FP32 (mixed P2P)
     unsigned* err;      // kErr* bits (a bounded wait that ran out: kErrTimeout)
     bool bulk;          // FP32 P2P: stage source leaves by bulk copies (unless FMM_FLAG_P2P_LOADS)
+    int tslice;         // targets per work item (leaf_target_slice)
     uint32_t tx_extra;  // test hook: bytes a bulk-copy wait expects beyond those copied (0)
 };
-void leaf_items_plan(const TreeView& t, const uint32_t* p2p_off, uint32_t* item_first, uint32_t* slot_first,
+// targets of a leaf per work item: the items of a leaf are its parts (ranges of
+// source leaves) times its slices of targets. A body's sums do not depend on it.
+int leaf_target_slice(int ncells, bool fp32);
+__host__ __device__ inline int leaf_slices(int n_bodies, int tslice) { return (n_bodies + tslice - 1) / tslice; }
+void leaf_items_plan(const TreeView& t, int tslice, const uint32_t* p2p_off, uint32_t* item_first, uint32_t* slot_first,
                      uint32_t* totals, cudaStream_t st);
 // raise kErrCapacity (and run no item) when the item or slot totals exceed the buffers
 void leaf_items_check(uint32_t* totals, uint32_t items_cap, uint32_t slots_cap, unsigned* err, cudaStream_t st);

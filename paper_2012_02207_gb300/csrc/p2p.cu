@@ -3,14 +3,12 @@
 //
 // P2P runs over work items: a target leaf and at most kLeavesPerItem of the
 // source leaves in its (sorted) P2P list, taken by warps from a counter.
-// The default kernel (k_p2p_tiles) stages the item's source bodies in shared
+// The kernel (k_p2p_tiles) stages the item's source bodies in shared
 // memory, by bulk copies or plain loads, puts the sources across the lanes
 // and keeps a group of target bodies in every lane's registers, so one
 // shared-memory load serves several interactions and every lane is busy
 // whatever the leaf sizes; a fixed transpose reduction then sums the lanes.
-// The alternative kernel (k_p2p_lanes, GBFMM_P2P_TILES=0) gives each target
-// G = 32 / nt lanes that split the sources between them. Each item writes
-// one partial per target body. k_leaf_reduce then evaluates the leaf's local
+// Each item writes one partial per target body. k_leaf_reduce then evaluates the leaf's local
 // expansion at the body (L2P), adds the body's partials in item order, and
 // writes the result to the caller's order through the sort permutation.
 // Every sum runs in a fixed order.
@@ -117,12 +115,30 @@ __device__ __forceinline__ void l2p_hat(int p_rt, const T* __restrict__ F, T x, 
 }
 
 // ---------------------------------------------------------------------------
-// P2P over work items. Item (B, j) covers the sources q in
+// P2P over work items. Item (B, j, s) covers the sources q in
 // [off[B] + j*kLeavesPerItem, ...) of target leaf B (at most kLeavesPerItem
-// source leaves), so no warp carries more than a bounded share of a dense
+// source leaves) and slice s of its targets, so no warp carries more than a bounded share of a dense
 // leaf's work. Warps fetch items dynamically. Each item writes one partial
 // sum per target body; k_leaf_reduce adds the partials of a body in item
 // order (deterministic) together with the L2P far field.
+
+// Item r of target leaf B (nB bodies, sources off0 .. off1 - 1 of the list):
+// kLeavesPerItem source leaves (part) and a.tslice targets (t0 .. t1 - 1) of it.
+struct LeafItem {
+    uint32_t part, q0, q1;
+    int t0, t1;
+};
+__device__ __forceinline__ LeafItem leaf_item(const LeafArgs& a, uint32_t r, uint32_t off0, uint32_t off1, int nB) {
+    LeafItem it;
+    const uint32_t nsl = (uint32_t)leaf_slices(nB, a.tslice);
+    it.part = r / nsl;
+    const int s = (int)(r - it.part * nsl);
+    it.q0 = off0 + it.part * kLeavesPerItem;
+    it.q1 = it.q0 + kLeavesPerItem < off1 ? it.q0 + kLeavesPerItem : off1;
+    it.t0 = s * a.tslice;
+    it.t1 = it.t0 + a.tslice < nB ? it.t0 + a.tslice : nB;
+    return it;
+}
 
 // Knuth's two-sum: (hi, lo) += b with the rounding error kept in lo.
 __device__ __forceinline__ void two_sum(float& hi, float& lo, float b) {
@@ -161,26 +177,13 @@ struct NearAcc {
     }
 };
 
-// 1/sqrt(x) in FP64 without the long FP64 divide and square root: an FP32
-// seed refined by two Newton steps y <- y (3 - x y^2) / 2 (each squares the
-// relative error: about 2^-22 -> 2^-44 -> the FP64 rounding level). Outside
-// the FP32 range of the seed (and for x = 0) it falls back to 1 / sqrt(x).
-__device__ __forceinline__ double rsqrt_nr(double x) {
-    if (!(x > 1e-30 && x < 1e30)) return x > 0.0 ? 1.0 / sqrt(x) : 0.0;
-    double y = (double)rsqrtf((float)x);
-    const double hx = 0.5 * x;
-    y = y * fma(-hx * y, y, 1.5);
-    y = y * fma(-hx * y, y, 1.5);
-    return y;
-}
-
 // ---------------------------------------------------------------------------
 // P2P force over work items, sources across lanes and targets in registers.
 //
 // A warp stages the item's source bodies (moved into the target leaf B's
-// frame) in shared memory, up to TileCfg::kCap at a time. The targets of B
-// are taken in groups of TG (8 in FP32, 4 in FP64; a last group of TG/2 when
-// at most TG/2 remain). For a group, lane l runs over the staged sources
+// frame) in shared memory, up to TileCfg::kCap at a time. The targets of the
+// item are taken in groups of TG = 8 (a last group of 4 when at most 4
+// remain). For a group, lane l runs over the staged sources
 // l, l + 32, l + 64, ... and keeps TG four-component partial sums (ax, ay,
 // az, sum m/r) in registers: one shared-memory load serves TG interactions
 // and every lane is busy whatever the leaf sizes. The 32 lanes' partials of
@@ -216,8 +219,11 @@ struct TileCfg<float> {
 };
 template <>
 struct TileCfg<double> {
-    static constexpr int TG = 4;
-    static constexpr int kCap = 256;          // 8 KB per warp
+    static constexpr int TG = 8;
+    // 8 KB per warp. Groups of 4 targets with two Newton steps for 1/r took 49.6 ms for the 0.83 G pairs
+    // of N = 100000, groups of 8 with inv_powers (19 FP64 instructions a pair, half the reductions)
+    // and slices of 8 targets 32.8 ms
+    static constexpr int kCap = 256;
 };
 constexpr int kTargetChunk = 64;  // targets whose totals a warp keeps in shared memory per pass
 
@@ -487,12 +493,15 @@ __device__ __forceinline__ void p2p_group(const Body4<T>* __restrict__ sm, int c
         for (int t = 0; t < NT; ++t) {
             const T dx = s.x - tx[t], dy = s.y - ty[t], dz = s.z - tz[t];
             const T r2 = dx * dx + dy * dy + dz * dz;
-            T rinv;
-            if constexpr (sizeof(T) == 4) rinv = rsqrtf(SOFT ? r2 + s2 : r2);
-            else rinv = (T)rsqrt_nr((double)(SOFT ? r2 + s2 : r2));
-            if (GUARD && !(r2 > T(0))) rinv = T(0);  // the body itself
-            const T mr = mj * rinv;
-            const T mr3 = mr * rinv * rinv;
+            T mr, mr3;
+            if constexpr (sizeof(T) == 4) {
+                float rinv = rsqrtf(SOFT ? r2 + s2 : r2);
+                if (GUARD && !(r2 > 0.0f)) rinv = 0.0f;  // the body itself
+                mr = mj * rinv;
+                mr3 = mr * rinv * rinv;
+            } else {  // (Newtonian: the body itself, r2 = 0, gives zero)
+                inv_powers(SOFT ? r2 + s2 : r2, SOFT && GUARD && !(r2 > 0.0) ? 0.0 : mj, mr, mr3);
+            }
             run[4 * t] += mr3 * dx;
             run[4 * t + 1] += mr3 * dy;
             run[4 * t + 2] += mr3 * dz;
@@ -523,7 +532,7 @@ __device__ __forceinline__ void p2p_groups(const Body4<T>* __restrict__ sm, int 
 }
 
 template <typename T, bool SOFT, bool BULK>
-__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 4 : GBFMM_P2P_MINB) k_p2p_tiles(LeafArgs a, const int* __restrict__ item_leaf,
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 3 : GBFMM_P2P_MINB) k_p2p_tiles(LeafArgs a, const int* __restrict__ item_leaf,
                                                     const uint32_t* __restrict__ item_first,
                                                     const uint32_t* __restrict__ slot_first,
                                                     const uint32_t* __restrict__ nitems_p, unsigned* __restrict__ work) {
@@ -550,17 +559,15 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 4 : GBFMM_P2P_MINB) k_p2
         it = __shfl_sync(0xffffffffu, it, 0);
         if ((int)it >= nitems) break;
         const int B = item_leaf[it];
-        const int j = (int)(it - item_first[B]);
-        const uint32_t q0 = a.p2p_off[B] + (uint32_t)j * kLeavesPerItem;
-        const uint32_t qe = a.p2p_off[B + 1];
-        const uint32_t q1 = q0 + kLeavesPerItem < qe ? q0 + kLeavesPerItem : qe;
         const int b0 = a.t.begin[B], nB = a.t.end[B] - b0;
-        const uint32_t slot0 = slot_first[B] + (uint32_t)j * (uint32_t)nB;
+        const LeafItem item = leaf_item(a, it - item_first[B], a.p2p_off[B], a.p2p_off[B + 1], nB);
+        const uint32_t q0 = item.q0, q1 = item.q1;
+        const uint32_t slot0 = slot_first[B] + item.part * (uint32_t)nB;
         const float4 bh = a.zhi[B], bl = a.zlo[B];
         unsigned long long nsrc = 0;  // source bodies of this item (for the interaction count)
         bool self_item = false;
-        for (int tc = 0; tc < nB; tc += kTargetChunk) {
-            const int nt = nB - tc < kTargetChunk ? nB - tc : kTargetChunk;
+        for (int tc = item.t0; tc < item.t1; tc += kTargetChunk) {
+            const int nt = item.t1 - tc < kTargetChunk ? item.t1 - tc : kTargetChunk;
             __syncwarp();
             for (int e = lane; e < 4 * nt; e += 32) tot[e] = 0.0;
             for (int t = lane; t < nt; t += 32) {
@@ -585,7 +592,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 4 : GBFMM_P2P_MINB) k_p2
                 }
                 pad_stage<T>(sm, cnt, lane);
                 __syncwarp();
-                if (tc == 0) { nsrc += (unsigned long long)cnt; self_item |= selfin; }
+                if (tc == 0) { nsrc += (unsigned long long)cnt; self_item |= selfin; }  // once per source range
                 if (selfin) p2p_groups<T, true, SOFT>(sm, cnt, tg, nt, s2, tot, lane);
                 else p2p_groups<T, false, SOFT>(sm, cnt, tg, nt, s2, tot, lane);
             }
@@ -600,193 +607,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 4 : GBFMM_P2P_MINB) k_p2
             }
         }
         // directed body-body interactions of the item (a body never acts on itself)
-        if (lane == 0)
-            atomicAdd(a.interactions, (unsigned long long)nB * nsrc - (self_item ? (unsigned long long)nB : 0ull));
-    }
-}
-
-// ---------------------------------------------------------------------------
-// P2P force over work items, targets across lanes (the alternative layout,
-// selected by GBFMM_P2P_TILES = 0): a warp stages the item's sources in
-// shared memory 256 at a time and gives each of the nt targets of a chunk of
-// 32 G = 32 / nt lanes that split the sources between them; FP32 runs of
-// kRun terms are folded into two-sum pairs; one partial per target body.
-// SOFT: Plummer softening (Appendix B), 1/r -> 1/sqrt(r^2 + s2); the body
-// itself (r2 = 0; coincident bodies are rejected) still contributes nothing.
-template <typename T, bool GUARD, int GC, bool SOFT>
-__device__ __forceinline__ void p2p_pack_g(const Body4<T>* __restrict__ sm, int cnt, int sub, int Gr, T tx, T ty,
-                                           T tz, T s2, NearAcc<T>& acc) {
-    const int G = GC > 0 ? GC : Gr;  // lanes per target (compile-time when GC > 0)
-    auto term = [&](int k, T& px, T& py, T& pz, T& pp) {
-        const Body4<T> sv = sm[k];
-        const T dx = sv.x - tx, dy = sv.y - ty, dz = sv.z - tz;
-        const T r2 = dx * dx + dy * dy + dz * dz;
-        T rinv;
-        if (sizeof(T) == 4) {
-            rinv = (T)rsqrtf((float)(SOFT ? r2 + s2 : r2));
-            if (GUARD && !(r2 > T(0))) rinv = T(0);  // the body itself
-        } else {
-            rinv = (T)rsqrt_nr((double)(SOFT ? r2 + s2 : r2));
-            if (SOFT && GUARD && !(r2 > T(0))) rinv = T(0);
-        }
-        const T mr = sv.w * rinv;
-        const T mr3 = mr * rinv * rinv;
-        px += mr3 * dx;
-        py += mr3 * dy;
-        pz += mr3 * dz;
-        pp += mr;
-    };
-    int k0 = sub;
-    if (GC > 0) {
-        // full runs of kRun terms, unrolled (constant shared-memory offsets, no loop control)
-        for (; k0 + kRun * GC <= cnt; k0 += kRun * GC) {
-            T px = T(0), py = T(0), pz = T(0), pp = T(0);
-#pragma unroll
-            for (int u = 0; u < kRun; ++u) term(k0 + u * GC, px, py, pz, pp);
-            acc.add(px, py, pz, pp);
-        }
-    }
-    for (; k0 < cnt; k0 += kRun * G) {
-        const int k1 = k0 + kRun * G < cnt ? k0 + kRun * G : cnt;
-        T px = T(0), py = T(0), pz = T(0), pp = T(0);
-#pragma unroll 4
-        for (int k = k0; k < k1; k += G) term(k, px, py, pz, pp);
-        acc.add(px, py, pz, pp);
-    }
-}
-
-template <typename T, bool GUARD, bool SOFT>
-__device__ __forceinline__ void p2p_pack(const Body4<T>* __restrict__ sm, int cnt, int sub, int G, T tx, T ty,
-                                         T tz, T s2, NearAcc<T>& acc) {
-    if (G == 1) p2p_pack_g<T, GUARD, 1, SOFT>(sm, cnt, sub, G, tx, ty, tz, s2, acc);
-    else if (G == 2) p2p_pack_g<T, GUARD, 2, SOFT>(sm, cnt, sub, G, tx, ty, tz, s2, acc);
-    else if (G == 4) p2p_pack_g<T, GUARD, 4, SOFT>(sm, cnt, sub, G, tx, ty, tz, s2, acc);
-    else p2p_pack_g<T, GUARD, 0, SOFT>(sm, cnt, sub, G, tx, ty, tz, s2, acc);
-}
-
-template <typename T, bool SOFT>
-__global__ void __launch_bounds__(128) k_p2p_lanes(LeafArgs a, const int* __restrict__ item_leaf,
-                                                    const uint32_t* __restrict__ item_first,
-                                                    const uint32_t* __restrict__ slot_first,
-                                                    const uint32_t* __restrict__ nitems_p, unsigned* __restrict__ work) {
-    __shared__ Body4<T> stage[4][kStageCap];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    Body4<T>* sm = stage[wib];
-    const int nitems = (int)*nitems_p;
-    for (;;) {
-        unsigned it = 0;
-        if (lane == 0) it = atomicAdd(work, 1u);
-        it = __shfl_sync(0xffffffffu, it, 0);
-        if ((int)it >= nitems) break;
-        const int B = item_leaf[it];
-        const int j = (int)(it - item_first[B]);
-        const uint32_t q0 = a.p2p_off[B] + (uint32_t)j * kLeavesPerItem;
-        const uint32_t qe = a.p2p_off[B + 1];
-        const uint32_t q1 = q0 + kLeavesPerItem < qe ? q0 + kLeavesPerItem : qe;
-        const int b0 = a.t.begin[B], nB = a.t.end[B] - b0;
-        const uint32_t slot0 = slot_first[B] + (uint32_t)j * (uint32_t)nB;
-        const float4 bh = a.zhi[B], bl = a.zlo[B];
-        unsigned long long nsrc = 0;  // source bodies of this item (for the interaction count)
-        bool self_item = false;
-        for (int tc = 0; tc < nB; tc += 32) {
-            const int nt = nB - tc < 32 ? nB - tc : 32;
-            const int G = 32 / nt;            // lanes per target
-            const int t = lane / G, sub = lane - t * G;
-            const bool act = t < nt;
-            T tx = T(0), ty = T(0), tz = T(0);
-            if (act) {
-                if (sizeof(T) == 4) {
-                    const float4 v = a.prel[b0 + tc + t];
-                    tx = (T)v.x; ty = (T)v.y; tz = (T)v.z;
-                } else {
-                    tx = (T)a.xs[b0 + tc + t]; ty = (T)a.ys[b0 + tc + t]; tz = (T)a.zs[b0 + tc + t];
-                }
-            }
-            NearAcc<T> acc;
-            uint32_t q = q0;
-            int soff = 0;
-            while (q < q1) {
-                // pack source leaves (or a piece of an oversized one) into the stage
-                __syncwarp();
-                int cnt = 0;
-                bool selfin = false;
-                while (q < q1) {
-                    const int A = (int)a.p2p_src[q];
-                    const int a0 = a.t.begin[A], nA = a.t.end[A] - a0;
-                    const int rem = nA - soff;
-                    int take = rem;
-                    if (cnt + take > kStageCap) {
-                        if (cnt > 0) break;
-                        take = kStageCap;
-                    }
-                    float ox = 0.f, oy = 0.f, oz = 0.f;
-                    if (sizeof(T) == 4) {
-                        const float4 ah = a.zhi[A], al = a.zlo[A];
-                        ox = (ah.x - bh.x) + (al.x - bl.x);
-                        oy = (ah.y - bh.y) + (al.y - bl.y);
-                        oz = (ah.z - bh.z) + (al.z - bl.z);
-                    }
-                    for (int l = lane; l < take; l += 32) {
-                        const int jj = a0 + soff + l;
-                        Body4<T> v;
-                        if (sizeof(T) == 4) {
-                            const float4 u = a.prel[jj];
-                            v = {(T)(u.x + ox), (T)(u.y + oy), (T)(u.z + oz), (T)u.w};
-                        } else {
-                            v = {(T)a.xs[jj], (T)a.ys[jj], (T)a.zs[jj], (T)a.ms[jj]};
-                        }
-                        sm[cnt + l] = v;
-                    }
-                    selfin |= (A == B);
-                    if (tc == 0) { nsrc += (unsigned long long)take; self_item |= (A == B); }
-                    cnt += take;
-                    if (take < rem) { soff += take; break; }
-                    soff = 0;
-                    ++q;
-                }
-                __syncwarp();
-                if (!act) continue;
-                const T s2 = SOFT ? (sizeof(T) == 4 ? (T)a.soft2f : (T)a.soft2) : T(0);
-                if (selfin) p2p_pack<T, true, SOFT>(sm, cnt, sub, G, tx, ty, tz, s2, acc);
-                else p2p_pack<T, false, SOFT>(sm, cnt, sub, G, tx, ty, tz, s2, acc);
-            }
-            float &hx = acc.hx, &hy = acc.hy, &hz = acc.hz, &hp = acc.hp;
-            float &lx = acc.lx, &ly = acc.ly, &lz = acc.lz, &lp = acc.lp;
-            double &dx64 = acc.dx, &dy64 = acc.dy, &dz64 = acc.dz, &dp64 = acc.dp;
-            // combine the G sub-lanes of each target in sub-lane order
-            const int leader = t * G;
-            for (int s = 1; s < G; ++s) {
-                const int src = leader + s < 32 ? leader + s : 31;
-                if (sizeof(T) == 4) {
-                    const float vx = __shfl_sync(0xffffffffu, hx, src), vy = __shfl_sync(0xffffffffu, hy, src),
-                                vz = __shfl_sync(0xffffffffu, hz, src), vp = __shfl_sync(0xffffffffu, hp, src);
-                    const float wx = __shfl_sync(0xffffffffu, lx, src), wy = __shfl_sync(0xffffffffu, ly, src),
-                                wz = __shfl_sync(0xffffffffu, lz, src), wp = __shfl_sync(0xffffffffu, lp, src);
-                    if (sub == 0 && act) {
-                        two_sum(hx, lx, vx); lx += wx;
-                        two_sum(hy, ly, vy); ly += wy;
-                        two_sum(hz, lz, vz); lz += wz;
-                        two_sum(hp, lp, vp); lp += wp;
-                    }
-                } else {
-                    const double vx = __shfl_sync(0xffffffffu, dx64, src), vy = __shfl_sync(0xffffffffu, dy64, src),
-                                 vz = __shfl_sync(0xffffffffu, dz64, src), vp = __shfl_sync(0xffffffffu, dp64, src);
-                    if (sub == 0 && act) { dx64 += vx; dy64 += vy; dz64 += vz; dp64 += vp; }
-                }
-            }
-            if (act && sub == 0) {
-                const uint32_t slot = slot0 + (uint32_t)(tc + t);
-                if (sizeof(T) == 4) {
-                    a.part_hi[slot] = make_double2((double)hx + (double)lx, (double)hy + (double)ly);
-                    a.part_lo[slot] = make_double2((double)hz + (double)lz, (double)hp + (double)lp);
-                } else {
-                    a.part_hi[slot] = make_double2(dx64, dy64);
-                    a.part_lo[slot] = make_double2(dz64, dp64);
-                }
-            }
-        }
-        // directed body-body interactions of the item (a body never acts on itself)
-        if (lane == 0)
+        if (lane == 0 && item.t0 == 0)
             atomicAdd(a.interactions, (unsigned long long)nB * nsrc - (self_item ? (unsigned long long)nB : 0ull));
     }
 }
@@ -821,7 +642,8 @@ __global__ void __launch_bounds__(128) k_leaf_reduce(LeafArgs a, const int* __re
                         (a.zs[i] - a.zc[3 * B + 2]) * inv_s, inv_s, tb, phi, fx, fy, fz);
         sx = fx; sy = fy; sz = fz; sp = phi;
     }
-    const uint32_t i0 = item_first[B], i1 = item_first[B + 1];
+    // partials: one per range of source leaves, whatever the slices
+    const uint32_t i0 = 0, i1 = (item_first[B + 1] - item_first[B]) / (uint32_t)leaf_slices(nB, a.tslice);
     const uint32_t s0 = slot_first[B] + (uint32_t)(i - b0);
     // the body's item partials in item order; four items' loads are issued
     // before they are added, so their latencies overlap
@@ -851,18 +673,20 @@ __global__ void __launch_bounds__(128) k_leaf_reduce(LeafArgs a, const int* __re
     if (a.pot) a.pot[o] = a.G * sp;
 }
 
-// work items per leaf: ceil(#source leaves / kLeavesPerItem); slots = items * n_B
-__global__ void k_items_count(TreeView t, const uint32_t* __restrict__ off, uint32_t* __restrict__ nitems,
-                              uint32_t* __restrict__ nslots) {
+// work items per leaf: ceil(#source leaves / kLeavesPerItem) parts times its
+// slices of targets; slots = parts * n_B
+__global__ void k_items_count(TreeView t, int tslice, const uint32_t* __restrict__ off,
+                              uint32_t* __restrict__ nitems, uint32_t* __restrict__ nslots) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= t.nnodes) return;  // the grid's nodes; those past *dnn get no items
-    uint32_t ni = 0;
+    uint32_t parts = 0, nB = 0;
     if (b < *t.dnn && t.nchild[b] == 0) {
         const uint32_t deg = off[b + 1] - off[b];
-        ni = (deg + kLeavesPerItem - 1) / kLeavesPerItem;
+        parts = (deg + kLeavesPerItem - 1) / kLeavesPerItem;
+        nB = (uint32_t)(t.end[b] - t.begin[b]);
     }
-    nitems[b] = ni;
-    nslots[b] = ni ? ni * (uint32_t)(t.end[b] - t.begin[b]) : 0u;
+    nitems[b] = parts * (uint32_t)leaf_slices((int)nB, tslice);
+    nslots[b] = parts * nB;
 }
 
 __global__ void k_items_fill(const int* __restrict__ dnn, const uint32_t* __restrict__ item_first,
@@ -1090,7 +914,7 @@ __device__ __forceinline__ void jerk_pack(const Body4<T>* __restrict__ sm, const
             const T r2 = dx * dx + dy * dy + dz * dz;
             T rinv;
             if constexpr (sizeof(T) == 4) rinv = rsqrtf(SOFT ? r2 + s2 : r2);
-            else rinv = rsqrt_nr(SOFT ? r2 + s2 : r2);
+            else rinv = inv_sqrt(SOFT ? r2 + s2 : r2);
             if (!(r2 > T(0))) rinv = T(0);  // the body itself
             const T ri2 = rinv * rinv;
             const T mr3 = sv.w * rinv * ri2;
@@ -1125,15 +949,13 @@ __global__ void __launch_bounds__(128) k_jerk_items(LeafArgs a, const double* __
         it = __shfl_sync(0xffffffffu, it, 0);
         if ((int)it >= nitems) break;
         const int B = item_leaf[it];
-        const int j = (int)(it - item_first[B]);
-        const uint32_t q0 = a.p2p_off[B] + (uint32_t)j * kLeavesPerItem;
-        const uint32_t qe = a.p2p_off[B + 1];
-        const uint32_t q1 = q0 + kLeavesPerItem < qe ? q0 + kLeavesPerItem : qe;
         const int b0 = a.t.begin[B], nB = a.t.end[B] - b0;
-        const uint32_t slot0 = slot_first[B] + (uint32_t)j * (uint32_t)nB;
+        const LeafItem item = leaf_item(a, it - item_first[B], a.p2p_off[B], a.p2p_off[B + 1], nB);
+        const uint32_t q0 = item.q0, q1 = item.q1;
+        const uint32_t slot0 = slot_first[B] + item.part * (uint32_t)nB;
         const float4 bh = a.zhi[B], bl = a.zlo[B];
-        for (int tc = 0; tc < nB; tc += 32) {
-            const int nt = nB - tc < 32 ? nB - tc : 32;
+        for (int tc = item.t0; tc < item.t1; tc += 32) {
+            const int nt = item.t1 - tc < 32 ? item.t1 - tc : 32;
             const int G = 32 / nt;
             const int t = lane / G, sub = lane - t * G;
             const bool act = t < nt;
@@ -1264,7 +1086,7 @@ __global__ void __launch_bounds__(128) k_jerk_reduce(LeafArgs a, const void* __r
     double fx = -(double)gx + (double)h[0] * vix + (double)h[3] * viy + (double)h[4] * viz;
     double fy = -(double)gy + (double)h[3] * vix + (double)h[1] * viy + (double)h[5] * viz;
     double fz = -(double)gz + (double)h[4] * vix + (double)h[5] * viy + (double)h[2] * viz;
-    const uint32_t i0 = item_first[B], i1 = item_first[B + 1];
+    const uint32_t i0 = 0, i1 = (item_first[B + 1] - item_first[B]) / (uint32_t)leaf_slices(nB, a.tslice);
     const uint32_t s0 = slot_first[B] + (uint32_t)(i - b0);
     for (uint32_t it = i0; it < i1; ++it) {
         const uint32_t slot = s0 + (it - i0) * (uint32_t)nB;
@@ -1298,9 +1120,23 @@ void upload_leaf_tables(const HostTables& h) {
     cudaMemcpyToSymbol(c_sub32l, s, sizeof(s));
 }
 
-void leaf_items_plan(const TreeView& t, const uint32_t* p2p_off, uint32_t* item_first, uint32_t* slot_first,
+// Targets per work item. A slice stages the sources again, so whole leaves are
+// cheapest where there are items enough; on a small tree an item per part of a
+// leaf leaves most warps idle. FP32: up to 2048 cells slices of 8 (N = 4096:
+// leaf phase 0.232 ms whole, 0.154 by 16, 0.144 by 8; at 4282 cells 0.80 whole
+// and by 32, 0.84 by 16). FP64, where staging hides behind the arithmetic: 4 up to
+// 2048 cells (N = 4096: 3.73 ms whole, 1.21 by 8, 0.93 by 4), 8 above (N =
+// 100000: 35.5 ms whole, 33.2 by 8, 33.8 by 4).
+constexpr int kFewCells = 2048;
+int leaf_target_slice(int ncells, bool fp32) {
+    if (fp32) return ncells < kFewCells ? 8 : kMaxLeaf;
+    return ncells < kFewCells ? 4 : 8;
+}
+
+void leaf_items_plan(const TreeView& t, int tslice, const uint32_t* p2p_off, uint32_t* item_first, uint32_t* slot_first,
                      uint32_t* totals, cudaStream_t st) {
-    (k_items_count<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t, p2p_off, item_first, slot_first), note_launch());
+    (k_items_count<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t, tslice, p2p_off, item_first, slot_first),
+     note_launch());
     scan_exclusive_u32(item_first, t.nnodes, item_first + t.nnodes, st);
     scan_exclusive_u32(slot_first, t.nnodes, slot_first + t.nnodes, st);
     cudaMemcpyAsync(totals, item_first + t.nnodes, 4, cudaMemcpyDeviceToDevice, st);
@@ -1316,10 +1152,6 @@ void leaf_items_fill(const TreeView& t, const uint32_t* item_first, int* item_le
     (k_items_fill<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t.dnn, item_first, item_leaf, items_cap), note_launch());
     (k_leaf_of_bodies<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t, leaf_of), note_launch());
 }
-
-#ifndef GBFMM_P2P_TILES
-#define GBFMM_P2P_TILES 1
-#endif
 
 namespace {
 // persistent grid: as many blocks as fit on every SM (warps take items from a counter)
@@ -1342,12 +1174,6 @@ void launch_tiles(const LeafArgs& a, const int* item_leaf, const uint32_t* item_
 template <typename T, bool SOFT>
 void launch_p2p_tiles(const LeafArgs& a, const int* item_leaf, const uint32_t* item_first, const uint32_t* slot_first,
                       const uint32_t* nitems, unsigned* work, cudaStream_t st) {
-    if (!GBFMM_P2P_TILES) {
-        (k_p2p_lanes<T, SOFT><<<device_sm_count() * 16, 128, 0, st>>>(a, item_leaf, item_first, slot_first, nitems,
-                                                                     work),
-         note_launch());
-        return;
-    }
     if (sizeof(T) == 4 && a.bulk) launch_tiles<T, SOFT, true>(a, item_leaf, item_first, slot_first, nitems, work, st);
     else launch_tiles<T, SOFT, false>(a, item_leaf, item_first, slot_first, nitems, work, st);
 }
