@@ -349,6 +349,7 @@ struct LeafArgs {
     unsigned* err;      // kErr* bits (a bounded wait that ran out: kErrTimeout)
     bool bulk;          // FP32 P2P: stage source leaves by bulk copies (unless FMM_FLAG_P2P_LOADS)
     int tslice;         // targets per work item (leaf_target_slice)
+    float one = 1.0f;   // a 1 the compiler does not see (f32x2.cuh)
     uint32_t tx_extra;  // test hook: bytes a bulk-copy wait expects beyond those copied (0)
 };
 // targets of a leaf per work item: the items of a leaf are its parts (ranges of

@@ -17,6 +17,7 @@
 // FP32; a source leaf A is moved into the target leaf B's frame by the
 // FP32-rounded offset z_A - z_B (computed from double-float centres). Terms
 // are FP32 (rsqrtf); each staged pack's sum is accumulated in FP64.
+#include "f32x2.cuh"
 #include "fp64_math.cuh"
 #include "gbfmm_internal.cuh"
 
@@ -472,40 +473,81 @@ __device__ __forceinline__ T transpose_reduce(T* v, int lane) {
 // at most kCap / 32 terms.
 template <typename T, int NT, bool GUARD, bool SOFT>
 __device__ __forceinline__ void p2p_group(const Body4<T>* __restrict__ sm, int cnt, const Body4<T>* __restrict__ tg,
-                                          int t0, int nt, T s2, double* tot, int lane) {
+                                          int t0, int nt, T s2, double* tot, int lane, float one) {
     const int g = (lane >> 2) & (NT - 1);
-    T tx[NT], ty[NT], tz[NT];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-        const int i = t0 + (t ^ g);
-        const Body4<T> v = tg[i < nt ? i : nt - 1];
-        tx[t] = v.x; ty[t] = v.y; tz[t] = v.z;
-    }
     T run[NT * 4];
-#pragma unroll
-    for (int e = 0; e < NT * 4; ++e) run[e] = T(0);
     // the stage is padded to a multiple of 32 with massless far bodies (pad_stage)
     const int per_lane = (cnt + 31) >> 5;
-    for (int u = 0; u < per_lane; ++u) {
-        const Body4<T> s = sm[lane + 32 * u];
-        const T mj = s.w;
+    if constexpr (sizeof(T) == 4) {
+        // two targets to a packed operation: 13 operations of the FMA pipe a pair as before, at half the issue
+        // slots, which were the bound (74% of cycles). 2^20 bodies, 5.8 G pairs: 4.24 -> 3.59 ms, FMA pipe 54 ->
+        // 62%; without the moves of the sources into the target frame it would take 3.3 ms
+        f32x2 nx[NT / 2], ny[NT / 2], nz[NT / 2], acc[NT * 2];  // negated targets; per pair x, y, z, sum m/r
+#pragma unroll
+        for (int t = 0; t < NT; t += 2) {
+            const int i = t0 + (t ^ g), j = t0 + ((t + 1) ^ g);
+            const Body4<T> u = tg[i < nt ? i : nt - 1], v = tg[j < nt ? j : nt - 1];
+            nx[t / 2] = f2_pack(-u.x, -v.x);
+            ny[t / 2] = f2_pack(-u.y, -v.y);
+            nz[t / 2] = f2_pack(-u.z, -v.z);
+        }
+#pragma unroll
+        for (int e = 0; e < NT * 2; ++e) acc[e] = 0ull;
+        const f32x2 one2 = f2_pack(one, one), s22 = f2_pack(s2, s2);
+        Body4<T> nxt = sm[lane];  // one source ahead (the last step's reads the targets behind the stage, unused)
+        for (int u = 0; u < per_lane; ++u) {
+            const Body4<T> s = nxt;
+            nxt = sm[lane + 32 * (u + 1)];
+            const f32x2 sx = f2_pack(s.x, s.x), sy = f2_pack(s.y, s.y), sz = f2_pack(s.z, s.z), sw = f2_pack(s.w, s.w);
+#pragma unroll
+            for (int t = 0; t < NT / 2; ++t) {
+                const f32x2 dx = f2_add<true>(sx, nx[t]), dy = f2_add<true>(sy, ny[t]), dz = f2_add<true>(sz, nz[t]);
+                const f32x2 r2 = f2_fma<true>(dz, dz, f2_fma<true>(dx, dx, f2_mul<true>(dy, dy)));
+                float ra, rb, qa, qb;
+                f2_unpack(r2, ra, rb);
+                f2_unpack(SOFT ? f2_add<true>(r2, s22) : r2, qa, qb);
+                qa = rsqrtf(qa);
+                qb = rsqrtf(qb);
+                if (GUARD) {  // the body itself
+                    if (!(ra > 0.0f)) qa = 0.0f;
+                    if (!(rb > 0.0f)) qb = 0.0f;
+                }
+                const f32x2 rinv = f2_pack(qa, qb);
+                const f32x2 mr = f2_mul<true>(sw, rinv);
+                const f32x2 mr3 = f2_mul<true>(f2_mul<true>(mr, rinv), rinv);
+                acc[4 * t] = f2_fma<true>(mr3, dx, acc[4 * t]);
+                acc[4 * t + 1] = f2_fma<true>(mr3, dy, acc[4 * t + 1]);
+                acc[4 * t + 2] = f2_fma<true>(mr3, dz, acc[4 * t + 2]);
+                acc[4 * t + 3] = f2_fma<true>(mr, one2, acc[4 * t + 3]);  // a sum: the product rounded first
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < NT / 2; ++t)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) f2_unpack(acc[4 * t + c], run[8 * t + c], run[8 * t + 4 + c]);
+    } else {
+        T tx[NT], ty[NT], tz[NT];
 #pragma unroll
         for (int t = 0; t < NT; ++t) {
-            const T dx = s.x - tx[t], dy = s.y - ty[t], dz = s.z - tz[t];
-            const T r2 = dx * dx + dy * dy + dz * dz;
-            T mr, mr3;
-            if constexpr (sizeof(T) == 4) {
-                float rinv = rsqrtf(SOFT ? r2 + s2 : r2);
-                if (GUARD && !(r2 > 0.0f)) rinv = 0.0f;  // the body itself
-                mr = mj * rinv;
-                mr3 = mr * rinv * rinv;
-            } else {  // (Newtonian: the body itself, r2 = 0, gives zero)
-                inv_powers(SOFT ? r2 + s2 : r2, SOFT && GUARD && !(r2 > 0.0) ? 0.0 : mj, mr, mr3);
+            const int i = t0 + (t ^ g);
+            const Body4<T> v = tg[i < nt ? i : nt - 1];
+            tx[t] = v.x; ty[t] = v.y; tz[t] = v.z;
+        }
+#pragma unroll
+        for (int e = 0; e < NT * 4; ++e) run[e] = T(0);
+        for (int u = 0; u < per_lane; ++u) {
+            const Body4<T> s = sm[lane + 32 * u];
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                const T dx = s.x - tx[t], dy = s.y - ty[t], dz = s.z - tz[t];
+                const T r2 = dx * dx + dy * dy + dz * dz;
+                T mr, mr3;  // (Newtonian: the body itself, r2 = 0, gives zero)
+                inv_powers(SOFT ? r2 + s2 : r2, SOFT && GUARD && !(r2 > 0.0) ? 0.0 : s.w, mr, mr3);
+                run[4 * t] += mr3 * dx;
+                run[4 * t + 1] += mr3 * dy;
+                run[4 * t + 2] += mr3 * dz;
+                run[4 * t + 3] += mr;
             }
-            run[4 * t] += mr3 * dx;
-            run[4 * t + 1] += mr3 * dy;
-            run[4 * t + 2] += mr3 * dz;
-            run[4 * t + 3] += mr;
         }
     }
     const T v = transpose_reduce<NT * 4>(run, lane);
@@ -524,11 +566,11 @@ __device__ __forceinline__ void pad_stage(Body4<T>* sm, int cnt, int lane) {
 
 template <typename T, bool GUARD, bool SOFT>
 __device__ __forceinline__ void p2p_groups(const Body4<T>* __restrict__ sm, int cnt, const Body4<T>* __restrict__ tg,
-                                           int nt, T s2, double* tot, int lane) {
+                                           int nt, T s2, double* tot, int lane, float one) {
     constexpr int TG = TileCfg<T>::TG;
     int t0 = 0;
-    for (; nt - t0 > TG / 2; t0 += TG) p2p_group<T, TG, GUARD, SOFT>(sm, cnt, tg, t0, nt, s2, tot, lane);
-    if (t0 < nt) p2p_group<T, TG / 2, GUARD, SOFT>(sm, cnt, tg, t0, nt, s2, tot, lane);
+    for (; nt - t0 > TG / 2; t0 += TG) p2p_group<T, TG, GUARD, SOFT>(sm, cnt, tg, t0, nt, s2, tot, lane, one);
+    if (t0 < nt) p2p_group<T, TG / 2, GUARD, SOFT>(sm, cnt, tg, t0, nt, s2, tot, lane, one);
 }
 
 template <typename T, bool SOFT, bool BULK>
@@ -593,8 +635,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 3 : GBFMM_P2P_MINB) k_p2
                 pad_stage<T>(sm, cnt, lane);
                 __syncwarp();
                 if (tc == 0) { nsrc += (unsigned long long)cnt; self_item |= selfin; }  // once per source range
-                if (selfin) p2p_groups<T, true, SOFT>(sm, cnt, tg, nt, s2, tot, lane);
-                else p2p_groups<T, false, SOFT>(sm, cnt, tg, nt, s2, tot, lane);
+                if (selfin) p2p_groups<T, true, SOFT>(sm, cnt, tg, nt, s2, tot, lane, a.one);
+                else p2p_groups<T, false, SOFT>(sm, cnt, tg, nt, s2, tot, lane, a.one);
             }
             __syncwarp();
             // totals to the item's partial slots: (ax, ay) in part_hi, (az, sum m/r) in part_lo
