@@ -474,7 +474,7 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
         (rc = ensure(ctx, ctx->ms, 8 * N)) || (rc = ensure(ctx, ctx->xf, 16 * N)) ||
         (rc = ensure(ctx, ctx->prel, 16 * N)) || (rc = ensure(ctx, ctx->lcp, N)) ||
         (rc = ensure(ctx, ctx->win, N)) || (rc = ensure(ctx, ctx->hi, N)) ||
-        (rc = ensure(ctx, ctx->chunk, 4 * ((size_t)(kMaxLevel + 1) * nchunks + 2))) ||
+        (rc = ensure(ctx, ctx->chunk, 4 * ((size_t)(kMaxLevel + 1) * nchunks + 2 + scan_scratch_words((int64_t)(kMaxLevel + 1) * nchunks)))) ||
         (rc = ensure(ctx, ctx->f, 4 * N)) || (rc = ensure(ctx, ctx->bbox, 8 * 6 * (size_t)bbox_partials(nclusters))) ||
         (rc = ensure(ctx, ctx->coff, 4 * ((size_t)nclusters + 1))) || (rc = ensure(ctx, ctx->box, 64 * (size_t)nclusters)))
         return rc;
@@ -656,7 +656,7 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
         (rc = ensure(ctx, ctx->part_hi, 16 * (size_t)(htot[1] + 1))) ||
         (rc = ensure(ctx, ctx->part_lo, 16 * (size_t)(htot[1] + 1))))
         return rc;
-    leaf_items_fill(t, item_first, as<int>(ctx->item_leaf), htot[0], as<int>(ctx->leaf_of), st);
+    leaf_items_fill(t, item_first, as<int>(ctx->item_leaf), htot[0], st);
     LeafArgs la{};
     la.t = t; la.p = p; la.G = ctx->cfg.G;
     la.soft2 = ctx->cfg.soft * ctx->cfg.soft;
@@ -675,10 +675,9 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
     la.tx_extra = (ctx->cfg.fault_inject & 2u) ? 16u : 0u;
     la.slots_cap = htot[1];
     la.tslice = tslice;
-    if (mixed) {
-        leaf_relative_f32(t, la.xs, la.ys, la.zs, la.ms, la.zc, as<float4>(ctx->prel), st);
-        la.prel = as<float4>(ctx->prel);
-    }
+    if (mixed) la.prel = as<float4>(ctx->prel);
+    leaf_bodies(t, la.xs, la.ys, la.zs, la.ms, la.zc, as<int>(ctx->leaf_of), mixed ? as<float4>(ctx->prel) : nullptr,
+                st);
     la.loc = far32 ? ctx->loc32.ptr : ctx->loc.ptr;
     leaf_eval(la, mixed, far32, as<int>(ctx->item_leaf), item_first, slot_first, totals,
               as<unsigned>(ctx->work), as<int>(ctx->leaf_of), st);

@@ -296,24 +296,34 @@ void launch_p2m_dw(const TreeView& t, int p, const double* xs, const double* ys,
 
 // P_n = s^n sqrt(sum_{m=-n}^{n} |Mhat_n^m|^2)  (Sec. 2.3)
 // (also the FP32 copies used by the walk's screen: Phat_n = P_n / s^n and r)
+// LANES threads per node, thread j the degrees n = j, j + LANES, ..: each
+// degree's sum and power of s keep their order. Four for small trees, where a
+// node's chain of operations bounds the launch (N = 4096: 28 us with one,
+// 11 us with four), one above kPnormCells, where the FP64 instructions
+// do (the degrees of unequal length leave lanes idle).
+constexpr int kPnormCells = 16384;
+template <int LANES>
 __global__ void k_pnorm(const int* __restrict__ dnn, int p, const double* __restrict__ mult,
                         const double* __restrict__ rr, const double* __restrict__ hs,
                         double* __restrict__ Pk, float* __restrict__ Phat,
                         float* __restrict__ r32) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = g / LANES, j = g % LANES;
     if (k >= *dnn) return;
     const double* M = mult + (size_t)ncoef_real(p) * k;
     const double s = hs[k];
     double sp = 1.0;
-    for (int n = 0; n <= p; ++n) {
+    for (int i = 0; i < j; ++i) sp *= s;
+    for (int n = j; n <= p; n += LANES) {
         double acc = M[hre(n, 0)] * M[hre(n, 0)];
         for (int m = 1; m <= n; ++m) acc += 2.0 * (M[hre(n, m)] * M[hre(n, m)] + M[him(n, m)] * M[him(n, m)]);
         const double nrm = sqrt(acc);
         Pk[(size_t)(p + 1) * k + n] = sp * nrm;
         Phat[(size_t)(p + 1) * k + n] = (float)nrm;
-        sp *= s;
+#pragma unroll
+        for (int i = 0; i < LANES; ++i) sp *= s;
     }
-    r32[k] = (float)rr[k];
+    if (j == 0) r32[k] = (float)rr[k];
 }
 
 __global__ void k_to_f32(const double* __restrict__ a, float* __restrict__ b, const int* __restrict__ dnn, int nr) {
@@ -496,7 +506,11 @@ void upward_pass(const TreeView& t, const int* h_level_start, int p, const doubl
     (void)nr;
     (void)h_level_start;
     for (int L = t.nlevels - 2; L >= 0; --L) m2m_level(t, L, p, geo, mult, contrib, tbl, dword, st);
-    (k_pnorm<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t.dnn, p, mult, r, hs, Pk, Phat, r32), note_launch());
+    if (t.nnodes < kPnormCells)
+        (k_pnorm<4><<<blocks_for(4 * (int64_t)t.nnodes, 128), 128, 0, st>>>(t.dnn, p, mult, r, hs, Pk, Phat, r32),
+         note_launch());
+    else
+        (k_pnorm<1><<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t.dnn, p, mult, r, hs, Pk, Phat, r32), note_launch());
 }
 
 void p2m_weights(const TreeView& t, int p, const double* xs, const double* ys, const double* zs, const double* w,

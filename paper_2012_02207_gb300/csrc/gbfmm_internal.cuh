@@ -113,6 +113,21 @@ struct TreeView {
     const int* nchild;
 };
 
+// Calls f(L0, L1, cells) for the internal levels from the deepest up: one
+// level at a time (L0 = L1) for those of many cells, then all the levels above the
+// last of these in one call, for a launch of a single block that walks them
+// (every cell a few threads): the launches of the small upper levels cost their
+// latency, not work. 512 cells of 8 threads are four rounds of a block.
+constexpr int kBlockLevelCells = 512;
+template <typename F>
+void for_levels_up(const TreeView& t, F f) {
+    int top = -1;  // levels 0 .. top have few cells each
+    while (top + 1 <= t.nlevels - 2 && t.lvl_cnt[top + 1] <= kBlockLevelCells) ++top;
+    for (int L = t.nlevels - 2; L > top; --L)
+        if (t.lvl_cnt[L] > 0) f(L, L, t.lvl_cnt[L]);
+    if (top >= 0) f(0, top, t.lvl_cnt[top]);
+}
+
 // Every kernel launch of the library calls note_launch(); fmm_get_stats
 // reports the count of the last solve.
 void note_launch();
@@ -361,14 +376,16 @@ void leaf_items_plan(const TreeView& t, int tslice, const uint32_t* p2p_off, uin
 // raise kErrCapacity (and run no item) when the item or slot totals exceed the buffers
 void leaf_items_check(uint32_t* totals, uint32_t items_cap, uint32_t slots_cap, unsigned* err, cudaStream_t st);
 void leaf_items_fill(const TreeView& t, const uint32_t* item_first, int* item_leaf, uint32_t items_cap,
-                     int* leaf_of, cudaStream_t st);
+                     cudaStream_t st);
 // nitems: device count of work items; p2p32: FP32 P2P on leaf-relative
 // bodies (else FP64); l2p32: FP32 L2P on FP32 hat locals (else FP64)
 void leaf_eval(const LeafArgs& a, bool p2p32, bool l2p32, const int* item_leaf, const uint32_t* item_first,
                const uint32_t* slot_first, const uint32_t* nitems, unsigned* work, const int* leaf_of,
                cudaStream_t st);
-void leaf_relative_f32(const TreeView& t, const double* xs, const double* ys, const double* zs,
-                       const double* ms, const double* zc, float4* prel, cudaStream_t st);
+// the leaf of every body and, where prel is not NULL, its leaf-relative FP32
+// position and mass
+void leaf_bodies(const TreeView& t, const double* xs, const double* ys, const double* zs, const double* ms,
+                 const double* zc, int* leaf_of, float4* prel, cudaStream_t st);
 // Jerk inputs in sorted order: velocities vs (3n, FP64) and v32 (FP32), and
 // the dipole weights w = m v (3n).
 void jerk_inputs(int n, const uint32_t* perm, const double* ms, const double* vx, const double* vy,

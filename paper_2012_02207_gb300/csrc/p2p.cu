@@ -748,20 +748,20 @@ __global__ void k_check_items(uint32_t* totals, uint32_t items_cap, uint32_t slo
     }
 }
 
-__global__ void k_leaf_of_bodies(TreeView t, int* __restrict__ leaf_of) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= *t.dnn || t.nchild[k] != 0) return;
-    for (int i = t.begin[k]; i < t.end[k]; ++i) leaf_of[i] = k;
-}
-
-__global__ void k_leaf_relative(TreeView t, const double* __restrict__ xs, const double* __restrict__ ys,
-                                const double* __restrict__ zs, const double* __restrict__ ms,
-                                const double* __restrict__ zc, float4* __restrict__ prel) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+// the leaf of every body, and (prel non-NULL) its leaf-relative FP32 position
+// and mass. Eight lanes per leaf, on neighbouring bodies (one thread per leaf
+// and a launch for each took 47 us at N = 4096 and 95 us at 2^20, this 9 and 46)
+__global__ void k_leaf_bodies(TreeView t, const double* __restrict__ xs, const double* __restrict__ ys,
+                              const double* __restrict__ zs, const double* __restrict__ ms,
+                              const double* __restrict__ zc, int* __restrict__ leaf_of, float4* __restrict__ prel) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = g >> 3;
     if (k >= *t.dnn || t.nchild[k] != 0) return;
     const double cx = zc[3 * k], cy = zc[3 * k + 1], cz = zc[3 * k + 2];
-    for (int i = t.begin[k]; i < t.end[k]; ++i)
-        prel[i] = make_float4((float)(xs[i] - cx), (float)(ys[i] - cy), (float)(zs[i] - cz), (float)ms[i]);
+    for (int i = t.begin[k] + (g & 7); i < t.end[k]; i += 8) {
+        leaf_of[i] = k;
+        if (prel) prel[i] = make_float4((float)(xs[i] - cx), (float)(ys[i] - cy), (float)(zs[i] - cz), (float)ms[i]);
+    }
 }
 
 // Direct FP64 sum, one thread per target, source tiles staged in shared
@@ -1190,9 +1190,8 @@ void leaf_items_check(uint32_t* totals, uint32_t items_cap, uint32_t slots_cap, 
 }
 
 void leaf_items_fill(const TreeView& t, const uint32_t* item_first, int* item_leaf, uint32_t items_cap,
-                     int* leaf_of, cudaStream_t st) {
+                     cudaStream_t st) {
     (k_items_fill<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t.dnn, item_first, item_leaf, items_cap), note_launch());
-    (k_leaf_of_bodies<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t, leaf_of), note_launch());
 }
 
 namespace {
@@ -1270,9 +1269,10 @@ void jerk_leaves(const LeafArgs& a, bool fp32, const void* locj, const double* v
     }
 }
 
-void leaf_relative_f32(const TreeView& t, const double* xs, const double* ys, const double* zs,
-                       const double* ms, const double* zc, float4* prel, cudaStream_t st) {
-    (k_leaf_relative<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t, xs, ys, zs, ms, zc, prel), note_launch());
+void leaf_bodies(const TreeView& t, const double* xs, const double* ys, const double* zs, const double* ms,
+                 const double* zc, int* leaf_of, float4* prel, cudaStream_t st) {
+    (k_leaf_bodies<<<blocks_for(8 * (int64_t)t.nnodes, 128), 128, 0, st>>>(t, xs, ys, zs, ms, zc, leaf_of, prel),
+     note_launch());
 }
 
 // Segments the sources are split into: as many as give every SM eight blocks

@@ -25,7 +25,7 @@
 namespace gbfmm {
 
 namespace {
-constexpr int kChunk = 256;  // bodies per thread in the node enumeration
+constexpr int kChunk = 256;  // bodies (threads) per block in the node enumeration
 constexpr int kBboxBlocks = 304;  // bounding-cube partials (2 blocks per SM)
 
 // block (c, s) of a grid of nclusters * slices blocks reduces slice s of cluster c
@@ -269,47 +269,76 @@ __global__ void k_window_max(const int8_t* __restrict__ win, int64_t n, int leaf
     hi[i] = (uint8_t)(d + 1 < kMaxLevel ? d + 1 : kMaxLevel);
 }
 
-__device__ __forceinline__ int start_lo(const int8_t* lcp, int64_t i) { return (int)lcp[i]; }
-
-// per (level, chunk) node-start counts, level-major
-__global__ void k_level_count(const int8_t* __restrict__ lcp, const uint8_t* __restrict__ hi,
-                              int64_t n, int nchunks, uint32_t* __restrict__ cnt) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= nchunks) return;
-    uint32_t local[kMaxLevel + 1];
-#pragma unroll
-    for (int L = 0; L <= kMaxLevel; ++L) local[L] = 0;
-    const int64_t b = (int64_t)c * kChunk;
-    const int64_t e = b + kChunk < n ? b + kChunk : n;
-    for (int64_t i = b; i < e; ++i) {
-        const int lo = start_lo(lcp, i), h = hi[i];
-#pragma unroll
-        for (int L = 0; L <= kMaxLevel; ++L) local[L] += (L > lo && L <= h) ? 1u : 0u;
-    }
-#pragma unroll
-    for (int L = 0; L <= kMaxLevel; ++L) cnt[(int64_t)L * nchunks + c] = local[L];
+// The levels at which a node starts at body i: lcp_i < L <= hi_i (none past
+// the last body).
+__device__ __forceinline__ void start_levels(const int8_t* lcp, const uint8_t* hi, int64_t i, int64_t n, int& lo,
+                                             int& h) {
+    lo = i < n ? (int)lcp[i] : kMaxLevel;
+    h = i < n ? (int)hi[i] : 0;
 }
 
-__global__ void k_level_emit(const int8_t* __restrict__ lcp, const uint8_t* __restrict__ hi,
-                             int64_t n, int nchunks, const uint32_t* __restrict__ off,
-                             int* __restrict__ level, int* __restrict__ begin, int64_t node_cap,
-                             unsigned* err) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= nchunks) return;
-    uint32_t next[kMaxLevel + 1];
+// Node starts per (level, chunk), level-major, and below their emission: a
+// thread per body, a warp vote per level (a thread per chunk of 256 bodies, its
+// bodies and levels in loops, took 33 + 170 us at N = 4096 and 43 + 192 us at
+// 2^20; now 3 + 4 and 10 + 14 us).
+__global__ void __launch_bounds__(kChunk) k_level_count(const int8_t* __restrict__ lcp,
+                                                        const uint8_t* __restrict__ hi, int64_t n, int nchunks,
+                                                        uint32_t* __restrict__ cnt) {
+    __shared__ uint32_t wcnt[kChunk / 32][kMaxLevel + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int lo, h;
+    start_levels(lcp, hi, (int64_t)blockIdx.x * kChunk + threadIdx.x, n, lo, h);
+    uint32_t mine = 0;  // lane L keeps level L's count
 #pragma unroll
-    for (int L = 0; L <= kMaxLevel; ++L) next[L] = off[(int64_t)L * nchunks + c];
-    const int64_t b = (int64_t)c * kChunk;
-    const int64_t e = b + kChunk < n ? b + kChunk : n;
-    for (int64_t i = b; i < e; ++i) {
-        const int lo = start_lo(lcp, i), h = hi[i];
+    for (int L = 0; L <= kMaxLevel; ++L) {
+        const unsigned b = __ballot_sync(0xffffffffu, L > lo && L <= h);
+        if (lane == L) mine = (uint32_t)__popc(b);
+    }
+    if (lane <= kMaxLevel) wcnt[warp][lane] = mine;
+    __syncthreads();
+    if (threadIdx.x <= kMaxLevel) {
+        uint32_t s = 0;
 #pragma unroll
-        for (int L = 0; L <= kMaxLevel; ++L) {
-            if (L > lo && L <= h) {
-                const uint32_t k = next[L]++;
-                if ((int64_t)k < node_cap) { level[k] = L; begin[k] = (int)i; }
-                else atomicOr(err, kErrCapacity);
-            }
+        for (int w = 0; w < kChunk / 32; ++w) s += wcnt[w][threadIdx.x];
+        cnt[(int64_t)threadIdx.x * nchunks + blockIdx.x] = s;
+    }
+}
+
+__global__ void __launch_bounds__(kChunk) k_level_emit(const int8_t* __restrict__ lcp,
+                                                       const uint8_t* __restrict__ hi, int64_t n, int nchunks,
+                                                       const uint32_t* __restrict__ off, int* __restrict__ level,
+                                                       int* __restrict__ begin, int64_t node_cap, unsigned* err) {
+    __shared__ uint32_t wnext[kChunk / 32][kMaxLevel + 1];  // counts, then each warp's first node per level
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * kChunk + threadIdx.x;
+    int lo, h;
+    start_levels(lcp, hi, i, n, lo, h);
+    uint32_t mine = 0;
+#pragma unroll
+    for (int L = 0; L <= kMaxLevel; ++L) {
+        const unsigned b = __ballot_sync(0xffffffffu, L > lo && L <= h);
+        if (lane == L) mine = (uint32_t)__popc(b);
+    }
+    if (lane <= kMaxLevel) wnext[warp][lane] = mine;
+    __syncthreads();
+    if (threadIdx.x <= kMaxLevel) {
+        uint32_t run = off[(int64_t)threadIdx.x * nchunks + blockIdx.x];
+#pragma unroll
+        for (int w = 0; w < kChunk / 32; ++w) {
+            const uint32_t c = wnext[w][threadIdx.x];
+            wnext[w][threadIdx.x] = run;
+            run += c;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int L = 0; L <= kMaxLevel; ++L) {
+        const bool start = L > lo && L <= h;
+        const unsigned b = __ballot_sync(0xffffffffu, start);
+        if (start) {
+            const uint32_t k = wnext[warp][L] + (uint32_t)__popc(b & ((1u << lane) - 1u));
+            if ((int64_t)k < node_cap) { level[k] = L; begin[k] = (int)i; }
+            else atomicOr(err, kErrCapacity);
         }
     }
 }
@@ -379,65 +408,105 @@ __global__ void k_finalize(const uint64_t* __restrict__ keys, int64_t n, int lea
     }
 }
 
-// Leaf geometry: sums over the leaf's bodies in sorted order.
+// Leaf geometry: sums over the leaf's bodies in sorted order. Four lanes per
+// leaf, one for each of the sums of m, m x, m y, m z (each a serial chain of FP64
+// additions, so four chains in flight a leaf); the largest distance with the
+// bodies dealt to the four lanes (a maximum does not depend on the order). One
+// thread per leaf took 54 us at N = 4096 and 134 us at 2^20, this 21 and 93 us.
 __global__ void k_geometry_leaves(TreeView t, const double* __restrict__ xs,
                                   const double* __restrict__ ys, const double* __restrict__ zs,
                                   const double* __restrict__ ms, double* __restrict__ M,
                                   double* __restrict__ S, double* __restrict__ zc,
                                   double* __restrict__ r) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= *t.dnn || t.nchild[k] != 0) return;
-    double Mk = 0.0, Sx = 0.0, Sy = 0.0, Sz = 0.0;
-    const int b = t.begin[k], e = t.end[k];
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = g >> 2, c = g & 3, lane0 = threadIdx.x & 28;
+    const bool leaf = k < *t.dnn && t.nchild[k] == 0;
+    const int b = leaf ? t.begin[k] : 0, e = leaf ? t.end[k] : 0;
+    const double* q = c == 1 ? xs : (c == 2 ? ys : zs);
+    double sum = 0.0;
+#pragma unroll 4
     for (int i = b; i < e; ++i) {
         const double mi = ms[i];
-        Mk = Mk + mi;
-        Sx = Sx + mi * xs[i];
-        Sy = Sy + mi * ys[i];
-        Sz = Sz + mi * zs[i];
+        sum = sum + (c ? mi * q[i] : mi);
     }
-    const double zx = Sx / Mk, zy = Sy / Mk, zz = Sz / Mk;
+    const double Mk = __shfl_sync(0xffffffffu, sum, lane0);
+    const double zq = sum / Mk;
+    const double zx = __shfl_sync(0xffffffffu, zq, lane0 + 1), zy = __shfl_sync(0xffffffffu, zq, lane0 + 2),
+                 zz = __shfl_sync(0xffffffffu, zq, lane0 + 3);
     // the largest distance: a correctly rounded square root is monotonic, so
     // the root of the largest squared distance equals the largest root (one
     // FP64 square root per leaf instead of one per body)
     double rr2 = 0.0;
-    for (int i = b; i < e; ++i) {
+#pragma unroll 2
+    for (int i = b + c; i < e; i += 4) {
         const double dx = xs[i] - zx, dy = ys[i] - zy, dz = zs[i] - zz;
         const double d2 = dx * dx + dy * dy + dz * dz;
         if (d2 > rr2) rr2 = d2;
     }
-    const double rr = sqrt(rr2);
-    M[k] = Mk;
-    S[3 * k] = Sx; S[3 * k + 1] = Sy; S[3 * k + 2] = Sz;
-    zc[3 * k] = zx; zc[3 * k + 1] = zy; zc[3 * k + 2] = zz;
-    r[k] = rr;
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        const double v = __shfl_xor_sync(0xffffffffu, rr2, o);
+        if (v > rr2) rr2 = v;
+    }
+    if (!leaf) return;
+    if (c == 0) {
+        M[k] = sum;
+        r[k] = sqrt(rr2);
+    } else {
+        S[3 * k + c - 1] = sum;
+        zc[3 * k + c - 1] = zq;
+    }
 }
 
-// Internal geometry of one level: sums over children in order.
-__global__ void k_geometry_internal(TreeView t, int L, double* __restrict__ M,
-                                    double* __restrict__ S, double* __restrict__ zc,
-                                    double* __restrict__ r) {
-    const int k = t.dls[L] + blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= t.dls[L + 1] || t.nchild[k] == 0) return;
-    const int c0 = t.first_child[k], c1 = c0 + t.nchild[k];
-    double Mk = 0.0, Sx = 0.0, Sy = 0.0, Sz = 0.0;
-    for (int c = c0; c < c1; ++c) {
-        Mk = Mk + M[c];
-        Sx = Sx + S[3 * c];
-        Sy = Sy + S[3 * c + 1];
-        Sz = Sz + S[3 * c + 2];
+// Internal geometry of levels L1, L1 - 1, .. L0: sums over children in order.
+// Eight lanes per node: lanes 0..3 each sum one of M and S over the children
+// (in order), lane j the distance of child j. A launch of one block takes
+// several levels (those of few nodes, one after the other with a block barrier
+// between), a larger grid takes one level. One thread per node and a launch per
+// level took 96 us at N = 4096 and 164 us at 2^20, this 35 and 135 us.
+__global__ void __launch_bounds__(1024) k_geometry_internal(TreeView t, int L0, int L1, double* __restrict__ M,
+                                                            double* __restrict__ S, double* __restrict__ zc,
+                                                            double* __restrict__ r) {
+    const int j = threadIdx.x & 7, lane0 = threadIdx.x & 24;
+    for (int L = L1; L >= L0; --L) {
+        const int k0 = t.dls[L], k1 = t.dls[L + 1];
+        // (whole warps go round together: the trip count depends on the warp's first node)
+        for (int kw = k0 + (int)((blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) >> 3); kw < k1;
+             kw += (int)(gridDim.x * blockDim.x) >> 3) {
+            const int k = kw + (lane0 >> 3);
+            const bool act = k < k1 && t.nchild[k] != 0;
+            const int c0 = act ? t.first_child[k] : 0, nc = act ? t.nchild[k] : 0;
+            double sum = 0.0;
+            if (j < 4)
+                for (int c = c0; c < c0 + nc; ++c) sum = sum + (j ? S[3 * c + j - 1] : M[c]);
+            const double Mk = __shfl_sync(0xffffffffu, sum, lane0);
+            const double zq = sum / Mk;
+            const double zx = __shfl_sync(0xffffffffu, zq, lane0 + 1), zy = __shfl_sync(0xffffffffu, zq, lane0 + 2),
+                         zz = __shfl_sync(0xffffffffu, zq, lane0 + 3);
+            double rr = 0.0;
+            if (j < nc) {
+                const int c = c0 + j;
+                const double dx = zc[3 * c] - zx, dy = zc[3 * c + 1] - zy, dz = zc[3 * c + 2] - zz;
+                const double d = sqrt(dx * dx + dy * dy + dz * dz) + r[c];
+                if (d > rr) rr = d;
+            }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) {
+                const double v = __shfl_xor_sync(0xffffffffu, rr, o);
+                if (v > rr) rr = v;
+            }
+            if (act) {
+                if (j == 0) {
+                    M[k] = sum;
+                    r[k] = rr;
+                } else if (j < 4) {
+                    S[3 * k + j - 1] = sum;
+                    zc[3 * k + j - 1] = zq;
+                }
+            }
+        }
+        __syncthreads();  // the level below is complete (one block) before its parents read it
     }
-    const double zx = Sx / Mk, zy = Sy / Mk, zz = Sz / Mk;
-    double rr = 0.0;
-    for (int c = c0; c < c1; ++c) {
-        const double dx = zc[3 * c] - zx, dy = zc[3 * c + 1] - zy, dz = zc[3 * c + 2] - zz;
-        const double d = sqrt(dx * dx + dy * dy + dz * dz) + r[c];
-        if (d > rr) rr = d;
-    }
-    M[k] = Mk;
-    S[3 * k] = Sx; S[3 * k + 1] = Sy; S[3 * k + 2] = Sz;
-    zc[3 * k] = zx; zc[3 * k + 1] = zy; zc[3 * k + 2] = zz;
-    r[k] = rr;
 }
 
 inline int blocks_for(int64_t n, int threads) { return (int)((n + threads - 1) / threads); }
@@ -482,17 +551,16 @@ void tree_build_count(TreeBuffers& b, int* sorted_in_1, cudaStream_t st) {
         (k_window_min<<<blocks_for(n - b.leaf_size, 256), 256, 0, st>>>(b.lcp, n, b.leaf_size, b.win), note_launch());
     (k_window_max<<<blocks_for(n, 256), 256, 0, st>>>(b.win, n, b.leaf_size, b.hi), note_launch());
     const int nchunks = tree_nchunks(n);
-    (k_level_count<<<blocks_for(nchunks, 128), 128, 0, st>>>(b.lcp, b.hi, n, nchunks, b.chunk_cnt), note_launch());
+    (k_level_count<<<nchunks, kChunk, 0, st>>>(b.lcp, b.hi, n, nchunks, b.chunk_cnt), note_launch());
     const int64_t cells = (int64_t)(kMaxLevel + 1) * nchunks;
-    scan_exclusive_u32(b.chunk_cnt, cells, b.chunk_cnt + cells, st);
+    scan_exclusive_u32_large(b.chunk_cnt, cells, b.chunk_cnt + cells, b.chunk_cnt + cells + 1, st);
 }
 
 void tree_build_emit(TreeBuffers& b, cudaStream_t st) {
     const int64_t n = b.n;
     const int nchunks = tree_nchunks(n);
     const int64_t cells = (int64_t)(kMaxLevel + 1) * nchunks;
-    (k_level_emit<<<blocks_for(nchunks, 128), 128, 0, st>>>(b.lcp, b.hi, n, nchunks, b.chunk_cnt,
-                                                           b.level, b.begin, b.node_cap, &b.ds->err), note_launch());
+    (k_level_emit<<<nchunks, kChunk, 0, st>>>(b.lcp, b.hi, n, nchunks, b.chunk_cnt, b.level, b.begin, b.node_cap, &b.ds->err), note_launch());
     (k_level_starts<<<1, 32, 0, st>>>(b.chunk_cnt, nchunks, b.chunk_cnt + cells, (int)b.node_cap, b.ds), note_launch());
 }
 
@@ -510,10 +578,15 @@ void cell_geometry(const TreeView& t, const double* xs, const double* ys, const 
                    const double* ms, const int* h_level_start, double* M, double* S, double* zc,
                    double* r, cudaStream_t st) {
     (void)h_level_start;
-    (k_geometry_leaves<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t, xs, ys, zs, ms, M, S, zc, r), note_launch());
-    for (int L = t.nlevels - 2; L >= 0; --L)
-        if (t.lvl_cnt[L] > 0)
-            (k_geometry_internal<<<blocks_for(t.lvl_cnt[L], 128), 128, 0, st>>>(t, L, M, S, zc, r), note_launch());
+    (k_geometry_leaves<<<blocks_for(4 * (int64_t)t.nnodes, 128), 128, 0, st>>>(t, xs, ys, zs, ms, M, S, zc, r),
+     note_launch());
+    for_levels_up(t, [&](int L0, int L1, int cnt) {
+        if (L0 < L1)
+            (k_geometry_internal<<<1, 1024, 0, st>>>(t, L0, L1, M, S, zc, r), note_launch());
+        else
+            (k_geometry_internal<<<blocks_for(8 * (int64_t)cnt, 128), 128, 0, st>>>(t, L0, L1, M, S, zc, r),
+             note_launch());
+    });
 }
 
 void coincident_exact(const TreeBuffers& b, uint64_t* hk0, uint32_t* hv0, uint64_t* hk1, uint32_t* hv1,
