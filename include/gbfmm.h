@@ -49,7 +49,8 @@ typedef enum {
     FMM_ERR_COINCIDENT = -5, /* two bodies share exactly the same position */
     FMM_ERR_CAPACITY = -6,   /* an internal list outgrew its capacity after one regrow */
     FMM_ERR_TIMEOUT = -7     /* a bounded device-side wait ran out (the P2P's bulk-copy
-                                staging); the context stays usable */
+                                staging, the walk's appends, a sort); the context stays
+                                usable */
 } fmm_status;
 
 typedef enum {
@@ -267,14 +268,15 @@ int fmm_export_swap(int64_t* ncos, int64_t* nsin, double* cos_blocks, double* si
  * keys, perm[n] the caller index of each sorted body (ties keep input order),
  * box[4] (may be NULL) the cube centre and half-size. These are exactly the
  * keys and permutation fmm_solve builds its octree from.
- * Scratch: a static device array of about 4.3 MB in the library, held by every
+ * Scratch: a static device array of about 4.4 MB in the library, held by every
  * GPU that loads it until the process exits. The first call on a device looks
  * up the array's address (cudaGetSymbolAddress), so make that first call
  * before any stream capture. All calls share the array: calls that overlap on
  * the GPU (other streams, other host threads) race. The call synchronises its
  * stream before returning.
  * Errors: FMM_ERR_ARG for n outside [0, 262144] or NULL pointers,
- * FMM_ERR_NONFINITE for a NaN or infinite position, FMM_ERR_CUDA; the message
+ * FMM_ERR_NONFINITE for a NaN or infinite position, FMM_ERR_TIMEOUT for a
+ * bounded wait of the sort that ran out, FMM_ERR_CUDA; the message
  * is fmm_last_error(NULL). */
 int fmm_morton_sort_noalloc(int64_t n, const double* x, const double* y, const double* z,
                             uint64_t* keys, int64_t* perm, double* box, void* cuda_stream);

@@ -9,6 +9,7 @@
 // The host reads back three small things (node count, level starts, list
 // sizes); everything else stays on the device.
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
@@ -331,17 +332,18 @@ int build_directed(fmm_ctx* ctx, int which, cudaStream_t st) {
         uint32_t* kb = ka + (2 * np + 1);
         pairs_to_directed32(as<int2>(ctx->lists[which]), ctx->ds->list_cnt + which, np, ctx->nb, ka,
                             as<unsigned long long>(ctx->dcount) + 2 + which, nkeys, st);
-        const int in1 = radix_sort32(ka, kb, 2 * np, 2 * ctx->nb, as<uint32_t>(ctx->hist), st, nkeys, lo_bit);
-        directed_offsets_src32(in1 ? kb : ka, 2 * np, nkeys, ctx->nb, &ctx->ds->nnodes,
+        const int in1 = radix_sort32(ka, kb, 2 * np, 2 * ctx->nb, as<uint32_t>(ctx->hist), &ctx->ds->sort_err, st, nkeys,
+                                       lo_bit);
+        directed_offsets_src32(in1 ? kb : ka, 2 * np, nkeys, ctx->nb, &ctx->ds->nnodes, &ctx->ds->sort_err,
                                as<uint32_t>(ctx->dsrc[which]), as<uint32_t>(ctx->doff[which]), st);
         return FMM_OK;
     }
     pairs_to_directed(as<int2>(ctx->lists[which]), ctx->ds->list_cnt + which, np, ctx->nb,
                       as<uint64_t>(ctx->dkeys[which]), as<unsigned long long>(ctx->dcount) + 2 + which, nkeys, st);
     const int in1 = radix_sort(as<uint64_t>(ctx->dkeys[which]), nullptr, as<uint64_t>(ctx->dalt[which]), nullptr,
-                               2 * np, 2 * ctx->nb, as<uint32_t>(ctx->hist), st, nkeys, lo_bit);
+                               2 * np, 2 * ctx->nb, as<uint32_t>(ctx->hist), &ctx->ds->sort_err, st, nkeys, lo_bit);
     directed_offsets(as<uint64_t>(in1 ? ctx->dalt[which] : ctx->dkeys[which]), 2 * np, nkeys, ctx->nb,
-                     &ctx->ds->nnodes, as<uint32_t>(ctx->dsrc[which]), as<uint32_t>(ctx->doff[which]), st);
+                     &ctx->ds->nnodes, &ctx->ds->sort_err, as<uint32_t>(ctx->dsrc[which]), as<uint32_t>(ctx->doff[which]), st);
     return FMM_OK;
 }
 
@@ -484,7 +486,8 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
          (rc = ensure(ctx, ctx->cid, 4 * N))))
         return rc;
     CK(rec(0));
-    CK(cudaMemsetAsync(&ctx->ds->err, 0, sizeof(unsigned), st));
+    static_assert(offsetof(DevScalars, sort_err) == offsetof(DevScalars, err) + sizeof(unsigned), "both words at once");
+    CK(cudaMemsetAsync(&ctx->ds->err, 0, 2 * sizeof(unsigned), st));
     CK(cudaMemcpyAsync(ctx->coff.ptr, gp ? gp->h_coff : ctx->h_coff.data(), 4 * ((size_t)nclusters + 1),
                        cudaMemcpyHostToDevice, st));
     TreeBuffers tb{};
@@ -505,14 +508,16 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
     tree_build_count(tb, &in1, st);
     ctx->sorted_in_1 = in1;
     uint32_t total = 0;
-    unsigned err = 0;
+    unsigned errs[2] = {0, 0};  // err, sort_err
+    unsigned& err = errs[0];
     if (gp) {
         total = (uint32_t)gp->node_cap;
     } else {
         CK(cudaMemcpyAsync(&total, as<uint32_t>(ctx->chunk) + (size_t)(kMaxLevel + 1) * nchunks, 4,
                            cudaMemcpyDeviceToHost, st));
-        CK(cudaMemcpyAsync(&err, &ctx->ds->err, 4, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(errs, &ctx->ds->err, 8, cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
+        if (errs[1]) return fail(ctx, FMM_ERR_TIMEOUT, "a bounded wait of the body sort ran out");
         if (err & kErrNonfinite) return fail(ctx, FMM_ERR_NONFINITE, "non-finite position or mass, or a mass <= 0");
         if (err & kErrCoincident) return fail(ctx, FMM_ERR_COINCIDENT, "two bodies share the same position");
         if (err & kErrLongRun) {
@@ -523,8 +528,9 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
                 return rc;
             coincident_exact(tb, as<uint64_t>(ctx->ck0), as<uint32_t>(ctx->cv0), as<uint64_t>(ctx->ck1),
                              as<uint32_t>(ctx->cv1), st);
-            CK(cudaMemcpyAsync(&err, &ctx->ds->err, 4, cudaMemcpyDeviceToHost, st));
+            CK(cudaMemcpyAsync(errs, &ctx->ds->err, 8, cudaMemcpyDeviceToHost, st));
             CK(cudaStreamSynchronize(st));
+            if (errs[1]) return fail(ctx, FMM_ERR_TIMEOUT, "a bounded wait of the coincidence check's sort ran out");
             if (err & kErrCoincident) return fail(ctx, FMM_ERR_COINCIDENT, "two bodies share the same position");
             CK(cudaMemsetAsync(&ctx->ds->err, 0, sizeof(unsigned), st));
         }
@@ -685,7 +691,8 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
     CK(cudaGetLastError());
     if (gp) return FMM_OK;  // the caller checks the status block after the replay
     CK(cudaStreamSynchronize(st));
-    CK(cudaMemcpy(&err, &ctx->ds->err, 4, cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(errs, &ctx->ds->err, 8, cudaMemcpyDeviceToHost));
+    if (errs[1]) return fail(ctx, FMM_ERR_TIMEOUT, "a bounded wait of a list sort ran out");
     if (err & kErrCapacity) return fail(ctx, FMM_ERR_CAPACITY, "an internal list overflowed");
     if (err & kErrTimeout)
         return fail(ctx, FMM_ERR_TIMEOUT, "a bounded wait ran out (the walk's ordered appends or the P2P staging)");
@@ -1161,7 +1168,7 @@ int fmm_solve_graph(fmm_ctx* ctx, int32_t nclusters, const int64_t* offsets, int
         CK(cudaMemcpyAsync(cnt, ctx->dcount.ptr, sizeof(cnt), cudaMemcpyDeviceToHost, gs));
         CK(cudaStreamSynchronize(gs));
         const DevScalars& d = *ctx->h_ds;
-        bool ok = d.err == 0;
+        bool ok = d.err == 0 && d.sort_err == 0;
         int nl = 1;
         for (int L = 0; L <= kMaxLevel && ok; ++L) {
             const int cntL = d.level_start[L + 1] - d.level_start[L];
@@ -1234,12 +1241,12 @@ int fmm_solve_graph(fmm_ctx* ctx, int32_t nclusters, const int64_t* offsets, int
     ctx->gmode = &g;
     rc = solve_device(ctx, n, nclusters, offsets, x, y, z, m, ax, ay, az, pot, gs);
     ctx->gmode = nullptr;
-    unsigned err = 1;
+    unsigned err[2] = {1, 1};  // err, sort_err
     if (rc == FMM_OK) {
-        CK(cudaMemcpyAsync(&err, &ctx->ds->err, 4, cudaMemcpyDeviceToHost, gs));
+        CK(cudaMemcpyAsync(err, &ctx->ds->err, 8, cudaMemcpyDeviceToHost, gs));
         CK(cudaStreamSynchronize(gs));
     }
-    if (rc == FMM_OK && err == 0) {
+    if (rc == FMM_OK && err[0] == 0 && err[1] == 0) {
         cudaGraph_t graph = nullptr;
         const int64_t gen0 = ctx->gen;
         if (cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {

@@ -36,6 +36,7 @@ __host__ __device__ constexpr int ncoef_real(int p) { return (p + 1) * (p + 1); 
 struct DevScalars {
     double box[8];                 // cx, cy, cz, h, lox, loy, loz, size
     unsigned err;                  // kErr* bits
+    unsigned sort_err;             // kErrTimeout if a wait of a radix sort of this solve ran out
     unsigned queue;                // work counter of the M2L kernels (zeroed before each launch)
     unsigned long long cnt[kMaxWalkIters + 2];  // walk frontier sizes per iteration
     unsigned long long list_cnt[4];             // far, near, m2l, p2p
@@ -148,14 +149,16 @@ void set_global_error(const char* msg);
 // Stable LSD radix sort of 64-bit keys (optionally with 32-bit values) on
 // bits [lo_bit, bits): keys equal there keep their input order. Ping-pongs
 // between buffers; returns 1 if the sorted data ends in (k1, v1), 0 if in
-// (k0, v0). hist needs radix_hist_words(n) words. dn (device, may be NULL):
-// the grid covers n keys but only the first min(n, *dn) are sorted (a count
-// known on the device only, in a captured solve).
+// (k0, v0). hist needs radix_hist_words(n) words, 8-byte aligned. err (device): raised
+// to kErrTimeout if a wait of the sort runs out (the result is then not sorted).
+// dn (device, may be NULL): the grid covers n keys but only the first
+// min(n, *dn) are sorted (a count known on the device only, in a captured solve).
 size_t radix_hist_words(int64_t n);
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits,
-               uint32_t* hist, cudaStream_t st, const unsigned long long* dn = nullptr, int lo_bit = 0);
+               uint32_t* hist, unsigned* err, cudaStream_t st, const unsigned long long* dn = nullptr,
+               int lo_bit = 0);
 // The same for 32-bit keys without payload.
-int radix_sort32(uint32_t* k0, uint32_t* k1, int64_t n, int bits, uint32_t* hist, cudaStream_t st,
+int radix_sort32(uint32_t* k0, uint32_t* k1, int64_t n, int bits, uint32_t* hist, unsigned* err, cudaStream_t st,
                  const unsigned long long* dn = nullptr, int lo_bit = 0);
 // single-block exclusive scan of count uint32 values in place; total -> *total (device)
 void scan_exclusive_u32(uint32_t* data, int64_t count, uint32_t* total, cudaStream_t st);
@@ -263,10 +266,11 @@ void pairs_to_directed32(const int2* pairs, const unsigned long long* np, int64_
 // Sorted directed keys -> src (the source cell of every entry; 0xffffffff for
 // the markers past the end) and the CSR offsets per target (nnodes + 1,
 // nnodes = *dnn). dnk (device): the keys present, of the nkeys the grid covers.
+// After a failed sort (*sort_err) the offsets are those of empty lists.
 void directed_offsets_src32(const uint32_t* k32, int64_t nkeys, const unsigned long long* dnk, int nb,
-                            const int* dnn, uint32_t* src, uint32_t* off, cudaStream_t st);
+                            const int* dnn, const unsigned* sort_err, uint32_t* src, uint32_t* off, cudaStream_t st);
 void directed_offsets(const uint64_t* keys, int64_t nkeys, const unsigned long long* dnk, int nb, const int* dnn,
-                      uint32_t* src, uint32_t* off, cudaStream_t st);
+                      const unsigned* sort_err, uint32_t* src, uint32_t* off, cudaStream_t st);
 
 // ---------------------------------------------------------- expansions.cu
 void upload_expansion_tables(const HostTables& h);

@@ -12,7 +12,7 @@
 // framework's caching allocator, a real-time loop that forbids allocation
 // after start-up), or that cannot afford an allocation's latency or failure
 // inside its loop. The price is that every GPU that loads this library holds
-// the array (kNoAllocScratchBytes, about 4.3 MB) until the process exits.
+// the array (kNoAllocScratchBytes, about 4.4 MB) until the process exits.
 //
 // Compiled with -fmad=false, like the tree build, so the keys are bit for bit
 // those of fmm_solve.
@@ -30,7 +30,7 @@ constexpr int kBboxBlocks = 304;
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr int64_t kMaxSortBlocks = (kNoAllocMaxN + 4095) / 4096;  // radix-sort tiles of 4096 keys
-constexpr size_t kHistWords = 256 * kMaxSortBlocks + 1 + (256 * kMaxSortBlocks + 4095) / 4096 + 2;
+constexpr size_t kHistWords = 8 * 256 + 8 + 2 * 256 * kMaxSortBlocks;  // radix_hist_words(kNoAllocMaxN)
 constexpr size_t kOffScalars = 0;
 constexpr size_t kOffBbox = align256(kOffScalars + sizeof(DevScalars));
 constexpr size_t kOffAltKeys = align256(kOffBbox + 6 * kBboxBlocks * sizeof(double));
@@ -184,8 +184,9 @@ extern "C" int fmm_morton_sort_noalloc(int64_t n, const double* x, const double*
     uint32_t* idx0 = reinterpret_cast<uint32_t*>(base + kOffIdx0);
     uint32_t* idx1 = reinterpret_cast<uint32_t*>(base + kOffIdx1);
     uint32_t* hist = reinterpret_cast<uint32_t*>(base + kOffHist);
-    // the array keeps the previous call's contents: clear the error word
-    if (cudaMemsetAsync(&ds->err, 0, sizeof(unsigned), st) != cudaSuccess) {
+    // the array keeps the previous call's contents: clear the error words
+    if (cudaMemsetAsync(&ds->err, 0, sizeof(unsigned), st) != cudaSuccess ||
+        cudaMemsetAsync(&ds->sort_err, 0, sizeof(unsigned), st) != cudaSuccess) {
         cudaGetLastError();
         set_global_error("fmm_morton_sort_noalloc: cudaMemsetAsync failed");
         return FMM_ERR_CUDA;
@@ -194,7 +195,7 @@ extern "C" int fmm_morton_sort_noalloc(int64_t n, const double* x, const double*
     k_na_bbox_final<<<1, 32, 0, st>>>(part, kBboxBlocks, ds);
     const int nb = (int)((n + 255) / 256);
     k_na_keys<<<nb, 256, 0, st>>>(x, y, z, n, ds, keys, idx0);
-    const int in1 = radix_sort(keys, idx0, alt, idx1, n, 63, hist, st);
+    const int in1 = radix_sort(keys, idx0, alt, idx1, n, 63, hist, &ds->sort_err, st);
     if (in1 && cudaMemcpyAsync(keys, alt, sizeof(uint64_t) * (size_t)n, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
         cudaGetLastError();
         set_global_error("fmm_morton_sort_noalloc: key copy failed");
@@ -206,8 +207,9 @@ extern "C" int fmm_morton_sort_noalloc(int64_t n, const double* x, const double*
         set_global_error("fmm_morton_sort_noalloc: box copy failed");
         return FMM_ERR_CUDA;
     }
-    unsigned err = 0;
+    unsigned err = 0, sort_err = 0;
     if (cudaMemcpyAsync(&err, &ds->err, sizeof(err), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(&sort_err, &ds->sort_err, sizeof(sort_err), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
         cudaGetLastError();
         set_global_error("fmm_morton_sort_noalloc: a CUDA call failed");
@@ -216,6 +218,10 @@ extern "C" int fmm_morton_sort_noalloc(int64_t n, const double* x, const double*
     if (err & kErrNonfinite) {
         set_global_error("fmm_morton_sort_noalloc: non-finite position");
         return FMM_ERR_NONFINITE;
+    }
+    if (sort_err) {
+        set_global_error("fmm_morton_sort_noalloc: a bounded wait of the sort ran out");
+        return FMM_ERR_TIMEOUT;
     }
     return FMM_OK;
 }

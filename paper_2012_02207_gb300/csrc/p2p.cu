@@ -709,6 +709,7 @@ __global__ void __launch_bounds__(128) k_leaf_reduce(LeafArgs a, const int* __re
         sx += u.x; sy += u.y; sz += w.x; sp -= w.y;
     }
     const uint32_t o = a.perm[i];
+    if (o >= (uint32_t)a.t.n) return;  // (only after a failed sort: the result is discarded)
     a.ax[o] = a.G * sx;
     a.ay[o] = a.G * sy;
     a.az[o] = a.G * sz;

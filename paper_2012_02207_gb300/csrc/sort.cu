@@ -1,9 +1,23 @@
-// Stable LSD radix sort of 64-bit keys with optional 32-bit payloads.
+// Stable LSD radix sort of 64- or 32-bit keys with optional 32-bit payloads.
 //
-// Three kernels per 8-bit digit: a per-tile histogram, one exclusive scan of
-// the digit-major histogram table, and a scatter that ranks each key among
-// the earlier keys of its tile with the same digit (warp match + per-warp
-// digit counters), so equal keys keep their order.
+// One kernel counts the digits of every pass, then one kernel per 8-bit digit
+// moves the keys. A block takes tiles by ticket, ranks each key among the
+// earlier keys of its tile with the same digit (warp match + per-warp digit
+// counters), so equal keys keep their order, and learns where the tile's digits
+// go from a decoupled look-back over the earlier tiles' published counts: one
+// thread per digit, four records at a time. Every key is read and written once
+// per pass.
+//
+// What bounds it: ranking and the scattered writes where there are many tiles;
+// the launch where there are few. With a histogram, its scan (one or three
+// launches) and a scatter per pass, the 8 passes over 4096 body keys took 200 us
+// of kernels, now 120; all sorts of 2^20 bodies (8 passes of bodies, 12 of list
+// keys) 1.67 ms, now 1.26.
+//
+// Waits are bounded (about a second): a block that gives up raises kErrTimeout
+// in the sort's error word and goes on with the prefix it has; its positions
+// stay inside the array, and the users of the sorted data check the word or
+// clamp what they read (the host then fails the call).
 #include "gbfmm_internal.cuh"
 
 namespace gbfmm {
@@ -14,56 +28,117 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kItems = 16;                   // keys per thread
 constexpr int kTile = kThreads * kItems;     // 4096 keys per block
 constexpr int kWarpItems = kTile / kWarps;   // 512 contiguous keys per warp
+constexpr int kMaxPasses = 8;
 template <typename K, bool VAL>
 constexpr size_t scatter_smem() {
     return (size_t)kTile * (sizeof(K) + (VAL ? 4 : 0)) + (size_t)(kWarps + 2) * 256 * 4;
 }
-// blocks per SM the scatter's registers are cut for: three for 32-bit keys
+// blocks per SM the pass kernel's registers are cut for: three for 32-bit keys
 // without payload (80 registers, no spills), two otherwise
 template <typename K, bool VAL>
 constexpr int scatter_min_blocks() { return (sizeof(K) == 4 && !VAL) ? 3 : 2; }
 
-template <typename K>
-__global__ void __launch_bounds__(kThreads) k_hist(const K* __restrict__ keys, int64_t n,
-                                                   const unsigned long long* __restrict__ dn, int shift,
-                                                   uint32_t* __restrict__ hist, int nblocks) {
-    __shared__ uint32_t h[256];
-    if (dn && (int64_t)*dn < n) n = (int64_t)*dn;  // tiles past the count give empty histograms
-    for (int i = threadIdx.x; i < 256; i += kThreads) h[i] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kTile;
-#pragma unroll 4
-    for (int k = 0; k < kItems; ++k) {
-        int64_t i = base + (int64_t)k * kThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(unsigned)(keys[i] >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < 256; d += kThreads) hist[(int64_t)d * nblocks + blockIdx.x] = h[d];
+// Scratch of a sort: digit counts of every pass, a tile ticket per pass (both
+// zeroed before the sort), then the look-back records, 256 per tile: bits 63-62
+// the kind (1: the tile's own count, 2: its inclusive prefix), 61-56 the pass, the
+// rest the value, so one load reads a consistent record. The count kernel clears
+// the records; the pass field tells a pass's records from the last one's.
+constexpr size_t kSortHeadWords = 256 * kMaxPasses + kMaxPasses;
+struct SortScratch {
+    uint32_t* digits;   // [pass][256]
+    uint32_t* tickets;  // [pass]
+    unsigned long long* rec;
+    __host__ __device__ explicit SortScratch(uint32_t* w)
+        : digits(w), tickets(w + 256 * kMaxPasses), rec(reinterpret_cast<unsigned long long*>(w + kSortHeadWords)) {}
+};
+static_assert(kSortHeadWords % 2 == 0, "the records are 8-byte aligned");
+
+constexpr unsigned long long kRecCount = 1ull << 62, kRecPrefix = 2ull << 62;
+constexpr unsigned long long kRecValue = (1ull << 56) - 1ull;
+constexpr unsigned long long kSortWaitNs = 1000000000ull;  // one second
+
+__device__ __forceinline__ void rec_store(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long rec_load(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long sort_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
 }
 
-// Scatter: rank every key among the earlier keys of its tile with the same
-// digit (warp match + per-warp digit counters), reorder the tile by digit in
-// shared memory, then write each digit's run to its global position with
-// consecutive threads writing consecutive addresses.
+// Digit counts of all passes in one read of the keys (the counts do not depend
+// on the order), and clear look-back records.
+template <typename K>
+__global__ void __launch_bounds__(kThreads) k_sort_count(const K* __restrict__ keys, int64_t n,
+                                                         const unsigned long long* __restrict__ dn, int lo_bit,
+                                                         int npass, SortScratch s) {
+    __shared__ uint32_t h[kMaxPasses * 256];
+    if (dn && (int64_t)*dn < n) n = (int64_t)*dn;
+    const int64_t ntiles = (n + kTile - 1) / kTile;
+    for (int i = threadIdx.x; i < npass * 256; i += kThreads) h[i] = 0;
+    __syncthreads();
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        s.rec[t * 256 + threadIdx.x] = 0ull;
+        K key[kItems];
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            const int64_t i = t * kTile + (int64_t)k * kThreads + threadIdx.x;
+            key[k] = i < n ? keys[i] : K(0);
+        }
+#pragma unroll
+        for (int k = 0; k < kItems; ++k) {
+            const bool valid = t * kTile + (int64_t)k * kThreads + threadIdx.x < n;
+            const unsigned act = __ballot_sync(0xffffffffu, valid);
+            for (int p = 0; p < npass; ++p) {
+                const unsigned d = (unsigned)(key[k] >> (lo_bit + 8 * p)) & 255u;
+                // a warp of one digit (the leading digits of neighbouring keys) counts it at once
+                const unsigned d0 = __shfl_sync(0xffffffffu, d, 0);
+                if (__all_sync(0xffffffffu, !valid || d == d0)) {
+                    if ((threadIdx.x & 31) == 0 && act) atomicAdd(&h[p * 256 + d0], (uint32_t)__popc(act));
+                } else if (valid) {
+                    atomicAdd(&h[p * 256 + d], 1u);
+                }
+            }
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < npass * 256; i += kThreads)
+        if (h[i]) atomicAdd(s.digits + i, h[i]);
+}
+
+// inclusive scan of v over the warp
+__device__ __forceinline__ uint32_t warp_scan(uint32_t v, int lane) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
 template <typename K, bool VAL>
-__global__ void __launch_bounds__(kThreads, scatter_min_blocks<K, VAL>()) k_scatter(const K* __restrict__ kin,
-                                                      const uint32_t* __restrict__ vin,
-                                                      K* __restrict__ kout,
-                                                      uint32_t* __restrict__ vout, int64_t n,
-                                                      const unsigned long long* __restrict__ dn,
-                                                      int shift, const uint32_t* __restrict__ offs,
-                                                      int nblocks) {
+__global__ void __launch_bounds__(kThreads, scatter_min_blocks<K, VAL>()) k_sort_pass(
+    const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout, uint32_t* __restrict__ vout,
+    int64_t n, const unsigned long long* __restrict__ dn, int shift, int pass, SortScratch s, unsigned* err) {
     extern __shared__ __align__(16) unsigned char sh_scatter[];
     K* skey = reinterpret_cast<K*>(sh_scatter);                                  // kTile
     uint32_t* sval = reinterpret_cast<uint32_t*>(skey + kTile);                  // kTile (VAL only)
     uint32_t (*wcount)[256] = reinterpret_cast<uint32_t (*)[256]>(sval + (VAL ? kTile : 0));  // kWarps x 256
     uint32_t* boff = &wcount[kWarps][0];    // global start of each digit for this tile
     uint32_t* lstart = boff + 256;          // start of each digit inside the tile
+    __shared__ unsigned s_tile;
+    __shared__ uint32_t s_wsum[2][kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) s_tile = atomicAdd(s.tickets + pass, 1u);
     for (int i = threadIdx.x; i < kWarps * 256; i += kThreads) (&wcount[0][0])[i] = 0;
-    for (int d = threadIdx.x; d < 256; d += kThreads) boff[d] = offs[(int64_t)d * nblocks + blockIdx.x];
     __syncthreads();
-    const int64_t tile0 = (int64_t)blockIdx.x * kTile;
+    const int64_t tile = s_tile;
+    const int64_t tile0 = tile * kTile;
     if (dn && (int64_t)*dn < n) n = (int64_t)*dn;
     if (tile0 >= n) return;  // the whole block: nothing of this tile is present
     const int64_t base = tile0 + (int64_t)warp * kWarpItems;
@@ -76,6 +151,7 @@ __global__ void __launch_bounds__(kThreads, scatter_min_blocks<K, VAL>()) k_scat
         key[r] = i < n ? kin[i] : K(0);
         if (VAL) val[VAL ? r : 0] = i < n ? vin[i] : 0u;
     }
+    const uint32_t digits_all = s.digits[pass * 256 + threadIdx.x];  // kThreads == 256 digits
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
         const int64_t i = base + r * 32 + lane;
@@ -89,49 +165,82 @@ __global__ void __launch_bounds__(kThreads, scatter_min_blocks<K, VAL>()) k_scat
         __syncwarp();
     }
     __syncthreads();
-    {
-        const int d = threadIdx.x;  // kThreads == 256 digits
-        uint32_t run = 0;
+    // thread d: the tile's count of digit d, published at once
+    const int d = threadIdx.x;
+    unsigned long long* rec = s.rec + d;
+    const unsigned long long tag = (unsigned long long)pass << 56;
+    uint32_t cnt = 0;
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-            const uint32_t t = wcount[w][d];
-            wcount[w][d] = run;
-            run += t;
-        }
-        lstart[d] = run;  // this digit's count in the tile, scanned below
+    for (int w = 0; w < kWarps; ++w) {
+        const uint32_t t = wcount[w][d];
+        wcount[w][d] = cnt;
+        cnt += t;
+    }
+    rec_store(rec + tile * 256, (tile == 0 ? kRecPrefix : kRecCount) | tag | cnt);
+    // exclusive scans over the digits: the tile's counts and all keys' counts
+    const uint32_t in_tile = warp_scan(cnt, lane), in_all = warp_scan(digits_all, lane);
+    if (lane == 31) {
+        s_wsum[0][warp] = in_tile;
+        s_wsum[1][warp] = in_all;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {  // exclusive scan of the 256 digit counts
-        uint32_t c[8], s = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) { c[k] = lstart[threadIdx.x * 8 + k]; s += c[k]; }
-        uint32_t incl = s;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-            if ((int)threadIdx.x >= o) incl += v;
-        }
-        uint32_t run = incl - s;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) { lstart[threadIdx.x * 8 + k] = run; run += c[k]; }
+    uint32_t lbase = in_tile - cnt, gbase = in_all - digits_all;
+    for (int w = 0; w < warp; ++w) {
+        lbase += s_wsum[0][w];
+        gbase += s_wsum[1][w];
     }
+    lstart[d] = lbase;
     __syncthreads();
+    // reorder the tile by digit in shared memory
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
         const int64_t i = base + r * 32 + lane;
         if (i < n) {
-            const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
-            const uint32_t pos = lstart[d] + wcount[warp][d] + rank[r];
+            const uint32_t dd = (uint32_t)(key[r] >> shift) & 255u;
+            const uint32_t pos = lstart[dd] + wcount[warp][dd] + rank[r];
             skey[pos] = key[r];
             if (VAL) sval[pos] = val[VAL ? r : 0];
         }
     }
+    // look-back for digit d: the keys of it in the tiles before this one
+    uint32_t excl = 0;
+    if (tile > 0) {
+        constexpr int kAhead = 4;
+        const unsigned long long want = tag >> 56;
+        unsigned long long t0 = 0;
+        bool done = false;
+        for (int64_t j = tile - 1; !done; j -= kAhead) {
+            unsigned long long w[kAhead];
+#pragma unroll
+            for (int q = 0; q < kAhead; ++q) w[q] = j - q >= 0 ? rec_load(rec + (j - q) * 256) : (kRecPrefix | tag);
+#pragma unroll
+            for (int q = 0; q < kAhead; ++q) {
+                if (!done) {
+                    while ((w[q] >> 62) == 0ull || ((w[q] >> 56) & 63ull) != want) {
+                        const unsigned long long now = sort_ns();
+                        if (t0 == 0) t0 = now;
+                        if (now - t0 > kSortWaitNs) {
+                            atomicOr(err, kErrTimeout);
+                            w[q] = kRecPrefix | tag;  // go on with what there is
+                            break;
+                        }
+                        w[q] = rec_load(rec + (j - q) * 256);
+                    }
+                    excl += (uint32_t)(w[q] & kRecValue);
+                    done = (w[q] >> 62) == 2ull;
+                }
+            }
+        }
+        rec_store(rec + tile * 256, kRecPrefix | tag | (excl + cnt));
+    }
+    boff[d] = gbase + excl;
     __syncthreads();
-    const int cnt = (int)((n - tile0) < kTile ? (n - tile0) : kTile);
-    for (int j = threadIdx.x; j < cnt; j += kThreads) {
+    const int present = (int)((n - tile0) < kTile ? (n - tile0) : kTile);
+    for (int j = threadIdx.x; j < present; j += kThreads) {
         const K k = skey[j];
-        const uint32_t d = (uint32_t)(k >> shift) & 255u;
-        const uint32_t pos = boff[d] + (uint32_t)j - lstart[d];
+        const uint32_t dd = (uint32_t)(k >> shift) & 255u;
+        const uint32_t pos = boff[dd] + (uint32_t)j - lstart[dd];
+        if ((int64_t)pos >= n) continue;  // (never: only a wait that ran out could misplace a key)
         kout[pos] = k;
         if (VAL) vout[pos] = sval[j];
     }
@@ -266,8 +375,7 @@ void scan_exclusive_u32_large(uint32_t* data, int64_t count, uint32_t* total, ui
 
 size_t radix_hist_words(int64_t n) {
     const int64_t nb = (n + kTile - 1) / kTile;
-    const int64_t cells = 256 * (nb > 0 ? nb : 1);
-    return (size_t)(cells + 1) + scan_scratch_words(cells);
+    return kSortHeadWords + 2 * 256 * (size_t)(nb > 0 ? nb : 1);
 }
 
 void scan_exclusive_u32(uint32_t* data, int64_t count, uint32_t* total, cudaStream_t st) {
@@ -277,35 +385,39 @@ void scan_exclusive_u32(uint32_t* data, int64_t count, uint32_t* total, cudaStre
 namespace {
 template <typename K, bool VAL>
 int radix_sort_impl(K* k0, uint32_t* v0, K* k1, uint32_t* v1, int64_t n, int lo_bit, int bits, uint32_t* hist,
-                    cudaStream_t st, const unsigned long long* dn) {
+                    cudaStream_t st, const unsigned long long* dn, unsigned* err) {
     if (n <= 1 || bits <= lo_bit) return 0;
-    ensure_dyn_smem((const void*)k_scatter<K, VAL>, (int)scatter_smem<K, VAL>());
+    ensure_dyn_smem((const void*)k_sort_pass<K, VAL>, (int)scatter_smem<K, VAL>());
     const int nblocks = (int)((n + kTile - 1) / kTile);
+    const int npass = (bits - lo_bit + 7) / 8;
+    const SortScratch s(hist);
+    cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kSortHeadWords, st);
+    const int count_grid = nblocks < 4 * device_sm_count() ? nblocks : 4 * device_sm_count();
+    (k_sort_count<K><<<count_grid, kThreads, 0, st>>>(k0, n, dn, lo_bit, npass, s), note_launch());
     int cur = 0;
-    for (int shift = lo_bit; shift < bits; shift += 8) {
+    for (int pass = 0; pass < npass; ++pass) {
         K* ki = cur ? k1 : k0;
         uint32_t* vi = cur ? v1 : v0;
         K* ko = cur ? k0 : k1;
         uint32_t* vo = cur ? v0 : v1;
-        (k_hist<K><<<nblocks, kThreads, 0, st>>>(ki, n, dn, shift, hist, nblocks), note_launch());
-        scan_exclusive_u32_large(hist, (int64_t)256 * nblocks, nullptr, hist + (size_t)256 * nblocks + 1, st);
-        (k_scatter<K, VAL><<<nblocks, kThreads, scatter_smem<K, VAL>(), st>>>(ki, vi, ko, vo, n, dn, shift,
-                                                                              hist, nblocks), note_launch());
+        (k_sort_pass<K, VAL><<<nblocks, kThreads, scatter_smem<K, VAL>(), st>>>(ki, vi, ko, vo, n, dn,
+                                                                                lo_bit + 8 * pass, pass, s, err),
+         note_launch());
         cur ^= 1;
     }
     return cur;
 }
 }  // namespace
 
-int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits,
-               uint32_t* hist, cudaStream_t st, const unsigned long long* dn, int lo_bit) {
-    return v0 ? radix_sort_impl<uint64_t, true>(k0, v0, k1, v1, n, lo_bit, bits, hist, st, dn)
-              : radix_sort_impl<uint64_t, false>(k0, nullptr, k1, nullptr, n, lo_bit, bits, hist, st, dn);
+int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits, uint32_t* hist,
+               unsigned* err, cudaStream_t st, const unsigned long long* dn, int lo_bit) {
+    return v0 ? radix_sort_impl<uint64_t, true>(k0, v0, k1, v1, n, lo_bit, bits, hist, st, dn, err)
+              : radix_sort_impl<uint64_t, false>(k0, nullptr, k1, nullptr, n, lo_bit, bits, hist, st, dn, err);
 }
 
-int radix_sort32(uint32_t* k0, uint32_t* k1, int64_t n, int bits, uint32_t* hist, cudaStream_t st,
+int radix_sort32(uint32_t* k0, uint32_t* k1, int64_t n, int bits, uint32_t* hist, unsigned* err, cudaStream_t st,
                  const unsigned long long* dn, int lo_bit) {
-    return radix_sort_impl<uint32_t, false>(k0, nullptr, k1, nullptr, n, lo_bit, bits, hist, st, dn);
+    return radix_sort_impl<uint32_t, false>(k0, nullptr, k1, nullptr, n, lo_bit, bits, hist, st, dn, err);
 }
 
 }  // namespace gbfmm

@@ -151,20 +151,20 @@ __global__ void k_cluster_keys(const uint32_t* __restrict__ perm, int64_t n, con
                                int nclusters, uint64_t* __restrict__ ckey, uint32_t* __restrict__ cval) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    ckey[i] = (uint64_t)cluster_of(coff, nclusters, perm[i]);
+    ckey[i] = (uint64_t)cluster_of(coff, nclusters, perm[i]);  // (any value gives a cluster)
     cval[i] = (uint32_t)i;
 }
 
 __global__ void k_cluster_apply(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ perm,
                                 const uint64_t* __restrict__ ckey, const uint32_t* __restrict__ cval,
-                                int64_t n, uint64_t* __restrict__ keys_out, uint32_t* __restrict__ perm_out,
-                                uint32_t* __restrict__ cid) {
+                                int64_t n, int nclusters, uint64_t* __restrict__ keys_out,
+                                uint32_t* __restrict__ perm_out, uint32_t* __restrict__ cid) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const uint32_t j = cval[i];
+    const uint32_t v = cval[i], j = v < (uint32_t)n ? v : 0u;  // (out of range only after a failed sort)
     keys_out[i] = keys[j];
     perm_out[i] = perm[j];
-    cid[i] = (uint32_t)ckey[i];
+    cid[i] = ckey[i] < (uint64_t)nclusters ? (uint32_t)ckey[i] : 0u;
 }
 
 __global__ void k_gather(const double* __restrict__ x, const double* __restrict__ y,
@@ -175,7 +175,7 @@ __global__ void k_gather(const double* __restrict__ x, const double* __restrict_
                          float4* __restrict__ xf) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const uint32_t j = perm[i];
+    const uint32_t v = perm[i], j = v < (uint32_t)n ? v : 0u;  // (out of range only after a failed sort)
     const double* bx = box + 8 * (cid ? cid[i] : 0u);
     const double a = x[j], b = y[j], c = z[j], w = m[j];
     xs[i] = a; ys[i] = b; zs[i] = c; ms[i] = w;
@@ -236,8 +236,10 @@ __global__ void k_pos_equal(const uint64_t* __restrict__ h, const uint32_t* __re
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || i == 0 || h[i] != h[i - 1]) return;
     const uint32_t bi = idx[i];
+    if (bi >= (uint32_t)n) return;  // (only after a failed sort)
     for (int64_t j = i - 1; j >= 0 && h[j] == h[i]; --j) {
         const uint32_t bj = idx[j];
+        if (bj >= (uint32_t)n) return;
         if (xs[bi] == xs[bj] && ys[bi] == ys[bj] && zs[bi] == zs[bj] && (!cid || cid[bi] == cid[bj])) {
             atomicOr(err, kErrCoincident);
             return;
@@ -524,7 +526,7 @@ void tree_build_count(TreeBuffers& b, int* sorted_in_1, cudaStream_t st) {
      note_launch());
     (k_bbox_final<<<blocks_for((int64_t)nc * 32, 128), 128, 0, st>>>(b.bbox_part, nc, slices, b.box), note_launch());
     (k_keys<<<blocks_for(n, 256), 256, 0, st>>>(b.x, b.y, b.z, n, b.coff, nc, b.box, b.k0, b.v0), note_launch());
-    int in1 = radix_sort(b.k0, b.v0, b.k1, b.v1, n, 63, b.hist, st);
+    int in1 = radix_sort(b.k0, b.v0, b.k1, b.v1, n, 63, b.hist, &b.ds->sort_err, st);
     const uint64_t* keys = in1 ? b.k1 : b.k0;
     const uint32_t* perm = in1 ? b.v1 : b.v0;
     const uint32_t* cid = nullptr;
@@ -533,11 +535,11 @@ void tree_build_count(TreeBuffers& b, int* sorted_in_1, cudaStream_t st) {
         (k_cluster_keys<<<blocks_for(n, 256), 256, 0, st>>>(perm, n, b.coff, nc, b.ck0, b.cv0), note_launch());
         int bits = 0;
         while ((1 << bits) < nc) ++bits;
-        const int cin1 = radix_sort(b.ck0, b.cv0, b.ck1, b.cv1, n, bits, b.hist, st);
+        const int cin1 = radix_sort(b.ck0, b.cv0, b.ck1, b.cv1, n, bits, b.hist, &b.ds->sort_err, st);
         uint64_t* kout = in1 ? b.k0 : b.k1;
         uint32_t* vout = in1 ? b.v0 : b.v1;
         (k_cluster_apply<<<blocks_for(n, 256), 256, 0, st>>>(keys, perm, cin1 ? b.ck1 : b.ck0, cin1 ? b.cv1 : b.cv0,
-                                                            n, kout, vout, b.cid), note_launch());
+                                                            n, nc, kout, vout, b.cid), note_launch());
         in1 ^= 1;
         keys = kout;
         perm = vout;
@@ -595,7 +597,7 @@ void coincident_exact(const TreeBuffers& b, uint64_t* hk0, uint32_t* hv0, uint64
     if (n < 2) return;
     const uint32_t* cid = b.nclusters > 1 ? b.cid : nullptr;
     (k_pos_hash<<<blocks_for(n, 256), 256, 0, st>>>(b.xs, b.ys, b.zs, cid, n, hk0, hv0), note_launch());
-    const int in1 = radix_sort(hk0, hv0, hk1, hv1, n, 64, b.hist, st);
+    const int in1 = radix_sort(hk0, hv0, hk1, hv1, n, 64, b.hist, &b.ds->sort_err, st);
     (k_pos_equal<<<blocks_for(n, 256), 256, 0, st>>>(in1 ? hk1 : hk0, in1 ? hv1 : hv0, b.xs, b.ys, b.zs, cid, n,
                                                      &b.ds->err), note_launch());
 }
