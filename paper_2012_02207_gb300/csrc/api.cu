@@ -141,7 +141,6 @@ struct fmm_ctx {
     // sizes, split flags and scan, the fast count; per-depth slow/fast lists
     Buf h_all, h_gat, h_acc, h_acc2, h_tau, h_flag, h_scan, h_scr, h_nf;
     std::vector<Buf> h_S, h_F;
-    Buf dpart;       // per-segment partial sums of the direct sum
     Buf step_upper;  // per-body bounds of the step sizes
     // walk and lists
     // per list: sorted directed keys, the sort's second buffer (its own, so a
@@ -819,22 +818,14 @@ struct HoldRun {
     int64_t kicks = 0, fmm_solves = 0, direct_solves = 0, max_depth = 0, splits = 0;
 };
 
-// scratch of a direct sum over n bodies at ntgt targets
-int ensure_direct(fmm_ctx* ctx, int64_t n, int64_t ntgt) {
-    const int nseg = direct_segments(n, ntgt);
-    return nseg > 1 ? ensure(ctx, ctx->dpart, sizeof(double) * 4 * (size_t)ntgt * nseg, false) : FMM_OK;
-}
-
 // accelerations of the first ntgt of k compact bodies (columns of g, stride k)
 // from all k, into acc (3 columns of stride k; a 4th column is scratch)
 int hold_force(HoldRun& R, int k, const double* g, int ntgt, double* acc, bool force_direct) {
     fmm_ctx* ctx = R.ctx;
     const size_t K = (size_t)k;
     if (force_direct || k < R.direct_below) {
-        const int rc = ensure_direct(ctx, k, ntgt);
-        if (rc != FMM_OK) return rc;
         direct_sum_f64(k, g, g + K, g + 2 * K, g + 6 * K, ctx->cfg.G, ctx->cfg.soft, ntgt, nullptr, acc, acc + K,
-                       acc + 2 * K, acc + 3 * K, as<double>(ctx->dpart), R.st);
+                       acc + 2 * K, acc + 3 * K, R.st);
         CK(cudaGetLastError());
         R.direct_solves++;
         return FMM_OK;
@@ -1056,7 +1047,7 @@ void fmm_destroy(fmm_ctx* ctx) {
                   &ctx->part_lo, &ctx->work, &ctx->coff, &ctx->box, &ctx->ck0, &ctx->ck1, &ctx->cv0,
                   &ctx->cv1, &ctx->cid, &ctx->jv, &ctx->jv32, &ctx->jw, &ctx->jmom, &ctx->jmult,
                   &ctx->jmult32, &ctx->jloc, &ctx->jloc32, &ctx->h_all, &ctx->h_gat, &ctx->h_acc, &ctx->h_acc2,
-                  &ctx->h_tau, &ctx->h_flag, &ctx->h_scan, &ctx->h_scr, &ctx->h_nf, &ctx->geo, &ctx->dpart, &ctx->step_upper};
+                  &ctx->h_tau, &ctx->h_flag, &ctx->h_scan, &ctx->h_scr, &ctx->h_nf, &ctx->geo, &ctx->step_upper};
     for (Buf* b : all) release(*b);
     for (Buf& b : ctx->h_S) release(b);
     for (Buf& b : ctx->h_F) release(b);
@@ -1356,10 +1347,7 @@ int fmm_direct(fmm_ctx* ctx, int64_t n, const double* x, const double* y, const 
     if (n < 0 || ntargets < 0) return fail(ctx, FMM_ERR_ARG, "negative size");
     cudaSetDevice(ctx->device);
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const int64_t nt = targets ? ntargets : n;
-    const int rc = ensure_direct(ctx, n, nt);
-    if (rc != FMM_OK) return rc;
-    direct_sum_f64(n, x, y, z, m, ctx->cfg.G, ctx->cfg.soft, nt, targets, ax, ay, az, pot, as<double>(ctx->dpart), st);
+    direct_sum_f64(n, x, y, z, m, ctx->cfg.G, ctx->cfg.soft, targets ? ntargets : n, targets, ax, ay, az, pot, st);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(st));
     return FMM_OK;

@@ -434,11 +434,9 @@ size_t hold_small_smem(int k);
 void hold_small(int k, const int* idx, double* x, double* y, double* z, double* vx, double* vy, double* vz,
                 const double* m, double G, double soft, double eta, bool sym, double dt, double dt_min, int depth,
                 unsigned long long* stats, cudaStream_t st);
-// soft: Plummer softening length (0: Newtonian); part: scratch of
-// 4 ntgt direct_segments(n, ntgt) doubles when that is more than one segment
-int direct_segments(int64_t n, int64_t ntgt);
+// soft: Plummer softening length (0: Newtonian)
 void direct_sum_f64(int64_t n, const double* x, const double* y, const double* z, const double* m,
                     double G, double soft, int64_t ntgt, const int64_t* tgt, double* ax, double* ay, double* az,
-                    double* pot, double* part, cudaStream_t st);
+                    double* pot, cudaStream_t st);
 
 }  // namespace gbfmm

@@ -765,76 +765,65 @@ __global__ void k_leaf_bodies(TreeView t, const double* __restrict__ xs, const d
     }
 }
 
-// Direct FP64 sum, one thread per target, source tiles staged in shared
-// memory. Block (t, s) sums segment s of the sources; with more than one
-// segment the partial sums go to part (4 columns of ntgt per segment) and
-// k_direct_sum adds them in segment order. Bound by the FP64 pipe, 18
-// instructions a pair, once every SM has warps: 8192 targets of 131072 bodies
-// as 32 blocks of 256 took 241 ms, split into 19 segments 36.2 ms
-// (FP64 pipe 90% active).
-constexpr int kDirectThreads = 128;
-
-__global__ void __launch_bounds__(kDirectThreads) k_direct(int64_t n, const double* __restrict__ x,
-                                                           const double* __restrict__ y,
-                                                           const double* __restrict__ z,
-                                                           const double* __restrict__ m, double G, double soft2,
-                                                           int64_t seg, int64_t ntgt,
-                                                           const int64_t* __restrict__ tgt, double* ax, double* ay,
-                                                           double* az, double* pot, double* part) {
-    __shared__ double4 tile[kDirectThreads];
-    const int64_t t = (int64_t)blockIdx.x * kDirectThreads + threadIdx.x;
-    const bool act = t < ntgt;
-    const int64_t i = act ? (tgt ? tgt[t] : t) : 0;
-    const double xi = act ? x[i] : 0.0, yi = act ? y[i] : 0.0, zi = act ? z[i] : 0.0;
-    double sx = 0.0, sy = 0.0, sz = 0.0, sp = 0.0;
-    const int64_t jb = (int64_t)blockIdx.y * seg, je = jb + seg < n ? jb + seg : n;
-    for (int64_t j0 = jb; j0 < je; j0 += kDirectThreads) {
-        const int64_t j = j0 + threadIdx.x;
-        if (j < je) tile[threadIdx.x] = make_double4(x[j], y[j], z[j], m[j]);
-        __syncthreads();
-        const int cnt = (int)(je - j0 < kDirectThreads ? je - j0 : kDirectThreads);
-        const int self = act && i >= j0 && i < j0 + cnt ? (int)(i - j0) : -1;
-#pragma unroll 4
-        for (int k = 0; k < cnt; ++k) {
-            const double4 s = tile[k];
-            const double dx = s.x - xi, dy = s.y - yi, dz = s.z - zi;
+// Direct FP64 sum: each target's terms are added one after the other in source
+// order, as a plain loop adds them (the reference that errors are measured
+// with; a sum in segments is more exact, but another rounding). Only the additions
+// have to be serial: a warp takes T targets, its lanes form the terms of 32
+// sources for all of them in shared memory, then lane 4 t + c adds component c of
+// target t in order. Both halves keep every lane busy (T = 8), so the FP64
+// instructions are 22 a pair against 19 of a thread per target, and there is a
+// warp per 8 targets where that layout has one per 32: 8192 targets of 131072
+// bodies as 32 blocks of 256 threads took 241 ms with two Newton steps for 1/r,
+// this 45.1 (a sum in segments 36.2).
+template <int T>
+__global__ void __launch_bounds__(32) k_direct(int64_t n, const double* __restrict__ x, const double* __restrict__ y,
+                                               const double* __restrict__ z, const double* __restrict__ m, double G,
+                                               double soft2, int64_t ntgt, const int64_t* __restrict__ tgt,
+                                               double* ax, double* ay, double* az, double* pot) {
+    __shared__ double term[32][4 * T + 1];  // (an odd pitch: no bank conflicts by rows or columns)
+    const int lane = threadIdx.x;
+    const int64_t t0 = (int64_t)blockIdx.x * T;
+    double tx[T], ty[T], tz[T];
+    int64_t ti[T];
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+        const int64_t k = t0 + t < ntgt ? t0 + t : ntgt - 1;  // (the last target repeated: its copies are not written)
+        ti[t] = tgt ? tgt[k] : k;
+        tx[t] = x[ti[t]]; ty[t] = y[ti[t]]; tz[t] = z[ti[t]];
+    }
+    double sum = 0.0;  // lane 4 t + c: component c of target t
+    auto load = [&](int64_t j) { return j < n ? make_double4(x[j], y[j], z[j], m[j]) : make_double4(0, 0, 0, 0); };
+    double4 nxt = load(lane);
+    for (int64_t j0 = 0; j0 < n; j0 += 32) {
+        const double4 s = nxt;
+        const int64_t j = j0 + lane;
+        nxt = load(j + 32);
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            const double dx = s.x - tx[t], dy = s.y - ty[t], dz = s.z - tz[t];
             const double r2 = fma(dx, dx, fma(dy, dy, fma(dz, dz, soft2)));  // soft2 = 0: Newtonian
             double mr, mr3;
-            inv_powers(r2, k == self ? 0.0 : s.w, mr, mr3);
-            sx = fma(mr3, dx, sx);
-            sy = fma(mr3, dy, sy);
-            sz = fma(mr3, dz, sz);
-            sp += mr;
+            inv_powers(r2, j == ti[t] ? 0.0 : s.w, mr, mr3);
+            term[lane][4 * t] = mr3 * dx;
+            term[lane][4 * t + 1] = mr3 * dy;
+            term[lane][4 * t + 2] = mr3 * dz;
+            term[lane][4 * t + 3] = mr;
         }
-        __syncthreads();
+        __syncwarp();
+        const int cnt = n - j0 < 32 ? (int)(n - j0) : 32;
+        if (lane < 4 * T) {
+#pragma unroll 8
+            for (int k = 0; k < cnt; ++k) sum += term[k][lane];
+        }
+        __syncwarp();
     }
-    if (!act) return;
-    if (part) {
-        double* p = part + (size_t)blockIdx.y * 4 * ntgt + t;
-        p[0] = sx;
-        p[ntgt] = sy;
-        p[2 * ntgt] = sz;
-        p[3 * ntgt] = sp;
-        return;
-    }
-    ax[t] = G * sx;
-    ay[t] = G * sy;
-    az[t] = G * sz;
-    if (pot) pot[t] = -G * sp;
-}
-
-__global__ void k_direct_sum(int64_t ntgt, int nseg, double G, const double* __restrict__ part, double* ax,
-                             double* ay, double* az, double* pot) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ntgt) return;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int k = 0; k < nseg; ++k)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) s[c] += part[((size_t)k * 4 + c) * ntgt + t];
-    ax[t] = G * s[0];
-    ay[t] = G * s[1];
-    az[t] = G * s[2];
-    if (pot) pot[t] = -G * s[3];
+    const int64_t k = t0 + (lane >> 2);
+    if (lane >= 4 * T || k >= ntgt) return;
+    const int c = lane & 3;
+    if (c == 0) ax[k] = G * sum;
+    else if (c == 1) ay[k] = G * sum;
+    else if (c == 2) az[k] = G * sum;
+    else if (pot) pot[k] = -G * sum;
 }
 
 inline int blocks_for(int64_t n, int threads) { return (int)((n + threads - 1) / threads); }
@@ -1276,29 +1265,17 @@ void leaf_bodies(const TreeView& t, const double* xs, const double* ys, const do
      note_launch());
 }
 
-// Segments the sources are split into: as many as give every SM eight blocks
-// (its FP64 pipe is full from about eight warps on; the blocks all take the
-// same time), each of at least 256 sources.
-int direct_segments(int64_t n, int64_t ntgt) {
-    const int64_t blocks = (ntgt + kDirectThreads - 1) / kDirectThreads;
-    if (blocks < 1) return 1;
-    const int64_t want = 8 * (int64_t)device_sm_count() / blocks, most = n / 256;
-    const int64_t s = want < most ? want : most;
-    return s > 1 ? (int)s : 1;
-}
-
+// Eight targets a warp where that gives every SM four warps, else four.
 void direct_sum_f64(int64_t n, const double* x, const double* y, const double* z, const double* m,
                     double G, double soft, int64_t ntgt, const int64_t* tgt, double* ax, double* ay, double* az,
-                    double* pot, double* part, cudaStream_t st) {
+                    double* pot, cudaStream_t st) {
     if (ntgt <= 0) return;
-    const int nseg = direct_segments(n, ntgt);
-    const int64_t seg = (n + nseg - 1) / nseg;
-    const dim3 grid((unsigned)blocks_for(ntgt, kDirectThreads), (unsigned)nseg);
-    (k_direct<<<grid, kDirectThreads, 0, st>>>(n, x, y, z, m, G, soft * soft, seg, ntgt, tgt, ax, ay, az, pot,
-                                               nseg > 1 ? part : nullptr),
-     note_launch());
-    if (nseg > 1)
-        (k_direct_sum<<<blocks_for(ntgt, 128), 128, 0, st>>>(ntgt, nseg, G, part, ax, ay, az, pot), note_launch());
+    if (ntgt >= 8 * 4 * (int64_t)device_sm_count())
+        (k_direct<8><<<blocks_for(ntgt, 8), 32, 0, st>>>(n, x, y, z, m, G, soft * soft, ntgt, tgt, ax, ay, az, pot),
+         note_launch());
+    else
+        (k_direct<4><<<blocks_for(ntgt, 4), 32, 0, st>>>(n, x, y, z, m, G, soft * soft, ntgt, tgt, ax, ay, az, pot),
+         note_launch());
 }
 
 }  // namespace gbfmm
