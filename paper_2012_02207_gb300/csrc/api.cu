@@ -131,7 +131,7 @@ struct fmm_ctx {
     std::vector<int> h_coff;
     // per-node
     Buf level, begin, end, parent, first_child, nchild, M, S, zc, r, hs, Pk, mult, mult32, loc, loc32,
-        fmin, fscratch, zhi, zlo, contrib, Phat, r32;
+        fmin, fscratch, zhi, zlo, contrib, Phat, kids;
     // P2P work items
     Buf item_first, slot_first, item_leaf, leaf_of, part_hi, part_lo, work;
     // jerks: sorted velocities (FP64, FP32), dipole weights, order p-1 moments,
@@ -372,7 +372,7 @@ int run_walk(fmm_ctx* ctx, int mode, cudaStream_t st) {
         }
         dual_tree_walk(mode, t, as<double>(ctx->zc), as<double>(ctx->r), as<double>(ctx->Pk),
                        as<float>(ctx->fmin), p, ctx->cfg.eps, binom_row0, as<float4>(ctx->zhi),
-                       as<float4>(ctx->zlo), as<float>(ctx->r32), as<float>(ctx->Phat), as<double>(ctx->M),
+                       as<float4>(ctx->zlo), as<int2>(ctx->kids), as<float>(ctx->Phat), as<double>(ctx->M),
                        ctx->cfg.soft, wb, ctx->ds, ctx->h_ds, g->walk_iters[mode], st);
         walk_check_finished(ctx->ds, g->walk_iters[mode], st);
         CK(cudaGetLastError());
@@ -398,7 +398,7 @@ int run_walk(fmm_ctx* ctx, int mode, cudaStream_t st) {
         CK(cudaMemsetAsync(&ctx->ds->err, 0, sizeof(unsigned), st));
         const int it = dual_tree_walk(mode, t, as<double>(ctx->zc), as<double>(ctx->r), as<double>(ctx->Pk),
                                       as<float>(ctx->fmin), p, ctx->cfg.eps, binom_row, as<float4>(ctx->zhi),
-                                      as<float4>(ctx->zlo), as<float>(ctx->r32), as<float>(ctx->Phat),
+                                      as<float4>(ctx->zlo), as<int2>(ctx->kids), as<float>(ctx->Phat),
                                       as<double>(ctx->M), ctx->cfg.soft, wb, ctx->ds, ctx->h_ds, 0, st);
         if (it == FMM_ERR_CAPACITY) {
             // the counters kept counting past the capacity: grow to what was asked for
@@ -546,8 +546,8 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
         (rc = ensure(ctx, ctx->Pk, 8 * K * (p + 1))) || (rc = ensure(ctx, ctx->mult, 8 * K * nr)) ||
         (rc = ensure(ctx, ctx->fmin, 4 * K)) || (rc = ensure(ctx, ctx->fscratch, 4 * 2 * K)) ||
         (rc = ensure(ctx, ctx->zhi, 16 * K)) || (rc = ensure(ctx, ctx->zlo, 16 * K)) ||
-        (rc = ensure(ctx, ctx->contrib, 8 * K * nr)) || (rc = ensure(ctx, ctx->Phat, 4 * K * (p + 1))) ||
-        (rc = ensure(ctx, ctx->r32, 4 * K)) || (rc = ensure(ctx, ctx->geo, sizeof(double) * kShiftGeo * K)) ||
+        (rc = ensure(ctx, ctx->contrib, 8 * K * nr)) || (rc = ensure(ctx, ctx->Phat, 4 * K * phat_stride(p))) ||
+        (rc = ensure(ctx, ctx->kids, 8 * K)) || (rc = ensure(ctx, ctx->geo, sizeof(double) * kShiftGeo * K)) ||
         (rc = ensure(ctx, ctx->item_first, 4 * (K + 2))) || (rc = ensure(ctx, ctx->slot_first, 4 * (K + 2))) ||
         (rc = ensure(ctx, ctx->leaf_of, 4 * N)) || (rc = ensure(ctx, ctx->work, 64)))
         return rc;
@@ -581,14 +581,13 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
     cell_geometry(t, as<double>(ctx->xs), as<double>(ctx->ys), as<double>(ctx->zs), as<double>(ctx->ms),
                   ctx->h_level_start, as<double>(ctx->M), as<double>(ctx->S), as<double>(ctx->zc),
                   as<double>(ctx->r), st);
-    hat_scales(t, as<int>(ctx->parent), as<double>(ctx->r), as<double>(ctx->hs), st);
-    shift_geometry(t, as<double>(ctx->zc), as<double>(ctx->hs), as<double>(ctx->geo), st);
-    node_centres_f32(t, as<double>(ctx->zc), as<double>(ctx->hs), as<float4>(ctx->zhi), as<float4>(ctx->zlo), st);
+    node_data(t, as<double>(ctx->zc), as<double>(ctx->r), as<double>(ctx->hs), as<double>(ctx->geo),
+              as<float4>(ctx->zhi), as<float4>(ctx->zlo), as<int2>(ctx->kids), st);
     CK(rec(1));
     // ---- upward pass
     upward_pass(t, ctx->h_level_start, p, as<double>(ctx->xs), as<double>(ctx->ys), as<double>(ctx->zs),
-                as<double>(ctx->ms), as<double>(ctx->zc), as<double>(ctx->r), as<double>(ctx->hs),
-                as<double>(ctx->geo), as<double>(ctx->mult), as<double>(ctx->Pk), as<float>(ctx->Phat), as<float>(ctx->r32), as<double>(ctx->contrib), ctx->tb,
+                as<double>(ctx->ms), as<double>(ctx->zc), as<double>(ctx->hs), as<double>(ctx->geo),
+                as<double>(ctx->mult), as<double>(ctx->Pk), as<float>(ctx->Phat), as<double>(ctx->contrib), ctx->tb,
                 mixed, st);
     CK(rec(2));
     // ---- scalar-force estimate
@@ -1042,7 +1041,7 @@ void fmm_destroy(fmm_ctx* ctx) {
                   &ctx->f, &ctx->bbox, &ctx->level, &ctx->begin, &ctx->end, &ctx->parent,
                   &ctx->first_child, &ctx->nchild, &ctx->M, &ctx->S, &ctx->zc, &ctx->r, &ctx->hs, &ctx->Pk,
                   &ctx->mult, &ctx->mult32, &ctx->loc, &ctx->loc32, &ctx->fmin, &ctx->fscratch,
-                  &ctx->front0, &ctx->front1, &ctx->walk_scan, &ctx->dcount, &ctx->zhi, &ctx->zlo, &ctx->contrib, &ctx->Phat, &ctx->r32,
+                  &ctx->front0, &ctx->front1, &ctx->walk_scan, &ctx->dcount, &ctx->zhi, &ctx->zlo, &ctx->contrib, &ctx->Phat, &ctx->kids,
                   &ctx->item_first, &ctx->slot_first, &ctx->item_leaf, &ctx->leaf_of, &ctx->part_hi,
                   &ctx->part_lo, &ctx->work, &ctx->coff, &ctx->box, &ctx->ck0, &ctx->ck1, &ctx->cv0,
                   &ctx->cv1, &ctx->cid, &ctx->jv, &ctx->jv32, &ctx->jw, &ctx->jmom, &ctx->jmult,

@@ -295,7 +295,7 @@ void launch_p2m_dw(const TreeView& t, int p, const double* xs, const double* ys,
 }
 
 // P_n = s^n sqrt(sum_{m=-n}^{n} |Mhat_n^m|^2)  (Sec. 2.3)
-// (also the FP32 copies used by the walk's screen: Phat_n = P_n / s^n and r)
+// (also the FP32 copies used by the walk's screen: Phat_n = P_n / s^n)
 // LANES threads per node, thread j the degrees n = j, j + LANES, ..: each
 // degree's sum and power of s keep their order. Four for small trees, where a
 // node's chain of operations bounds the launch (N = 4096: 28 us with one,
@@ -304,9 +304,7 @@ void launch_p2m_dw(const TreeView& t, int p, const double* xs, const double* ys,
 constexpr int kPnormCells = 16384;
 template <int LANES>
 __global__ void k_pnorm(const int* __restrict__ dnn, int p, const double* __restrict__ mult,
-                        const double* __restrict__ rr, const double* __restrict__ hs,
-                        double* __restrict__ Pk, float* __restrict__ Phat,
-                        float* __restrict__ r32) {
+                        const double* __restrict__ hs, double* __restrict__ Pk, float* __restrict__ Phat) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     const int k = g / LANES, j = g % LANES;
     if (k >= *dnn) return;
@@ -319,11 +317,10 @@ __global__ void k_pnorm(const int* __restrict__ dnn, int p, const double* __rest
         for (int m = 1; m <= n; ++m) acc += 2.0 * (M[hre(n, m)] * M[hre(n, m)] + M[him(n, m)] * M[him(n, m)]);
         const double nrm = sqrt(acc);
         Pk[(size_t)(p + 1) * k + n] = sp * nrm;
-        Phat[(size_t)(p + 1) * k + n] = (float)nrm;
+        Phat[(size_t)phat_stride(p) * k + n] = (float)nrm;
 #pragma unroll
         for (int i = 0; i < LANES; ++i) sp *= s;
     }
-    if (j == 0) r32[k] = (float)rr[k];
 }
 
 __global__ void k_to_f32(const double* __restrict__ a, float* __restrict__ b, const int* __restrict__ dnn, int nr) {
@@ -376,30 +373,6 @@ __global__ void k_l2l(TreeView t, int L, int p, Tab tb, const double* __restrict
         out[hre(n, m)] += sig[n] * are;
         if (m) out[him(n, m)] += sig[n] * aim;
     }
-}
-
-__global__ void k_hat_scales(const int* __restrict__ dnn, const int* __restrict__ parent,
-                             const double* __restrict__ r, double* __restrict__ hs) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= *dnn) return;
-    int root = k;
-    while (parent[root] >= 0) root = parent[root];
-    const double floor_s = kHatFloor * (r[root] > 0.0 ? r[root] : 1.0);
-    hs[k] = r[k] > floor_s ? r[k] : floor_s;
-}
-
-__global__ void k_node_centres(const int* __restrict__ dnn, const double* __restrict__ zc, const double* __restrict__ hs,
-                               float4* __restrict__ zhi, float4* __restrict__ zlo) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= *dnn) return;
-    float h[3], l[3];
-    for (int d = 0; d < 3; ++d) {
-        const double z = zc[3 * k + d];
-        h[d] = (float)z;
-        l[d] = (float)(z - (double)h[d]);
-    }
-    zhi[k] = make_float4(h[0], h[1], h[2], (float)hs[k]);
-    zlo[k] = make_float4(l[0], l[1], l[2], 0.0f);
 }
 
 inline int blocks_for(int64_t n, int threads) { return (int)((n + threads - 1) / threads); }
@@ -491,8 +464,8 @@ void upload_expansion_tables(const HostTables& h) {
 
 void upward_pass(const TreeView& t, const int* h_level_start, int p, const double* xs,
                  const double* ys, const double* zs, const double* ms, const double* zc,
-                 const double* r, const double* hs, const double* geo, double* mult, double* Pk, float* Phat,
-                 float* r32, double* contrib, const DevTables& tbl, bool dword, cudaStream_t st) {
+                 const double* hs, const double* geo, double* mult, double* Pk, float* Phat, double* contrib,
+                 const DevTables& tbl, bool dword, cudaStream_t st) {
     const TabF64 tb = tab64(tbl);
     if (dword && p <= 16)
         launch_p2m_dw<16, 4>(t, p, xs, ys, zs, ms, zc, hs, mult, st);
@@ -507,10 +480,10 @@ void upward_pass(const TreeView& t, const int* h_level_start, int p, const doubl
     (void)h_level_start;
     for (int L = t.nlevels - 2; L >= 0; --L) m2m_level(t, L, p, geo, mult, contrib, tbl, dword, st);
     if (t.nnodes < kPnormCells)
-        (k_pnorm<4><<<blocks_for(4 * (int64_t)t.nnodes, 128), 128, 0, st>>>(t.dnn, p, mult, r, hs, Pk, Phat, r32),
+        (k_pnorm<4><<<blocks_for(4 * (int64_t)t.nnodes, 128), 128, 0, st>>>(t.dnn, p, mult, hs, Pk, Phat),
          note_launch());
     else
-        (k_pnorm<1><<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t.dnn, p, mult, r, hs, Pk, Phat, r32), note_launch());
+        (k_pnorm<1><<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t.dnn, p, mult, hs, Pk, Phat), note_launch());
 }
 
 void p2m_weights(const TreeView& t, int p, const double* xs, const double* ys, const double* zs, const double* w,
@@ -529,15 +502,6 @@ void p2m_weights(const TreeView& t, int p, const double* xs, const double* ys, c
 void dipole_moments(const TreeView& t, int p, const double* X, const double* Y, const double* Z, const double* hs,
                     double* mult, cudaStream_t st) {
     (k_dipole_moments<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t, p, X, Y, Z, hs, mult), note_launch());
-}
-
-void hat_scales(const TreeView& t, const int* parent, const double* r, double* hs, cudaStream_t st) {
-    (k_hat_scales<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t.dnn, parent, r, hs), note_launch());
-}
-
-void node_centres_f32(const TreeView& t, const double* zc, const double* hs, float4* zhi, float4* zlo,
-                      cudaStream_t st) {
-    (k_node_centres<<<blocks_for(t.nnodes, 128), 128, 0, st>>>(t.dnn, zc, hs, zhi, zlo), note_launch());
 }
 
 __global__ void k_to_f32_strided(const double* __restrict__ a, float* __restrict__ b, const int* __restrict__ dnn,

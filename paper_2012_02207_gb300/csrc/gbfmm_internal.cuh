@@ -235,7 +235,9 @@ constexpr int kWalkThreads = 256;    // threads of a walk block
 constexpr int kWalkIPT = GBFMM_WALK_IPT;  // frontier pairs per thread
 constexpr int kWalkTile = kWalkThreads * kWalkIPT;  // frontier pairs per tile (one block)
 constexpr int kWalkScanWords = 3;    // per tile: one record per counter (next frontier, accepted, leaf)
-inline int64_t walk_scan_tiles(int64_t front_cap) { return front_cap / kWalkTile + 2; }
+constexpr int kWalkBlocksPerSM = 8;  // of the walk's grid
+// tiles of the largest frontier (smaller frontiers take smaller tiles, at most three rounds of a tile per SM)
+inline int64_t walk_scan_tiles(int64_t front_cap) { return front_cap / kWalkTile + 2 + 3 * device_sm_count(); }
 // Dual-tree walk from (root, root). mode 0: theta < 1 (lists far/near);
 // mode 1: the error-controlled MAC (lists m2l/p2p). Returns iterations or a
 // negative fmm_status. Counts land in ds->list_cnt.
@@ -243,7 +245,7 @@ constexpr int kWalkBadIndex = -100;  // dual_tree_walk: a frontier entry out of 
 // M: cell masses, soft: Plummer softening length (0: Newtonian MAC)
 int dual_tree_walk(int mode, const TreeView& t, const double* zc, const double* r, const double* P,
                    const float* fmin, int p, double eps, const double* binom_row, const float4* zhi,
-                   const float4* zlo, const float* r32, const float* Phat, const double* M, double soft,
+                   const float4* zlo, const int2* kids, const float* Phat, const double* M, double soft,
                    WalkBuffers& wb, DevScalars* ds, DevScalars* h_ds, int fixed_iters, cudaStream_t st);
 // a walk run for a planned nit steps must have an empty frontier after them
 // (else kErrCapacity)
@@ -278,14 +280,23 @@ void upload_expansion_tables(const HostTables& h);
 // size of its tree's root so that no cell (a single body has r = 0) gets a scale so small
 // that its FP32 local coefficients F s^n fall into the denormal range.
 constexpr double kHatFloor = 0x1p-40;
-void hat_scales(const TreeView& t, const int* parent, const double* r, double* hs, cudaStream_t st);
+// With it, per node: the geometry of the shift to its parent (kShiftGeo doubles:
+// cos phi, sin phi, cos theta, sin theta of b = z_C - z_P, |b| / s_P and s_C / s_P, read
+// by the M2M and L2L kernels), the double-float centre (zhi.w the FP32 hat scale,
+// zlo.w the FP32 size) and the children (first, count) for the walks and the FP32
+// kernels. FP64, one thread per node.
+constexpr int kShiftGeo = 6;
+void node_data(const TreeView& t, const double* zc, const double* r, double* hs, double* geo, float4* zhi,
+               float4* zlo, int2* kids, cudaStream_t st);
+// floats per cell of the FP32 degree norms (a multiple of four, for float4 loads)
+__host__ __device__ constexpr int phat_stride(int p) { return (p + 4) & ~3; }
 // Hat multipoles in FP64: P2M at leaves, M2M level by level; P_k per node.
 // dword: the P2M and M2M arithmetic runs in double-word FP32 (mixed precision).
-// r: node sizes (the walk's FP32 copy r32 is written from them); hs: hat scales.
+// hs: hat scales; Phat: phat_stride(p) floats per node.
 void upward_pass(const TreeView& t, const int* h_level_start, int p, const double* xs,
                  const double* ys, const double* zs, const double* ms, const double* zc,
-                 const double* r, const double* hs, const double* geo, double* mult, double* Pk, float* Phat,
-                 float* r32, double* contrib, const DevTables& tb, bool dword, cudaStream_t st);
+                 const double* hs, const double* geo, double* mult, double* Pk, float* Phat, double* contrib,
+                 const DevTables& tb, bool dword, cudaStream_t st);
 // hat P2M of the leaves with per-body weights w (in place of masses); dword:
 // double-word FP32 arithmetic (mixed precision) instead of FP64
 void p2m_weights(const TreeView& t, int p, const double* xs, const double* ys, const double* zs, const double* w,
@@ -294,11 +305,6 @@ void p2m_weights(const TreeView& t, int p, const double* xs, const double* ys, c
 // p - 1 hat moments X, Y, Z of their x, y, z components (the jerk's chi field)
 void dipole_moments(const TreeView& t, int p, const double* X, const double* Y, const double* Z, const double* hs,
                     double* mult, cudaStream_t st);
-// The geometry of every node's shift to its parent, kShiftGeo doubles per
-// node: cos phi, sin phi, cos theta, sin theta of b = z_C - z_P, |b| / s_P and
-// s_C / s_P (FP64, one thread per node); read by the M2M and L2L kernels.
-constexpr int kShiftGeo = 6;
-void shift_geometry(const TreeView& t, const double* zc, const double* hs, double* geo, cudaStream_t st);
 // rotation-accelerated M2M of one level: the children (level L + 1) into their
 // parents (level L); contrib: (p+1)^2 doubles per node (scratch); dword:
 // double-word FP32 arithmetic instead of FP64
@@ -312,9 +318,6 @@ void multipoles_to_f32(const double* mult, float* mult32, const TreeView& t, int
 // FP32 copy with each node's vector padded to `stride` floats (zeros after nr)
 void multipoles_to_f32_padded(const double* mult, float* mult32, const TreeView& t, int nr, int stride,
                               cudaStream_t st);
-// double-float node centres (hi, lo) and the FP32 hat scale in zhi.w
-void node_centres_f32(const TreeView& t, const double* zc, const double* hs, float4* zhi, float4* zlo,
-                      cudaStream_t st);
 // per-node minimum of the scalar-force estimate (leaves over bodies, then levels upward)
 
 // L2L level by level (FP64 or FP32 locals).

@@ -188,30 +188,47 @@ __device__ __forceinline__ void m2m_zshift_unit(int p, int u, int& n, int& ma, b
 // shared values per warp: vector, scratch, two power tables, u^k and (s_C/s_P)^k
 __host__ __device__ inline int m2m_warp_values(int p) { return 2 * ncoef_real(p) + 6 * (p + 1); }
 
-// The geometry of the shift from node C's centre to its parent P's, one
-// thread per node: with b = z_C - z_P, the angles of b (cos and sin of phi
-// and theta), u = |b| / s_P and s_C / s_P. The warps of the M2M and L2L
-// kernels read these instead of each evaluating the FP64 square roots and
-// divisions on all of their lanes (a warp's FP64 instruction occupies the
-// FP64 pipe about as long whether one lane or 32 need the value).
-__global__ void k_shift_geometry(TreeView t, const double* __restrict__ zc, const double* __restrict__ hs,
-                                 double* __restrict__ geo) {
+// Per-node data, one thread per node: the hat scale; the geometry of the
+// shift from node C's centre to its parent P's (with b = z_C - z_P, the angles of b
+// (cos and sin of phi and theta), u = |b| / s_P and s_C / s_P); the double-float
+// centre with the FP32 scale and size; the children. The warps of the M2M and
+// L2L kernels read the geometry instead of each evaluating the FP64 square roots
+// and divisions on all of their lanes (a warp's FP64 instruction occupies the FP64
+// pipe about as long whether one lane or 32 need the value).
+__global__ void k_node_data(TreeView t, const double* __restrict__ zc, const double* __restrict__ r,
+                            double* __restrict__ hs, double* __restrict__ geo, float4* __restrict__ zhi,
+                            float4* __restrict__ zlo, int2* __restrict__ kids) {
     const int C = blockIdx.x * blockDim.x + threadIdx.x;
     if (C >= *t.dnn) return;
     const int P = t.parent[C];
+    int root = C;
+    for (int a = P; a >= 0; a = t.parent[a]) root = a;
+    const double floor_s = kHatFloor * (r[root] > 0.0 ? r[root] : 1.0);
+    const double rC = r[C], sC = rC > floor_s ? rC : floor_s;
+    hs[C] = sC;
+    const double z[3] = {zc[3 * C], zc[3 * C + 1], zc[3 * C + 2]};
+    float h[3], l[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        h[d] = (float)z[d];
+        l[d] = (float)(z[d] - (double)h[d]);
+    }
+    zhi[C] = make_float4(h[0], h[1], h[2], (float)sC);
+    zlo[C] = make_float4(l[0], l[1], l[2], (float)rC);
+    kids[C] = make_int2(t.first_child[C], t.nchild[C]);
     if (P < 0) return;  // a root shifts nowhere
-    const double bx = zc[3 * C] - zc[3 * P], by = zc[3 * C + 1] - zc[3 * P + 1], bz = zc[3 * C + 2] - zc[3 * P + 2];
+    const double bx = z[0] - zc[3 * P], by = z[1] - zc[3 * P + 1], bz = z[2] - zc[3 * P + 2];
     const double rxy2 = bx * bx + by * by;
     const double rho = sqrt(rxy2 + bz * bz);
     const double rxy = sqrt(rxy2);
     double cp = 1.0, sp = 0.0, ct = 1.0, st = 0.0;
     if (rxy > 0.0) { cp = bx / rxy; sp = by / rxy; }
     if (rho > 0.0) { ct = bz / rho; st = rxy / rho; }
-    const double sP = hs[P];
+    const double sP = r[P] > floor_s ? r[P] : floor_s;
     double* g = geo + kShiftGeo * (size_t)C;
     g[0] = cp; g[1] = sp; g[2] = ct; g[3] = st;
     g[4] = rho / sP;
-    g[5] = hs[C] / sP;
+    g[5] = sC / sP;
 }
 
 template <typename T, int G>
@@ -235,7 +252,7 @@ __global__ void __launch_bounds__(128) k_m2m_rot(TreeView t, int Lc, int p,
     const double* src = mult + (size_t)nr * C;
     for (int q = lane; q < nr; q += G) wv.v[q] = ar_from<T>(src[q]);
     (void)P;
-    const double* gc = geo + kShiftGeo * (size_t)C;  // the shift's geometry (k_shift_geometry)
+    const double* gc = geo + kShiftGeo * (size_t)C;  // the shift's geometry (k_node_data)
     const double cp = gc[0], sp = gc[1], ct = gc[2], st = gc[3], u = gc[4], sg = gc[5];
     wpowers<G, T>(pwa, p, ar_from<T>(sp), ar_from<T>(cp), lane);
     wpowers<G, T>(pwb, p, ar_from<T>(ct), ar_from<T>(-st), lane);
@@ -312,7 +329,7 @@ __global__ void __launch_bounds__(128) k_l2l_rot(TreeView t, int L, int p,
     const int P = t.parent[C];
     const T* src = loc + (size_t)nr * P;
     for (int q = lane; q < nr; q += G) wv.v[q] = src[q];
-    const double* gc = geo + kShiftGeo * (size_t)C;  // the shift's geometry (k_shift_geometry)
+    const double* gc = geo + kShiftGeo * (size_t)C;  // the shift's geometry (k_node_data)
     const double cp = gc[0], sp = gc[1], ct = gc[2], st = gc[3], u = gc[4], sg = gc[5];
     wpowers<G, T>(pwa, p, ar_from<T>(sp), ar_from<T>(cp), lane);
     wpowers<G, T>(pwb, p, ar_from<T>(ct), ar_from<T>(-st), lane);
@@ -397,9 +414,10 @@ void launch_l2l(const TreeView& t, int L, int p, const double* geo, T* loc,
 
 }  // namespace
 
-void shift_geometry(const TreeView& t, const double* zc, const double* hs, double* geo, cudaStream_t st) {
+void node_data(const TreeView& t, const double* zc, const double* r, double* hs, double* geo, float4* zhi,
+               float4* zlo, int2* kids, cudaStream_t st) {
     if (t.nnodes > 0)
-        (k_shift_geometry<<<(t.nnodes + 127) / 128, 128, 0, st>>>(t, zc, hs, geo), note_launch());
+        (k_node_data<<<(t.nnodes + 127) / 128, 128, 0, st>>>(t, zc, r, hs, geo, zhi, zlo, kids), note_launch());
 }
 
 void l2l_level(const TreeView& t, int L, int p, const double* geo, void* loc, const DevTables& tb, bool fp32,
