@@ -24,7 +24,8 @@ NO_FMA = {"tree.cu", "walk.cu", "noalloc.cu", "timestep.cu", "hold.cu"}
 # FP32 kernels flush denormals: the hat scale floor keeps every coefficient
 # that matters far above the denormal range
 FTZ = {"p2p.cu", "m2l.cu"}
-M2L32_ORDERS = [4, 6, 8, 10, 12, 14]  # orders of the FP32 register M2L kernel
+M2L32_ORDERS = [4, 6, 8]  # orders of the FP32 M2L in straight-line steps
+M2L32_DEGREE_ORDERS = [10, 12, 14]  # and by degrees
 EXTRA_FLAGS = os.environ.get("GBFMM_NVCC_FLAGS", "").split()  # extra nvcc flags for experiments
 SOURCES = ["api.cu", "sort.cu", "tree.cu", "walk.cu", "expansions.cu", "m2l.cu", "m2l64.cu", "translate.cu", "p2p.cu", "noalloc.cu",
            "timestep.cu", "hold.cu", "peaks.cu"]
@@ -63,6 +64,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.run([sys.executable, os.path.join(CSRC, "gen_m2l.py")] + [str(p) for p in M2L32_ORDERS],
                        stdout=fh, check=True)
     os.replace(m2l_gen + ".tmp", m2l_gen)
+    m2l_steps = os.path.join(GEN, "m2l_steps.inc")
+    with open(m2l_steps + ".tmp", "w") as fh:
+        subprocess.run([sys.executable, os.path.join(CSRC, "gen_m2l_steps.py")] + [str(p) for p in M2L32_DEGREE_ORDERS],
+                       stdout=fh, check=True)
+    os.replace(m2l_steps + ".tmp", m2l_steps)
     common = ARCH + EXTRA_FLAGS + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
                      "-I", os.path.join(ROOT, "include"), "-I", GEN, "-I", CSRC]
     if verbose:
