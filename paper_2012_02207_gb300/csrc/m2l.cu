@@ -44,6 +44,32 @@ __device__ __forceinline__ PairGeo pair_geo(float4 ah, float4 al, float4 bh, flo
     return PairGeo{sp, cp, ct, st, sa * irho, sb * irho, irho};
 }
 
+// The sums over the lanes, acc[NV][32] -> out[NR] (locals keep the unpadded
+// stride). A lane takes the values j = lane, lane + 32, .. and adds the 32 lanes'
+// parts in the order of a butterfly, a binary tree over the bits of the lane's
+// number; the tree is the same from any lane, so each starts at another one and
+// the reads meet no bank conflicts. 260 instructions for 121 values, against 1,450
+// with a butterfly of shuffles per value: M2L at 1M bodies 6.84 -> 6.49 ms, 64 clusters at
+// P = 12 (six batches per target) 7.69 -> 7.12 ms.
+template <int P>
+__device__ __forceinline__ void store_local(const float4* acc, float* __restrict__ out) {
+    constexpr int NR = (P + 1) * (P + 1);
+    const int lane = threadIdx.x & 31;
+    const float* a = reinterpret_cast<const float*>(acc);
+#pragma unroll 1
+    for (int j = lane; j < NR; j += 32) {
+        const int at = (j >> 2) * 128 + (j & 3), c = (j >> 2) & 7;
+        float v[16];
+#pragma unroll
+        for (int l = 0; l < 16; ++l) v[l] = __fadd_rn(a[at + 4 * (l ^ c)], a[at + 4 * ((l + 16) ^ c)]);
+#pragma unroll
+        for (int h = 8; h > 0; h >>= 1)
+#pragma unroll
+            for (int l = 0; l < h; ++l) v[l] = __fadd_rn(v[l], v[l + h]);
+        out[j] = v[0];
+    }
+}
+
 // ------------------------------------------------------------------------
 // FP32, compile-time order P: coefficients live in registers. For the orders to 8.
 
@@ -82,11 +108,12 @@ __global__ void __launch_bounds__(128, 2) k_m2l32(const int* __restrict__ dnn, c
     float4* acc = sh_acc4 + (size_t)wib * NV * 32;
     // targets are taken from a shared counter: their source counts differ by
     // orders of magnitude, and a fixed stride leaves SMs idle at the end
+    int next_b = 0;  // (lane 0: asked for at a target's end, not earlier: a target held back is one more at the very end)
+    if (lane == 0) next_b = (int)atomicAdd(queue, 1u);
+    const int nnodes = *dnn;
     for (;;) {
-        int b = 0;
-        if (lane == 0) b = (int)atomicAdd(queue, 1u);
-        b = __shfl_sync(0xffffffffu, b, 0);
-        if (b >= *dnn) break;
+        const int b = __shfl_sync(0xffffffffu, next_b, 0);
+        if (b >= nnodes) break;
 #pragma unroll
         for (int j = 0; j < NV; ++j) acc[j * 32 + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
         const uint32_t q0 = off[b], q1 = off[b + 1];
@@ -123,14 +150,8 @@ __global__ void __launch_bounds__(128, 2) k_m2l32(const int* __restrict__ dnn, c
             }
         }
         __syncwarp();
-        float* out = loc + (size_t)NR * b;  // locals keep the unpadded stride
-        const float* accf = reinterpret_cast<const float*>(acc);
-        for (int j = 0; j < NR; ++j) {
-            float v = accf[((j >> 2) * 32 + lane) * 4 + (j & 3)];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) out[j] = v;
-        }
+        if (lane == 0) next_b = (int)atomicAdd(queue, 1u);
+        store_local<P>(acc, loc + (size_t)NR * b);
         __syncwarp();
     }
 }
@@ -148,7 +169,7 @@ __global__ void __launch_bounds__(128, 2) k_m2l32(const int* __restrict__ dnn, c
 // spills, and the source's values are loaded a degree ahead of their use.
 // M2L kernel, straight-line -> by degrees, ms: P = 12, 2.3M bodies of 64 clusters
 // 12.5 -> 7.7, 8M bodies 75 -> 47; P = 10, 1M bodies 7.5 -> 6.8, 64k .61 -> .58;
-// P = 14, 500k 6.9 -> 4.4. Bound by issue (57 % of the slots at P = 10, 49 % at 12) with
+// P = 14, 500k 6.9 -> 4.4. Bound by issue (60 % of the slots at P = 10, 52 % at 12) with
 // eight warps per SM, which is what registers and the sums' shared memory hold; three
 // blocks (168 registers) leave the L1 too small for the sources' rows: 8.8 ms at 1M.
 #include "m2l_steps.inc"
@@ -276,8 +297,15 @@ __device__ __forceinline__ void degrees(bool first, SourceAt& s, float* val, con
         degrees<P, N - 1>(first, s, val, ar, ai, br, bi, mid, acc, irho, next, mult, stride, zhi, zlo);
 }
 
+// Warps per block and blocks per SM: eight warps, the registers' limit, where the
+// sums of eight fit in shared memory. At P = 14 they are 29 KB per warp, so blocks of
+// one, seven to an SM (500k bodies: 4.9 ms with one block of four, 4.0 with three of
+// two, 3.7 so).
+__host__ __device__ constexpr int degree_warps(int P) { return P > 12 ? 1 : 4; }
+__host__ __device__ constexpr int degree_blocks(int P) { return P > 12 ? 7 : 2; }
+
 template <int P>
-__global__ void __launch_bounds__(128, 2) k_m2l32_deg(const int* __restrict__ dnn, const uint32_t* __restrict__ src,
+__global__ void __launch_bounds__(32 * degree_warps(P), degree_blocks(P)) k_m2l32_deg(const int* __restrict__ dnn, const uint32_t* __restrict__ src,
                                                       const uint32_t* __restrict__ off, const float* __restrict__ mult,
                                                       int stride, const float4* __restrict__ zhi,
                                                       const float4* __restrict__ zlo, float* __restrict__ loc,
@@ -288,11 +316,12 @@ __global__ void __launch_bounds__(128, 2) k_m2l32_deg(const int* __restrict__ dn
     extern __shared__ float4 sh_acc4[];  // [warp][NV][32]
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     float4* acc = sh_acc4 + (size_t)wib * NV * 32 + lane;
+    int next_b = 0;  // (lane 0: asked for at a target's end, not earlier: a target held back is one more at the very end)
+    if (lane == 0) next_b = (int)atomicAdd(queue, 1u);
+    const int nnodes = *dnn;
     for (;;) {
-        int b = 0;
-        if (lane == 0) b = (int)atomicAdd(queue, 1u);
-        b = __shfl_sync(0xffffffffu, b, 0);
-        if (b >= *dnn) break;
+        const int b = __shfl_sync(0xffffffffu, next_b, 0);
+        if (b >= nnodes) break;
 #pragma unroll 4
         for (int j = 0; j < NV; ++j) acc[j * 32] = make_float4(0.f, 0.f, 0.f, 0.f);
         const uint32_t q0 = off[b], q1 = off[b + 1];
@@ -326,14 +355,8 @@ __global__ void __launch_bounds__(128, 2) k_m2l32_deg(const int* __restrict__ dn
             }
         }
         __syncwarp();
-        float* out = loc + (size_t)NR * b;  // locals keep the unpadded stride
-        const float* accf = reinterpret_cast<const float*>(acc - lane);
-        for (int j = 0; j < NR; ++j) {
-            float v = accf[((j >> 2) * 32 + lane) * 4 + (j & 3)];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) out[j] = v;
-        }
+        if (lane == 0) next_b = (int)atomicAdd(queue, 1u);
+        store_local<P>(acc - lane, loc + (size_t)NR * b);
         __syncwarp();
     }
 }
@@ -348,9 +371,10 @@ void launch_m2l32(const int* dnn, const uint32_t* src, const uint32_t* off, cons
         if constexpr (P >= 10) return k_m2l32_deg<P>;
         else return k_m2l32<P>;
     }();
-    const size_t sh = (size_t)4 * (((P + 1) * (P + 1) + 3) / 4) * 32 * sizeof(float4);
+    constexpr int warps = P >= 10 ? degree_warps(P) : 4, blocks = P >= 10 ? degree_blocks(P) : 2;
+    const size_t sh = (size_t)warps * (((P + 1) * (P + 1) + 3) / 4) * 32 * sizeof(float4);
     ensure_dyn_smem((const void*)kernel, (int)sh);
-    (kernel<<<device_sm_count() * 2, 128, sh, st>>>(dnn, src, off, mult, stride, zhi, zlo, loc, queue), note_launch());
+    (kernel<<<device_sm_count() * blocks, 32 * warps, sh, st>>>(dnn, src, off, mult, stride, zhi, zlo, loc, queue), note_launch());
 }
 }  // namespace
 
