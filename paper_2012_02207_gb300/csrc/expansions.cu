@@ -192,8 +192,12 @@ __global__ void __launch_bounds__(WARPS * 32) k_p2m(TreeView t, int p, TabF64 tb
 // positions relative to the leaf centre are formed in FP64, split into
 // double words, and every recurrence step and tile sum runs on the FP32
 // pipes in the same order as k_p2m. The result is stored in FP64; its
-// relative error is of order 1e-13 instead of 1e-16, far below what the
-// FP32 translations downstream add.
+// relative error is of order 1e-15 instead of 1e-16, far below what the
+// FP32 translations downstream add. Bound by issue (72 % of the slots). The sums over
+// the bodies took half the time with one lane to an entry, as a column has at most
+// 2(p+1) entries and the last ones few: columns of 16 entries or less give an entry
+// 2, 4 or 8 lanes. With dw_dot2 in the recurrences, P2M and M2M together: 8M bodies
+// at p = 12 20.2 -> 14.3 ms, 1M at 10 2.17 -> 1.62 ms, 4k at 8 .185 -> .164 ms.
 // Shared memory per warp: the tile of one chunk's harmonics, 2(p+1) rows of
 // 33 (one per body, padded), and the sums, p+1 columns of 2(p+1) entries.
 __host__ __device__ inline int p2m_dw_warp_values(int p) { return 2 * (p + 1) * 33 + (p + 1) * 2 * (p + 1); }
@@ -230,14 +234,14 @@ __global__ void __launch_bounds__(WARPS * 32) k_p2m_dw(TreeView t, int p,
             const int nact = t.end[k] - i0 < 32 ? t.end[k] - i0 : 32;
             const dw x = act ? dw_from((xs[i] - cx) * is) : zero, y = act ? dw_from((ys[i] - cy) * is) : zero,
                      z = act ? dw_from((zs[i] - cz) * is) : zero, w = act ? dw_from(ms[i]) : zero;
-            const dw r2 = dw_add(dw_add(dw_mul(x, x), dw_mul(y, y)), dw_mul(z, z));
+            const dw r2 = dw_add(dw_dot2(x, x, y, y), dw_mul(z, z));
             dw dre = w, dim = zero;  // w * Shat_m^m
             // one code path for every column m (a rolled loop keeps the code small)
 #pragma unroll 1
             for (int m = 0; m <= p; ++m) {
                 if (m > 0) {
-                    const dw tq = dw_sub(dw_mul(dre, x), dw_mul(dim, y));
-                    dim = dw_mul(dw_add(dw_mul(dre, y), dw_mul(dim, x)), c_dw_d[m]);
+                    const dw tq = dw_dot2(dre, x, dw_neg(dim), y);
+                    dim = dw_mul(dw_dot2(dre, y, dim, x), c_dw_d[m]);
                     dre = dw_mul(tq, c_dw_d[m]);
                 }
                 dw s1r = dre, s1i = dim, s2r = zero, s2i = zero;
@@ -250,19 +254,27 @@ __global__ void __launch_bounds__(WARPS * 32) k_p2m_dw(TreeView t, int p,
                         vr = dw_mul(sz, s1r);
                         vi = dw_mul(sz, s1i);
                     } else {
-                        const dw a = dw_mul(c_dw_a[n][m], z), b = dw_mul(c_dw_b[n][m], r2);
-                        vr = dw_sub(dw_mul(a, s1r), dw_mul(b, s2r));
-                        vi = dw_sub(dw_mul(a, s1i), dw_mul(b, s2i));
+                        const dw a = dw_mul(c_dw_a[n][m], z), b = dw_neg(dw_mul(c_dw_b[n][m], r2));
+                        vr = dw_dot2(a, s1r, b, s2r);
+                        vi = dw_dot2(a, s1i, b, s2i);
                     }
                     tile(2 * (n - m))[lane] = vr;
                     tile(2 * (n - m) + 1)[lane] = vi;
                     s2r = s1r; s2i = s1i; s1r = vr; s1i = vi;
                 }
                 __syncwarp();
-                for (int ent = lane; ent < 2 * (p - m + 1); ent += 32) {
-                    dw sacc = acc(m)[ent];
-                    for (int l = 0; l < nact; ++l) sacc = dw_add(sacc, tile(ent)[l]);
-                    acc(m)[ent] = sacc;
+                // the column's entries over the bodies: `parts` lanes to an entry where it is short
+                const int ents = 2 * (p - m + 1);
+                const int parts = ents > 16 ? 1 : ents > 8 ? 2 : ents > 4 ? 4 : 8;
+                const int width = 32 / parts, part = lane / width;
+                for (int e0 = 0; e0 < ents; e0 += width) {
+                    const int ent = e0 + lane % width;
+                    const dw* row = tile(ent < ents ? ent : 0);
+                    dw v = zero;
+                    for (int l = part; l < nact; l += parts) v = dw_add(v, row[l]);
+                    for (int o = 16; o >= width; o >>= 1)
+                        v = dw_add(v, dw_make(__shfl_down_sync(0xffffffffu, v.hi, o), __shfl_down_sync(0xffffffffu, v.lo, o)));
+                    if (part == 0 && ent < ents) acc(m)[ent] = dw_add(acc(m)[ent], v);
                 }
                 __syncwarp();
             }

@@ -32,6 +32,14 @@ __device__ __forceinline__ dw ar_add(dw a, dw b) { return dw_add(a, b); }
 __device__ __forceinline__ dw ar_sub(dw a, dw b) { return dw_sub(a, b); }
 __device__ __forceinline__ dw ar_mul(dw a, dw b) { return dw_mul(a, b); }
 __device__ __forceinline__ dw ar_neg(dw a) { return dw_neg(a); }
+// a b + c d and a b - c d
+template <typename T> __device__ __forceinline__ T ar_dot2(T a, T b, T c, T d) { return a * b + c * d; }
+template <> __device__ __forceinline__ dw ar_dot2<dw>(dw a, dw b, dw c, dw d) { return dw_dot2(a, b, c, d); }
+template <typename T> __device__ __forceinline__ T ar_det2(T a, T b, T c, T d) { return a * b - c * d; }
+template <> __device__ __forceinline__ dw ar_det2<dw>(dw a, dw b, dw c, dw d) { return dw_dot2(a, b, dw_neg(c), d); }
+// a + x y
+template <typename T> __device__ __forceinline__ T ar_add_mul(T a, T x, T y) { return a + x * y; }
+template <> __device__ __forceinline__ dw ar_add_mul<dw>(dw a, dw x, dw y) { return dw_add_mul(a, x, y); }
 template <typename T> __device__ __forceinline__ T ar_from(double x);
 template <> __device__ __forceinline__ double ar_from<double>(double x) { return x; }
 template <> __device__ __forceinline__ dw ar_from<dw>(double x) { return dw_from(x); }
@@ -48,30 +56,25 @@ struct RotTables;
 template <>
 struct RotTables<double> {
     const double *cosb, *sinb, *zsh;
-    __device__ double c(int i) const { return __ldg(cosb + i); }
-    __device__ double s(int i) const { return __ldg(sinb + i); }
+    static __device__ double at(const double* p) { return __ldg(p); }
     __device__ double z(int i) const { return __ldg(zsh + i); }
 };
 template <>
 struct RotTables<dw> {
     const float2 *cosb, *sinb, *zsh;
-    __device__ dw c(int i) const { const float2 v = __ldg(cosb + i); return dw{v.x, v.y}; }
-    __device__ dw s(int i) const { const float2 v = __ldg(sinb + i); return dw{v.x, v.y}; }
+    static __device__ dw at(const float2* p) { const float2 v = __ldg(p); return dw{v.x, v.y}; }
     __device__ dw z(int i) const { const float2 v = __ldg(zsh + i); return dw{v.x, v.y}; }
 };
 template <>
 struct RotTables<float> {
     const float2 *cosb, *sinb, *zsh;
-    __device__ float c(int i) const { return __ldg(cosb + i).x; }
-    __device__ float s(int i) const { return __ldg(sinb + i).x; }
+    static __device__ float at(const float2* p) { return __ldg(p).x; }
     __device__ float z(int i) const { return __ldg(zsh + i).x; }
 };
 
 // coefficient q of the real layout -> (n, m, imaginary part?)
 __device__ __forceinline__ void decode_q(int q, int& n, int& m, bool& im) {
-    n = (int)sqrtf((float)q + 0.5f);
-    while (n * n > q) --n;
-    while ((n + 1) * (n + 1) <= q) ++n;
+    n = (int)sqrtf((float)q + 0.5f);  // (the root is never within a rounding of a whole number)
     const int r = q - n * n;
     if (r == 0) { m = 0; im = false; }
     else { m = (r + 1) >> 1; im = (r & 1) == 0; }
@@ -98,11 +101,11 @@ __device__ void wpowers(T* pw, int p, T c, T s, int lane) {
         T pr = ar_from<T>(1.0), pi = ar_from<T>(0.0), br = c, bi = s;
         for (int e = lane; e > 0; e >>= 1) {
             if (e & 1) {
-                const T tq = ar_sub(ar_mul(pr, br), ar_mul(pi, bi));
-                pi = ar_add(ar_mul(pr, bi), ar_mul(pi, br));
+                const T tq = ar_det2(pr, br, pi, bi);
+                pi = ar_dot2(pr, bi, pi, br);
                 pr = tq;
             }
-            const T tb = ar_sub(ar_mul(br, br), ar_mul(bi, bi));
+            const T tb = ar_det2(br, br, bi, bi);
             const T tm = ar_mul(br, bi);
             bi = ar_add(tm, tm);
             br = tb;
@@ -118,33 +121,40 @@ template <int G, typename T>
 __device__ void wrotz(WarpVec<T>& w, int p, const T* pw, bool conj, int lane) {
     const int ncx = p * (p + 1) / 2;  // complex coefficients with m >= 1
     for (int q = lane; q < ncx; q += G) {
-        int n = (int)((sqrtf(8.0f * q + 1.0f) - 1.0f) * 0.5f);  // q = n(n-1)/2 + (m-1), n >= 1
-        while (n * (n + 1) / 2 <= q) ++n;
-        while ((n - 1) * n / 2 > q) --n;
+        const int n = (int)((sqrtf(8.0f * q + 1.0f) + 1.0f) * 0.5f);  // q = n(n-1)/2 + (m-1), n >= 1
         const int mm = q - (n - 1) * n / 2 + 1;
         const T re = w.v[hre(n, mm)], im = w.v[him(n, mm)];
         const T pr = pw[2 * mm], pi = conj ? ar_neg(pw[2 * mm + 1]) : pw[2 * mm + 1];
-        w.v[hre(n, mm)] = ar_sub(ar_mul(re, pr), ar_mul(im, pi));
-        w.v[him(n, mm)] = ar_add(ar_mul(re, pi), ar_mul(im, pr));
+        w.v[hre(n, mm)] = ar_det2(re, pr, im, pi);
+        w.v[him(n, mm)] = ar_dot2(re, pi, im, pr);
     }
     gsync<G>();
 }
 
-template <int G, typename T>
-__device__ void wswap(WarpVec<T>& w, int p, const RotTables<T>& tb, int lane) {
+// v <- swap v. Real and imaginary outputs, which read the cosine and the sine
+// block, run through one loop with their own starts, so a warp with both does
+// not take the two one after the other (that left 16 of 32 lanes active; now 22.
+// With dw_add_mul the largest level of 64 clusters, 24k cells at p = 12: 518 -> 160 us;
+// the FP32 L2L of 8M bodies 3.58 -> 2.47 ms). scale: degree n also times scale[n].
+template <int G, bool SCALE, typename T>
+__device__ void wswap(WarpVec<T>& w, int p, const RotTables<T>& tb, int lane, const T* scale = nullptr) {
     const int nr = ncoef_real(p);
     for (int q = lane; q < nr; q += G) {
         int n, mm;
         bool im;
         decode_q(q, n, mm, im);
+        // order j of the input: v[n^2 + 2j - 1] (real; v[n^2] for j = 0) or v[n^2 + 2j] (imaginary)
+        const auto* block = im ? tb.sinb : tb.cosb;
+        const int row = im ? sin_off(n) + (mm - 1) * n - 1 : cos_off(n) + mm * (n + 1);
+        int j = im ? 2 - ((mm + n + 1) & 1) : (mm + n) & 1;
+        const T* x = w.v + n * n - (im ? 0 : 1);
         T acc = ar_from<T>(0.0);
-        if (!im) {
-            const int a0 = cos_off(n) + mm * (n + 1);
-            for (int j = (mm + n) & 1; j <= n; j += 2) acc = ar_add(acc, ar_mul(tb.c(a0 + j), w.v[hre(n, j)]));
-        } else {
-            const int b0 = sin_off(n) + (mm - 1) * n;
-            for (int j = ((mm + n + 1) & 1) ? 1 : 2; j <= n; j += 2) acc = ar_add(acc, ar_mul(tb.s(b0 + j - 1), w.v[him(n, j)]));
+        if (j == 0) {
+            acc = ar_add_mul(acc, tb.at(block + row), x[1]);
+            j = 2;
         }
+        for (; j <= n; j += 2) acc = ar_add_mul(acc, tb.at(block + row + j), x[2 * j]);
+        if (SCALE) acc = ar_mul(acc, scale[n]);
         w.t[q] = acc;
     }
     gsync<G>();
@@ -161,11 +171,9 @@ __device__ void wswap(WarpVec<T>& w, int p, const RotTables<T>& tb, int lane) {
 // (absent when len_a = n + 1) the rest.
 __device__ __forceinline__ void m2m_zshift_unit(int p, int u, int& n, int& ma, bool& ia, int& mb, bool& ib,
                                                 int& len_a) {
-    n = p;
-    while (u > n) {  // degree n owns n + 1 units
-        u -= n + 1;
-        --n;
-    }
+    const int left = (p + 1) * (p + 2) / 2 - 1 - u;  // units from the other end: n(n+1)/2 below degree n
+    n = (int)((sqrtf(8.0f * left + 1.0f) - 1.0f) * 0.5f);
+    u = n - (left - n * (n + 1) / 2);
     if (u == 0) {
         ma = mb = 0;
         ia = ib = false;
@@ -269,9 +277,9 @@ __global__ void __launch_bounds__(128) k_m2m_rot(TreeView t, int Lc, int p,
     }
     gsync<G>();
     wrotz<G>(wv, p, pwa, false, lane);  // Rz(pi/2 - phi)
-    wswap<G>(wv, p, tb, lane);
+    wswap<G, false>(wv, p, tb, lane);
     wrotz<G>(wv, p, pwb, false, lane);  // Rz(-theta)
-    wswap<G>(wv, p, tb, lane);
+    wswap<G, true>(wv, p, tb, lane, spow);  // (the source's degrees times (s_C/s_P)^n)
     // z-shift into the scratch vector, over balanced units (m2m_zshift_unit):
     // each output's terms in the same order as a plain loop over k
     const int nunits = (p + 1) * (p + 2) / 2;
@@ -282,24 +290,26 @@ __global__ void __launch_bounds__(128) k_m2m_rot(TreeView t, int Lc, int p,
         const int cza = zshift_offset(n, ma), czb = zshift_offset(n, mb);
         T acc_a = ar_from<T>(0.0), acc_b = ar_from<T>(0.0);
         for (int s = 0; s <= n; ++s) {
+            if (s == len_a) {  // on to output B
+                acc_a = acc_b;
+                acc_b = ar_from<T>(0.0);
+            }
             const bool in_a = s < len_a;
             const int k = in_a ? s : s - len_a;
             const int mm = in_a ? ma : mb;
             const bool im = in_a ? ia : ib;
-            const T term = ar_mul(ar_mul(tb.z((in_a ? cza : czb) + k), upow[k]),
-                                  ar_mul(spow[n - k], wv.v[im ? him(n - k, mm) : hre(n - k, mm)]));
-            const T sum = ar_add(in_a ? acc_a : acc_b, term);  // one add on every lane, no divergence
-            acc_a = in_a ? sum : acc_a;
-            acc_b = in_a ? acc_b : sum;
+            acc_b = ar_add_mul(acc_b, ar_mul(tb.z((in_a ? cza : czb) + k), upow[k]),
+                               wv.v[im ? him(n - k, mm) : hre(n - k, mm)]);
         }
+        if (len_a > n) acc_a = acc_b;
         wv.t[ia ? him(n, ma) : hre(n, ma)] = acc_a;
         if (len_a <= n) wv.t[ib ? him(n, mb) : hre(n, mb)] = acc_b;
     }
     gsync<G>();
     { T* tq = wv.v; wv.v = wv.t; wv.t = tq; }
-    wswap<G>(wv, p, tb, lane);
+    wswap<G, false>(wv, p, tb, lane);
     wrotz<G>(wv, p, pwb, true, lane);   // Rz(theta)
-    wswap<G>(wv, p, tb, lane);
+    wswap<G, false>(wv, p, tb, lane);
     wrotz<G>(wv, p, pwa, true, lane);   // Rz(phi - pi/2)
     double* dst = contrib + (size_t)nr * C;
     for (int q = lane; q < nr; q += G) dst[q] = ar_to(wv.v[q]);
@@ -345,9 +355,9 @@ __global__ void __launch_bounds__(128) k_l2l_rot(TreeView t, int L, int p,
     }
     gsync<G>();
     wrotz<G>(wv, p, pwa, false, lane);  // Rz(pi/2 - phi)
-    wswap<G>(wv, p, tb, lane);
+    wswap<G, false>(wv, p, tb, lane);
     wrotz<G>(wv, p, pwb, false, lane);  // Rz(-theta)
-    wswap<G>(wv, p, tb, lane);
+    wswap<G, false>(wv, p, tb, lane);
     for (int q = lane; q < nr; q += G) {
         int n, mm;
         bool im;
@@ -360,9 +370,9 @@ __global__ void __launch_bounds__(128) k_l2l_rot(TreeView t, int L, int p,
     }
     gsync<G>();
     { T* tq = wv.v; wv.v = wv.t; wv.t = tq; }
-    wswap<G>(wv, p, tb, lane);
+    wswap<G, false>(wv, p, tb, lane);
     wrotz<G>(wv, p, pwb, true, lane);   // Rz(theta)
-    wswap<G>(wv, p, tb, lane);
+    wswap<G, false>(wv, p, tb, lane);
     wrotz<G>(wv, p, pwa, true, lane);   // Rz(phi - pi/2)
     T* dst = loc + (size_t)nr * C;
     for (int q = lane; q < nr; q += G) dst[q] = ar_add(dst[q], wv.v[q]);
