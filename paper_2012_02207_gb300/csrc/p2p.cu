@@ -926,55 +926,90 @@ __global__ void k_jerk_inputs(int n, const uint32_t* __restrict__ perm, const do
 }
 
 // Near jerk over the same bounded work items as the P2P (a target leaf and
-// at most kLeavesPerItem of its source leaves, fetched dynamically): source
-// positions and velocities staged per warp in shared memory, G lanes per
-// target, runs of kRun terms folded into the accumulators (two-sum pairs in
-// FP32), one partial per (item, body) in part_hi = (jx, jy), part_lo.x = jz.
-// k_jerk_reduce adds a body's partials in item order.
-template <typename T, bool SOFT>
-__device__ __forceinline__ void jerk_pack(const Body4<T>* __restrict__ sm, const Body4<T>* __restrict__ su, int cnt,
-                                          int sub, int G, T tx, T ty, T tz, T tvx, T tvy, T tvz, T s2,
-                                          NearAcc<T>& acc) {
-    for (int k0 = sub; k0 < cnt; k0 += kRun * G) {
-        const int k1 = k0 + kRun * G < cnt ? k0 + kRun * G : cnt;
-        T px = T(0), py = T(0), pz = T(0);
-#pragma unroll 4
-        for (int k = k0; k < k1; k += G) {
-            const Body4<T> sv = sm[k], uv = su[k];
-            const T dx = sv.x - tx, dy = sv.y - ty, dz = sv.z - tz;
-            const T wx = uv.x - tvx, wy = uv.y - tvy, wz = uv.z - tvz;
-            const T r2 = dx * dx + dy * dy + dz * dz;
-            T rinv;
-            if constexpr (sizeof(T) == 4) rinv = rsqrtf(SOFT ? r2 + s2 : r2);
-            else rinv = inv_sqrt(SOFT ? r2 + s2 : r2);
-            if (!(r2 > T(0))) rinv = T(0);  // the body itself
-            const T ri2 = rinv * rinv;
-            const T mr3 = sv.w * rinv * ri2;
-            const T c = T(3) * (dx * wx + dy * wy + dz * wz) * ri2;
-            px += mr3 * (wx - c * dx);
-            py += mr3 * (wy - c * dy);
-            pz += mr3 * (wz - c * dz);
+// at most kLeavesPerItem of its source leaves, fetched dynamically): packs of
+// whole source leaves are staged per warp in shared memory, G lanes per target
+// take every G-th source, runs of kRun terms are folded into the accumulators
+// (two-sum pairs in FP32), one partial per (item, body) in part_hi = (jx, jy),
+// part_lo.x = jz. k_jerk_reduce adds a body's partials in item order.
+//
+// FP32: the terms of a lane are taken two at a time in packed operations (only the
+// sums, which are in source order, are scalar), 40 -> 27 instructions a term; the
+// stage keeps such a pair of sources side by side, so the operands need no
+// moves. The lanes read 32 source leaves' ranges and centres at once. 120,001
+// bodies, 1.5 G terms: 2.69 -> 2.15 ms (FMA pipe 48 -> 60 %; 26 of 32 lanes, as leaves of
+// 17 to 31 bodies leave some idle).
+constexpr int kJerkPairs = (kStageCap + 64) / 2;  // a pack, filled up to a multiple of 2 G
+
+struct JerkStage {
+    ulonglong2 xy[kJerkPairs], zw[kJerkPairs], uv[kJerkPairs];  // (x, y), (z, mass), (vx, vy) of two sources
+    f32x2 w[kJerkPairs];                                        // vz
+};
+
+// Source k goes to lane k % G as its term k / G; terms 2 i and 2 i + 1 of a lane make a pair.
+__device__ __forceinline__ void jerk_put(JerkStage& st, int k, int G, unsigned inv2g, float4 r, float4 v) {
+    const int j = (int)(((unsigned)k * inv2g) >> 20);  // k / (2 G), exact for k < 2^10, 2 G <= 64
+    const int in = k - 2 * G * j;
+    const int h = in >= G, pair = G * j + (h ? in - G : in);
+    float* xy = reinterpret_cast<float*>(&st.xy[pair]) + h;
+    float* zw = reinterpret_cast<float*>(&st.zw[pair]) + h;
+    float* uv = reinterpret_cast<float*>(&st.uv[pair]) + h;
+    xy[0] = r.x; xy[2] = r.y;
+    zw[0] = r.z; zw[2] = r.w;
+    uv[0] = v.x; uv[2] = v.y;
+    reinterpret_cast<float*>(&st.w[pair])[h] = v.z;
+}
+
+template <bool SOFT>
+__device__ __forceinline__ void jerk_pairs(const JerkStage& st, int npairs, int sub, int G, float4 t, float4 tv,
+                                           float s2, NearAcc<float>& acc) {
+    const f32x2 nx = f2_pack(-t.x, -t.x), ny = f2_pack(-t.y, -t.y), nz = f2_pack(-t.z, -t.z);
+    const f32x2 nu = f2_pack(-tv.x, -tv.x), nv = f2_pack(-tv.y, -tv.y), nw = f2_pack(-tv.z, -tv.z);
+    const f32x2 s22 = f2_pack(s2, s2), m3 = f2_pack(-3.0f, -3.0f);
+    for (int j0 = 0; j0 < npairs; j0 += kRun / 2) {
+        const int j1 = j0 + kRun / 2 < npairs ? j0 + kRun / 2 : npairs;
+        float px = 0.f, py = 0.f, pz = 0.f;
+#pragma unroll 2
+        for (int j = j0; j < j1; ++j) {
+            const int k = G * j + sub;
+            const ulonglong2 xy = st.xy[k], zw = st.zw[k], uv = st.uv[k];
+            const f32x2 dx = f2_add<true>(xy.x, nx), dy = f2_add<true>(xy.y, ny), dz = f2_add<true>(zw.x, nz);
+            const f32x2 wx = f2_add<true>(uv.x, nu), wy = f2_add<true>(uv.y, nv), wz = f2_add<true>(st.w[k], nw);
+            const f32x2 r2 = f2_fma<true>(dz, dz, f2_fma<true>(dx, dx, f2_mul<true>(dy, dy)));
+            float ra, rb, qa, qb;
+            f2_unpack(r2, ra, rb);
+            f2_unpack(SOFT ? f2_add<true>(r2, s22) : r2, qa, qb);
+            qa = rsqrtf(qa);
+            qb = rsqrtf(qb);
+            if (!(ra > 0.0f)) qa = 0.0f;  // the body itself
+            if (!(rb > 0.0f)) qb = 0.0f;
+            const f32x2 rinv = f2_pack(qa, qb), ri2 = f2_mul<true>(rinv, rinv);
+            const f32x2 mr3 = f2_mul<true>(f2_mul<true>(zw.y, rinv), ri2);
+            const f32x2 dot = f2_fma<true>(dz, wz, f2_fma<true>(dx, wx, f2_mul<true>(dy, wy)));
+            const f32x2 c = f2_mul<true>(f2_mul<true>(m3, dot), ri2);  // -3 (d . w) / r^2
+            float ma, mb, fa, fb;
+            f2_unpack(mr3, ma, mb);
+            f2_unpack(f2_fma<true>(c, dx, wx), fa, fb);
+            px = __fmaf_rn(mb, fb, __fmaf_rn(ma, fa, px));
+            f2_unpack(f2_fma<true>(c, dy, wy), fa, fb);
+            py = __fmaf_rn(mb, fb, __fmaf_rn(ma, fa, py));
+            f2_unpack(f2_fma<true>(c, dz, wz), fa, fb);
+            pz = __fmaf_rn(mb, fb, __fmaf_rn(ma, fa, pz));
         }
-        acc.add(px, py, pz, T(0));
+        acc.add(px, py, pz, 0.0f);
     }
 }
 
-template <typename T, bool SOFT>
-__global__ void __launch_bounds__(128) k_jerk_items(LeafArgs a, const double* __restrict__ vs,
-                                                     const float4* __restrict__ v32, const int* __restrict__ item_leaf,
-                                                     const uint32_t* __restrict__ item_first,
-                                                     const uint32_t* __restrict__ slot_first,
-                                                     const uint32_t* __restrict__ nitems_p,
-                                                     unsigned* __restrict__ work) {
-    constexpr int kCap = sizeof(T) == 8 ? kStageCap / 2 : kStageCap;  // 32 KB of staging per block
-    __shared__ Body4<T> stage[4][kCap];
-    __shared__ Body4<T> vstage[4][kCap];
+template <bool SOFT>
+__global__ void __launch_bounds__(128, 5) k_jerk_items_f32(LeafArgs a, const float4* __restrict__ v32,
+                                                        const int* __restrict__ item_leaf,
+                                                        const uint32_t* __restrict__ item_first,
+                                                        const uint32_t* __restrict__ slot_first,
+                                                        const uint32_t* __restrict__ nitems_p,
+                                                        unsigned* __restrict__ work) {
+    __shared__ JerkStage stages[4];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    Body4<T>* sm = stage[wib];
-    Body4<T>* su = vstage[wib];
+    JerkStage& st = stages[wib];
     const int nitems = (int)*nitems_p;
-    const size_t n = (size_t)a.t.n;
-    const T s2 = sizeof(T) == 4 ? (T)a.soft2f : (T)a.soft2;
     for (;;) {
         unsigned it = 0;
         if (lane == 0) it = atomicAdd(work, 1u);
@@ -989,21 +1024,170 @@ __global__ void __launch_bounds__(128) k_jerk_items(LeafArgs a, const double* __
         for (int tc = item.t0; tc < item.t1; tc += 32) {
             const int nt = item.t1 - tc < 32 ? item.t1 - tc : 32;
             const int G = 32 / nt;
+            const unsigned inv2g = ((1u << 20) + 2 * G - 1) / (2 * G);
             const int t = lane / G, sub = lane - t * G;
             const bool act = t < nt;
-            T tx = T(0), ty = T(0), tz = T(0), tvx = T(0), tvy = T(0), tvz = T(0);
+            float4 tp = make_float4(0.f, 0.f, 0.f, 0.f), tv = tp;
             if (act) {
-                const int ib = b0 + tc + t;
-                if constexpr (sizeof(T) == 4) {
-                    const float4 v = a.prel[ib], u = v32[ib];
-                    tx = v.x; ty = v.y; tz = v.z;
-                    tvx = u.x; tvy = u.y; tvz = u.z;
-                } else {
-                    tx = a.xs[ib]; ty = a.ys[ib]; tz = a.zs[ib];
-                    tvx = vs[ib]; tvy = vs[n + ib]; tvz = vs[2 * n + ib];
+                tp = a.prel[b0 + tc + t];
+                tv = v32[b0 + tc + t];
+            }
+            NearAcc<float> acc;
+            uint32_t q = q0;
+            int soff = 0;  // bodies of leaf q that went with the pack before
+            while (q < q1) {
+                __syncwarp();
+                int cnt = 0;
+                for (bool full = false; !full && q < q1;) {
+                    const int nl = q1 - q < 32u ? (int)(q1 - q) : 32;
+                    int a0 = 0, nA = 0;
+                    float ox = 0.f, oy = 0.f, oz = 0.f;
+                    if (lane < nl) {
+                        const int A = (int)a.p2p_src[q + lane];
+                        a0 = a.t.begin[A];
+                        nA = a.t.end[A] - a0;
+                        const float4 ah = a.zhi[A], al = a.zlo[A];
+                        ox = (ah.x - bh.x) + (al.x - bl.x);
+                        oy = (ah.y - bh.y) + (al.y - bl.y);
+                        oz = (ah.z - bh.z) + (al.z - bl.z);
+                    }
+                    if (lane == 0) {
+                        a0 += soff;
+                        nA -= soff;
+                    }
+                    int incl = nA;  // inclusive prefix sum of the sizes
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += v;
+                    }
+                    // leaves that fit whole; the first of an empty pack goes in pieces if it is too large
+                    int fit = __popc(__ballot_sync(0xffffffffu, lane < nl && cnt + incl <= kStageCap));
+                    const bool piece = cnt == 0 && fit == 0;
+                    if (piece) {
+                        if (lane == 0) nA = incl = kStageCap;
+                        fit = 1;
+                    }
+#pragma unroll 4
+                    for (int j = 0; j < fit; ++j) {
+                        const int aj = __shfl_sync(0xffffffffu, a0, j), nj = __shfl_sync(0xffffffffu, nA, j);
+                        const int dst = cnt + __shfl_sync(0xffffffffu, incl, j) - nj;
+                        const float oxj = __shfl_sync(0xffffffffu, ox, j), oyj = __shfl_sync(0xffffffffu, oy, j),
+                                    ozj = __shfl_sync(0xffffffffu, oz, j);
+                        for (int l = lane; l < nj; l += 32) {
+                            const float4 u = a.prel[aj + l];
+                            jerk_put(st, dst + l, G, inv2g, make_float4(u.x + oxj, u.y + oyj, u.z + ozj, u.w),
+                                     v32[aj + l]);
+                        }
+                    }
+                    if (piece) {
+                        cnt = kStageCap;
+                        soff += kStageCap;
+                        full = true;
+                    } else if (fit > 0) {
+                        cnt += __shfl_sync(0xffffffffu, incl, fit - 1);
+                        q += (uint32_t)fit;
+                        soff = 0;
+                    }
+                    if (fit < nl) full = true;
+                }
+                __syncwarp();
+                // fill up to whole pairs with massless copies of the first source
+                const int npairs = (cnt + 2 * G - 1) / (2 * G);
+                const float* f = reinterpret_cast<const float*>(&st.xy[0]);
+                const float4 r = make_float4(f[0], f[2], reinterpret_cast<const float*>(&st.zw[0])[0], 0.0f);
+                const float* g = reinterpret_cast<const float*>(&st.uv[0]);
+                const float4 v = make_float4(g[0], g[2], reinterpret_cast<const float*>(&st.w[0])[0], 0.0f);
+                for (int k = cnt + lane; k < 2 * G * npairs; k += 32) jerk_put(st, k, G, inv2g, r, v);
+                __syncwarp();
+                if (act) jerk_pairs<SOFT>(st, npairs, sub, G, tp, tv, a.soft2f, acc);
+            }
+            // combine the G sub-lanes of each target in sub-lane order
+            const int leader = t * G;
+            for (int s = 1; s < G; ++s) {
+                const int src = leader + s < 32 ? leader + s : 31;
+                const float vx = __shfl_sync(0xffffffffu, acc.hx, src), vy = __shfl_sync(0xffffffffu, acc.hy, src),
+                            vz = __shfl_sync(0xffffffffu, acc.hz, src);
+                const float wx = __shfl_sync(0xffffffffu, acc.lx, src), wy = __shfl_sync(0xffffffffu, acc.ly, src),
+                            wz = __shfl_sync(0xffffffffu, acc.lz, src);
+                if (sub == 0 && act) {
+                    two_sum(acc.hx, acc.lx, vx); acc.lx += wx;
+                    two_sum(acc.hy, acc.ly, vy); acc.ly += wy;
+                    two_sum(acc.hz, acc.lz, vz); acc.lz += wz;
                 }
             }
-            NearAcc<T> acc;
+            if (act && sub == 0) {
+                const uint32_t slot = slot0 + (uint32_t)(tc + t);
+                a.part_hi[slot] = make_double2((double)acc.hx + (double)acc.lx, (double)acc.hy + (double)acc.ly);
+                a.part_lo[slot] = make_double2((double)acc.hz + (double)acc.lz, 0.0);
+            }
+        }
+    }
+}
+
+template <bool SOFT>
+__device__ __forceinline__ void jerk_pack(const Body4<double>* __restrict__ sm, const Body4<double>* __restrict__ su,
+                                          int cnt, int sub, int G, double tx, double ty, double tz, double tvx,
+                                          double tvy, double tvz, double s2, NearAcc<double>& acc) {
+    for (int k0 = sub; k0 < cnt; k0 += kRun * G) {
+        const int k1 = k0 + kRun * G < cnt ? k0 + kRun * G : cnt;
+        double px = 0.0, py = 0.0, pz = 0.0;
+#pragma unroll 4
+        for (int k = k0; k < k1; k += G) {
+            const Body4<double> sv = sm[k], uv = su[k];
+            const double dx = sv.x - tx, dy = sv.y - ty, dz = sv.z - tz;
+            const double wx = uv.x - tvx, wy = uv.y - tvy, wz = uv.z - tvz;
+            const double r2 = dx * dx + dy * dy + dz * dz;
+            double rinv = inv_sqrt(SOFT ? r2 + s2 : r2);
+            if (!(r2 > 0.0)) rinv = 0.0;  // the body itself
+            const double ri2 = rinv * rinv;
+            const double mr3 = sv.w * rinv * ri2;
+            const double c = 3.0 * (dx * wx + dy * wy + dz * wz) * ri2;
+            px += mr3 * (wx - c * dx);
+            py += mr3 * (wy - c * dy);
+            pz += mr3 * (wz - c * dz);
+        }
+        acc.add(px, py, pz, 0.0);
+    }
+}
+
+template <bool SOFT>
+__global__ void __launch_bounds__(128) k_jerk_items_f64(LeafArgs a, const double* __restrict__ vs,
+                                                        const int* __restrict__ item_leaf,
+                                                        const uint32_t* __restrict__ item_first,
+                                                        const uint32_t* __restrict__ slot_first,
+                                                        const uint32_t* __restrict__ nitems_p,
+                                                        unsigned* __restrict__ work) {
+    constexpr int kCap = kStageCap / 2;  // 32 KB of staging per block
+    __shared__ Body4<double> stage[4][kCap];
+    __shared__ Body4<double> vstage[4][kCap];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    Body4<double>* sm = stage[wib];
+    Body4<double>* su = vstage[wib];
+    const int nitems = (int)*nitems_p;
+    const size_t n = (size_t)a.t.n;
+    for (;;) {
+        unsigned it = 0;
+        if (lane == 0) it = atomicAdd(work, 1u);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if ((int)it >= nitems) break;
+        const int B = item_leaf[it];
+        const int b0 = a.t.begin[B], nB = a.t.end[B] - b0;
+        const LeafItem item = leaf_item(a, it - item_first[B], a.p2p_off[B], a.p2p_off[B + 1], nB);
+        const uint32_t q0 = item.q0, q1 = item.q1;
+        const uint32_t slot0 = slot_first[B] + item.part * (uint32_t)nB;
+        for (int tc = item.t0; tc < item.t1; tc += 32) {
+            const int nt = item.t1 - tc < 32 ? item.t1 - tc : 32;
+            const int G = 32 / nt;
+            const int t = lane / G, sub = lane - t * G;
+            const bool act = t < nt;
+            double tx = 0.0, ty = 0.0, tz = 0.0, tvx = 0.0, tvy = 0.0, tvz = 0.0;
+            if (act) {
+                const int ib = b0 + tc + t;
+                tx = a.xs[ib]; ty = a.ys[ib]; tz = a.zs[ib];
+                tvx = vs[ib]; tvy = vs[n + ib]; tvz = vs[2 * n + ib];
+            }
+            NearAcc<double> acc;
             uint32_t q = q0;
             int soff = 0;
             while (q < q1) {
@@ -1018,23 +1202,10 @@ __global__ void __launch_bounds__(128) k_jerk_items(LeafArgs a, const double* __
                         if (cnt > 0) break;
                         take = kCap;
                     }
-                    float ox = 0.f, oy = 0.f, oz = 0.f;
-                    if constexpr (sizeof(T) == 4) {
-                        const float4 ah = a.zhi[A], al = a.zlo[A];
-                        ox = (ah.x - bh.x) + (al.x - bl.x);
-                        oy = (ah.y - bh.y) + (al.y - bl.y);
-                        oz = (ah.z - bh.z) + (al.z - bl.z);
-                    }
                     for (int l = lane; l < take; l += 32) {
                         const int jj = a0 + soff + l;
-                        if constexpr (sizeof(T) == 4) {
-                            const float4 u = a.prel[jj], w = v32[jj];
-                            sm[cnt + l] = {u.x + ox, u.y + oy, u.z + oz, u.w};
-                            su[cnt + l] = {w.x, w.y, w.z, 0.0f};
-                        } else {
-                            sm[cnt + l] = {a.xs[jj], a.ys[jj], a.zs[jj], a.ms[jj]};
-                            su[cnt + l] = {vs[jj], vs[n + jj], vs[2 * n + jj], 0.0};
-                        }
+                        sm[cnt + l] = {a.xs[jj], a.ys[jj], a.zs[jj], a.ms[jj]};
+                        su[cnt + l] = {vs[jj], vs[n + jj], vs[2 * n + jj], 0.0};
                     }
                     cnt += take;
                     if (take < rem) { soff += take; break; }
@@ -1042,37 +1213,20 @@ __global__ void __launch_bounds__(128) k_jerk_items(LeafArgs a, const double* __
                     ++q;
                 }
                 __syncwarp();
-                if (act) jerk_pack<T, SOFT>(sm, su, cnt, sub, G, tx, ty, tz, tvx, tvy, tvz, s2, acc);
+                if (act) jerk_pack<SOFT>(sm, su, cnt, sub, G, tx, ty, tz, tvx, tvy, tvz, a.soft2, acc);
             }
             // combine the G sub-lanes of each target in sub-lane order
             const int leader = t * G;
             for (int s = 1; s < G; ++s) {
                 const int src = leader + s < 32 ? leader + s : 31;
-                if constexpr (sizeof(T) == 4) {
-                    const float vx = __shfl_sync(0xffffffffu, acc.hx, src), vy = __shfl_sync(0xffffffffu, acc.hy, src),
-                                vz = __shfl_sync(0xffffffffu, acc.hz, src);
-                    const float wx = __shfl_sync(0xffffffffu, acc.lx, src), wy = __shfl_sync(0xffffffffu, acc.ly, src),
-                                wz = __shfl_sync(0xffffffffu, acc.lz, src);
-                    if (sub == 0 && act) {
-                        two_sum(acc.hx, acc.lx, vx); acc.lx += wx;
-                        two_sum(acc.hy, acc.ly, vy); acc.ly += wy;
-                        two_sum(acc.hz, acc.lz, vz); acc.lz += wz;
-                    }
-                } else {
-                    const double vx = __shfl_sync(0xffffffffu, acc.dx, src), vy = __shfl_sync(0xffffffffu, acc.dy, src),
-                                 vz = __shfl_sync(0xffffffffu, acc.dz, src);
-                    if (sub == 0 && act) { acc.dx += vx; acc.dy += vy; acc.dz += vz; }
-                }
+                const double vx = __shfl_sync(0xffffffffu, acc.dx, src), vy = __shfl_sync(0xffffffffu, acc.dy, src),
+                             vz = __shfl_sync(0xffffffffu, acc.dz, src);
+                if (sub == 0 && act) { acc.dx += vx; acc.dy += vy; acc.dz += vz; }
             }
             if (act && sub == 0) {
                 const uint32_t slot = slot0 + (uint32_t)(tc + t);
-                if constexpr (sizeof(T) == 4) {
-                    a.part_hi[slot] = make_double2((double)acc.hx + (double)acc.lx, (double)acc.hy + (double)acc.ly);
-                    a.part_lo[slot] = make_double2((double)acc.hz + (double)acc.lz, 0.0);
-                } else {
-                    a.part_hi[slot] = make_double2(acc.dx, acc.dy);
-                    a.part_lo[slot] = make_double2(acc.dz, 0.0);
-                }
+                a.part_hi[slot] = make_double2(acc.dx, acc.dy);
+                a.part_lo[slot] = make_double2(acc.dz, 0.0);
             }
         }
     }
@@ -1249,12 +1403,12 @@ void jerk_leaves(const LeafArgs& a, bool fp32, const void* locj, const double* v
     cudaMemsetAsync(work, 0, sizeof(unsigned), st);
     const bool soft = a.soft2 > 0.0;
     if (fp32) {
-        if (soft) (k_jerk_items<float, true><<<device_sm_count() * 16, 128, 0, st>>>(a, vs, v32, item_leaf, item_first, slot_first, nitems, work), note_launch());
-        else (k_jerk_items<float, false><<<device_sm_count() * 16, 128, 0, st>>>(a, vs, v32, item_leaf, item_first, slot_first, nitems, work), note_launch());
+        if (soft) (k_jerk_items_f32<true><<<device_sm_count() * 16, 128, 0, st>>>(a, v32, item_leaf, item_first, slot_first, nitems, work), note_launch());
+        else (k_jerk_items_f32<false><<<device_sm_count() * 16, 128, 0, st>>>(a, v32, item_leaf, item_first, slot_first, nitems, work), note_launch());
         (k_jerk_reduce<float><<<blocks_for(a.t.n, 128), 128, 0, st>>>(a, locj, vs, leaf_of, item_first, slot_first, jx, jy, jz), note_launch());
     } else {
-        if (soft) (k_jerk_items<double, true><<<device_sm_count() * 16, 128, 0, st>>>(a, vs, v32, item_leaf, item_first, slot_first, nitems, work), note_launch());
-        else (k_jerk_items<double, false><<<device_sm_count() * 16, 128, 0, st>>>(a, vs, v32, item_leaf, item_first, slot_first, nitems, work), note_launch());
+        if (soft) (k_jerk_items_f64<true><<<device_sm_count() * 16, 128, 0, st>>>(a, vs, item_leaf, item_first, slot_first, nitems, work), note_launch());
+        else (k_jerk_items_f64<false><<<device_sm_count() * 16, 128, 0, st>>>(a, vs, item_leaf, item_first, slot_first, nitems, work), note_launch());
         (k_jerk_reduce<double><<<blocks_for(a.t.n, 128), 128, 0, st>>>(a, locj, vs, leaf_of, item_first, slot_first, jx, jy, jz), note_launch());
     }
 }
