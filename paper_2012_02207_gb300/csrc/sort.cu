@@ -11,8 +11,8 @@
 // What bounds it: ranking and the scattered writes where there are many tiles;
 // the launch where there are few. With a histogram, its scan (one or three
 // launches) and a scatter per pass, the 8 passes over 4096 body keys took 200 us
-// of kernels, now 120; all sorts of 2^20 bodies (8 passes of bodies, 12 of list
-// keys) 1.67 ms, now 1.26.
+// of kernels, now 91; all sorts of 2^20 bodies (8 passes of bodies, 12 of list
+// keys) 1.67 ms, now 1.20.
 //
 // Waits are bounded (about a second): a block that gives up raises kErrTimeout
 // in the sort's error word and goes on with the prefix it has; its positions
@@ -23,20 +23,22 @@
 namespace gbfmm {
 
 namespace {
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
-constexpr int kItems = 16;                   // keys per thread
+constexpr int kItems = 8;                    // keys per thread
 constexpr int kTile = kThreads * kItems;     // 4096 keys per block
-constexpr int kWarpItems = kTile / kWarps;   // 512 contiguous keys per warp
+constexpr int kWarpItems = kTile / kWarps;   // 256 contiguous keys per warp
 constexpr int kMaxPasses = 8;
 template <typename K, bool VAL>
 constexpr size_t scatter_smem() {
     return (size_t)kTile * (sizeof(K) + (VAL ? 4 : 0)) + (size_t)(kWarps + 2) * 256 * 4;
 }
-// blocks per SM the pass kernel's registers are cut for: three for 32-bit keys
-// without payload (80 registers, no spills), two otherwise
-template <typename K, bool VAL>
-constexpr int scatter_min_blocks() { return (sizeof(K) == 4 && !VAL) ? 3 : 2; }
+// Blocks per SM the pass kernel's registers are cut for (40, a few spills for
+// 64-bit keys): a pass is a chain of waits (loads, ranks, look-back), so warps
+// in flight count. With 16 keys per thread of 256 and two blocks, 16 warps on an SM,
+// the 16 passes over the 64-bit list keys of 8M bodies took 8.4 ms, now 5.1 (16 keys a
+// thread in blocks of 512: faster there, .21 ms slower on its 8 passes over the bodies).
+constexpr int kPassBlocks = 3;
 
 // Scratch of a sort: digit counts of every pass, a tile ticket per pass (both
 // zeroed before the sort), then the look-back records, 256 per tile: bits 63-62
@@ -83,7 +85,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_count(const K* __restrict__ k
     for (int i = threadIdx.x; i < npass * 256; i += kThreads) h[i] = 0;
     __syncthreads();
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        s.rec[t * 256 + threadIdx.x] = 0ull;
+        if (threadIdx.x < 256) s.rec[t * 256 + threadIdx.x] = 0ull;
         K key[kItems];
 #pragma unroll
         for (int k = 0; k < kItems; ++k) {
@@ -122,7 +124,7 @@ __device__ __forceinline__ uint32_t warp_scan(uint32_t v, int lane) {
 }
 
 template <typename K, bool VAL>
-__global__ void __launch_bounds__(kThreads, scatter_min_blocks<K, VAL>()) k_sort_pass(
+__global__ void __launch_bounds__(kThreads, kPassBlocks) k_sort_pass(
     const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout, uint32_t* __restrict__ vout,
     int64_t n, const unsigned long long* __restrict__ dn, int shift, int pass, SortScratch s, unsigned* err) {
     extern __shared__ __align__(16) unsigned char sh_scatter[];
@@ -141,42 +143,46 @@ __global__ void __launch_bounds__(kThreads, scatter_min_blocks<K, VAL>()) k_sort
     const int64_t tile0 = tile * kTile;
     if (dn && (int64_t)*dn < n) n = (int64_t)*dn;
     if (tile0 >= n) return;  // the whole block: nothing of this tile is present
-    const int64_t base = tile0 + (int64_t)warp * kWarpItems;
+    const int present = (int)(n - tile0 < kTile ? n - tile0 : kTile);
+    const int mine = present - warp * kWarpItems - lane;  // item r of this thread is present if 32 r < mine
+    kin += tile0 + warp * kWarpItems + lane;
+    if (VAL) vin += tile0 + warp * kWarpItems + lane;
     K key[kItems];
-    uint32_t val[VAL ? kItems : 1], rank[kItems];
+    uint32_t val[VAL ? kItems : 1], rank[kItems / 2];  // (two 16-bit ranks to a word)
     // all loads first, so that they are in flight together
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
-        const int64_t i = base + r * 32 + lane;
-        key[r] = i < n ? kin[i] : K(0);
-        if (VAL) val[VAL ? r : 0] = i < n ? vin[i] : 0u;
+        key[r] = 32 * r < mine ? kin[32 * r] : K(0);
+        if (VAL) val[VAL ? r : 0] = 32 * r < mine ? vin[32 * r] : 0u;
     }
-    const uint32_t digits_all = s.digits[pass * 256 + threadIdx.x];  // kThreads == 256 digits
+    const uint32_t digits_all = threadIdx.x < 256 ? s.digits[pass * 256 + threadIdx.x] : 0u;
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
-        const int64_t i = base + r * 32 + lane;
-        const bool valid = i < n;
+        const bool valid = 32 * r < mine;
         const uint32_t d = valid ? (uint32_t)(key[r] >> shift) & 255u : 0xFFFFFFFFu;
         const unsigned peers = __match_any_sync(0xffffffffu, d);
         const uint32_t before = valid ? wcount[warp][d] : 0u;
-        rank[r] = before + __popc(peers & ((1u << lane) - 1u));
+        const uint32_t rk = before + __popc(peers & ((1u << lane) - 1u));
+        rank[r / 2] = r % 2 ? rank[r / 2] | rk << 16 : rk;
         __syncwarp();
         if (valid && lane == 31 - __clz(peers)) wcount[warp][d] = before + __popc(peers);
         __syncwarp();
     }
     __syncthreads();
-    // thread d: the tile's count of digit d, published at once
+    // thread d < 256: the tile's count of digit d, published at once
     const int d = threadIdx.x;
     unsigned long long* rec = s.rec + d;
     const unsigned long long tag = (unsigned long long)pass << 56;
-    uint32_t cnt = 0;
+    uint32_t cnt = 0, gbase = 0;
+    if (d < 256) {
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        const uint32_t t = wcount[w][d];
-        wcount[w][d] = cnt;
-        cnt += t;
+        for (int w = 0; w < kWarps; ++w) {
+            const uint32_t t = wcount[w][d];
+            wcount[w][d] = cnt;
+            cnt += t;
+        }
+        rec_store(rec + tile * 256, (tile == 0 ? kRecPrefix : kRecCount) | tag | cnt);
     }
-    rec_store(rec + tile * 256, (tile == 0 ? kRecPrefix : kRecCount) | tag | cnt);
     // exclusive scans over the digits: the tile's counts and all keys' counts
     const uint32_t in_tile = warp_scan(cnt, lane), in_all = warp_scan(digits_all, lane);
     if (lane == 31) {
@@ -184,27 +190,29 @@ __global__ void __launch_bounds__(kThreads, scatter_min_blocks<K, VAL>()) k_sort
         s_wsum[1][warp] = in_all;
     }
     __syncthreads();
-    uint32_t lbase = in_tile - cnt, gbase = in_all - digits_all;
-    for (int w = 0; w < warp; ++w) {
-        lbase += s_wsum[0][w];
-        gbase += s_wsum[1][w];
+    if (d < 256) {
+        uint32_t lbase = in_tile - cnt;
+        gbase = in_all - digits_all;
+        for (int w = 0; w < warp; ++w) {
+            lbase += s_wsum[0][w];
+            gbase += s_wsum[1][w];
+        }
+        lstart[d] = lbase;
     }
-    lstart[d] = lbase;
     __syncthreads();
     // reorder the tile by digit in shared memory
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
-        const int64_t i = base + r * 32 + lane;
-        if (i < n) {
+        if (32 * r < mine) {
             const uint32_t dd = (uint32_t)(key[r] >> shift) & 255u;
-            const uint32_t pos = lstart[dd] + wcount[warp][dd] + rank[r];
+            const uint32_t pos = lstart[dd] + wcount[warp][dd] + (rank[r / 2] >> 16 * (r % 2) & 0xffffu);
             skey[pos] = key[r];
             if (VAL) sval[pos] = val[VAL ? r : 0];
         }
     }
     // look-back for digit d: the keys of it in the tiles before this one
     uint32_t excl = 0;
-    if (tile > 0) {
+    if (tile > 0 && d < 256) {
         constexpr int kAhead = 4;
         const unsigned long long want = tag >> 56;
         unsigned long long t0 = 0;
@@ -233,9 +241,8 @@ __global__ void __launch_bounds__(kThreads, scatter_min_blocks<K, VAL>()) k_sort
         }
         rec_store(rec + tile * 256, kRecPrefix | tag | (excl + cnt));
     }
-    boff[d] = gbase + excl;
+    if (d < 256) boff[d] = gbase + excl;
     __syncthreads();
-    const int present = (int)((n - tile0) < kTile ? (n - tile0) : kTile);
     for (int j = threadIdx.x; j < present; j += kThreads) {
         const K k = skey[j];
         const uint32_t dd = (uint32_t)(k >> shift) & 255u;
