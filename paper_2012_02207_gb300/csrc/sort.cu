@@ -11,7 +11,7 @@
 // What bounds it: ranking and the scattered writes where there are many tiles;
 // the launch where there are few. With a histogram, its scan (one or three
 // launches) and a scatter per pass, the 8 passes over 4096 body keys took 200 us
-// of kernels, now 91; all sorts of 2^20 bodies (8 passes of bodies, 12 of list
+// of kernels, then 91, now 43 (k_sort_tile); all sorts of 2^20 bodies (8 passes of bodies, 12 of list
 // keys) 1.67 ms, now 1.20.
 //
 // Waits are bounded (about a second): a block that gives up raises kErrTimeout
@@ -123,6 +123,25 @@ __device__ __forceinline__ uint32_t warp_scan(uint32_t v, int lane) {
     return v;
 }
 
+// Rank of each of the thread's keys among the warp's earlier keys with the same
+// digit (two 16-bit ranks to a word); count (zero before): the warp's keys per digit.
+template <typename K>
+__device__ __forceinline__ void rank_items(const K* key, int mine, int shift, uint32_t* count, int lane,
+                                           uint32_t* rank) {
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        const bool valid = 32 * r < mine;
+        const uint32_t d = valid ? (uint32_t)(key[r] >> shift) & 255u : 0xFFFFFFFFu;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = valid ? count[d] : 0u;
+        const uint32_t rk = before + __popc(peers & ((1u << lane) - 1u));
+        rank[r / 2] = r % 2 ? rank[r / 2] | rk << 16 : rk;
+        __syncwarp();
+        if (valid && lane == 31 - __clz(peers)) count[d] = before + __popc(peers);
+        __syncwarp();
+    }
+}
+
 template <typename K, bool VAL>
 __global__ void __launch_bounds__(kThreads, kPassBlocks) k_sort_pass(
     const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout, uint32_t* __restrict__ vout,
@@ -156,18 +175,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_sort_pass(
         if (VAL) val[VAL ? r : 0] = 32 * r < mine ? vin[32 * r] : 0u;
     }
     const uint32_t digits_all = threadIdx.x < 256 ? s.digits[pass * 256 + threadIdx.x] : 0u;
-#pragma unroll
-    for (int r = 0; r < kItems; ++r) {
-        const bool valid = 32 * r < mine;
-        const uint32_t d = valid ? (uint32_t)(key[r] >> shift) & 255u : 0xFFFFFFFFu;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t before = valid ? wcount[warp][d] : 0u;
-        const uint32_t rk = before + __popc(peers & ((1u << lane) - 1u));
-        rank[r / 2] = r % 2 ? rank[r / 2] | rk << 16 : rk;
-        __syncwarp();
-        if (valid && lane == 31 - __clz(peers)) wcount[warp][d] = before + __popc(peers);
-        __syncwarp();
-    }
+    rank_items(key, mine, shift, wcount[warp], lane, rank);
     __syncthreads();
     // thread d < 256: the tile's count of digit d, published at once
     const int d = threadIdx.x;
@@ -250,6 +258,81 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_sort_pass(
         if ((int64_t)pos >= n) continue;  // (never: only a wait that ran out could misplace a key)
         kout[pos] = k;
         if (VAL) vout[pos] = sval[j];
+    }
+}
+
+// All passes of one tile in one block, for up to kTile keys, in place: a pass is
+// some 5 us of ranking and exchange in shared memory, where a launch of k_sort_pass
+// takes 10. 4096 body keys with the permutation: 91 -> 43 us.
+template <typename K, bool VAL>
+__global__ void __launch_bounds__(kThreads) k_sort_tile(K* __restrict__ keys, uint32_t* __restrict__ vals, int64_t n,
+                                                        const unsigned long long* __restrict__ dn, int lo_bit,
+                                                        int npass) {
+    extern __shared__ __align__(16) unsigned char sh_scatter[];
+    K* skey = reinterpret_cast<K*>(sh_scatter);
+    uint32_t* sval = reinterpret_cast<uint32_t*>(skey + kTile);
+    uint32_t (*wcount)[256] = reinterpret_cast<uint32_t (*)[256]>(sval + (VAL ? kTile : 0));
+    uint32_t* lstart = &wcount[kWarps][0];
+    __shared__ uint32_t s_wsum[kWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d = threadIdx.x;
+    if (dn && (int64_t)*dn < n) n = (int64_t)*dn;
+    const int first = warp * kWarpItems + lane;
+    const int mine = (int)n - first;  // item r of this thread is present if 32 r < mine
+    K key[kItems];
+    uint32_t val[VAL ? kItems : 1], rank[kItems / 2];
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        key[r] = 32 * r < mine ? keys[first + 32 * r] : K(0);
+        if (VAL) val[VAL ? r : 0] = 32 * r < mine ? vals[first + 32 * r] : 0u;
+    }
+    for (int pass = 0; pass < npass; ++pass) {
+        const int shift = lo_bit + 8 * pass;
+        for (int i = threadIdx.x; i < kWarps * 256; i += kThreads) (&wcount[0][0])[i] = 0;
+        __syncthreads();
+        rank_items(key, mine, shift, wcount[warp], lane, rank);
+        __syncthreads();
+        uint32_t cnt = 0;
+        if (d < 256) {
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const uint32_t t = wcount[w][d];
+                wcount[w][d] = cnt;
+                cnt += t;
+            }
+        }
+        const uint32_t in_tile = warp_scan(cnt, lane);
+        if (lane == 31) s_wsum[warp] = in_tile;
+        __syncthreads();
+        if (d < 256) {
+            uint32_t lbase = in_tile - cnt;
+            for (int w = 0; w < warp; ++w) lbase += s_wsum[w];
+            lstart[d] = lbase;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kItems; ++r) {
+            if (32 * r < mine) {
+                const uint32_t dd = (uint32_t)(key[r] >> shift) & 255u;
+                const uint32_t pos = lstart[dd] + wcount[warp][dd] + (rank[r / 2] >> 16 * (r % 2) & 0xffffu);
+                skey[pos] = key[r];
+                if (VAL) sval[pos] = val[VAL ? r : 0];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kItems; ++r) {
+            if (32 * r < mine) {
+                key[r] = skey[first + 32 * r];
+                if (VAL) val[VAL ? r : 0] = sval[first + 32 * r];
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        if (32 * r < mine) {
+            keys[first + 32 * r] = key[r];
+            if (VAL) vals[first + 32 * r] = val[VAL ? r : 0];
+        }
     }
 }
 
@@ -394,9 +477,14 @@ template <typename K, bool VAL>
 int radix_sort_impl(K* k0, uint32_t* v0, K* k1, uint32_t* v1, int64_t n, int lo_bit, int bits, uint32_t* hist,
                     cudaStream_t st, const unsigned long long* dn, unsigned* err) {
     if (n <= 1 || bits <= lo_bit) return 0;
+    const int npass = (bits - lo_bit + 7) / 8;
+    if (n <= kTile) {
+        ensure_dyn_smem((const void*)k_sort_tile<K, VAL>, (int)scatter_smem<K, VAL>());
+        (k_sort_tile<K, VAL><<<1, kThreads, scatter_smem<K, VAL>(), st>>>(k0, v0, n, dn, lo_bit, npass), note_launch());
+        return 0;
+    }
     ensure_dyn_smem((const void*)k_sort_pass<K, VAL>, (int)scatter_smem<K, VAL>());
     const int nblocks = (int)((n + kTile - 1) / kTile);
-    const int npass = (bits - lo_bit + 7) / 8;
     const SortScratch s(hist);
     cudaMemsetAsync(hist, 0, sizeof(uint32_t) * kSortHeadWords, st);
     const int count_grid = nblocks < 4 * device_sm_count() ? nblocks : 4 * device_sm_count();
