@@ -623,7 +623,7 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
         m2l_f32(t.dnn, p, mk, mo, as<float>(ctx->mult32), as<float4>(ctx->zhi), as<float4>(ctx->zlo),
                 as<float>(ctx->loc32), &ctx->ds->queue, st);
     } else {
-        m2l_f64(t.dnn, t.nnodes, p, mk, mo, as<double>(ctx->mult), as<double>(ctx->zc), as<double>(ctx->hs),
+        m2l_f64(t.dnn, p, mk, mo, as<double>(ctx->mult), as<double>(ctx->zc), as<double>(ctx->hs),
                 as<double>(ctx->loc), ctx->tb, &ctx->ds->queue, st);
         if (far32) multipoles_to_f32(as<double>(ctx->loc), as<float>(ctx->loc32), t, (int)nr, st);
     }
@@ -759,7 +759,7 @@ int jerk_pass(fmm_ctx* ctx, const double* vx, const double* vy, const double* vz
         m2l_f32(t.dnn, p, mk, mo, as<float>(ctx->jmult32), as<float4>(ctx->zhi), as<float4>(ctx->zlo),
                 as<float>(ctx->jloc32), &ctx->ds->queue, st);
     } else {
-        m2l_f64(t.dnn, t.nnodes, p, mk, mo, as<double>(ctx->jmult), zc, hs, as<double>(ctx->jloc), ctx->tb,
+        m2l_f64(t.dnn, p, mk, mo, as<double>(ctx->jmult), zc, hs, as<double>(ctx->jloc), ctx->tb,
                 &ctx->ds->queue, st);
         if (mixed) multipoles_to_f32(as<double>(ctx->jloc), as<float>(ctx->jloc32), t, (int)nr, st);
     }

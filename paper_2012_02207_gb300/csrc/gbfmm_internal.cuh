@@ -330,8 +330,7 @@ void downward_pass_f32(const TreeView& t, const int* h_level_start, int p, const
 // Rotation-accelerated M2L (Sec. 2.4), gathered per target over the sorted
 // directed list; writes the locals of every node (zero without sources).
 // queue: a device counter, zeroed here; warps take target cells (below *dnn) from it.
-// ncells: the cells of the grid (>= *dnn), which decides how the work is split.
-void m2l_f64(const int* dnn, int ncells, int p, const uint32_t* src, const uint32_t* off,
+void m2l_f64(const int* dnn, int p, const uint32_t* src, const uint32_t* off,
              const double* mult, const double* zc, const double* hs, double* loc,
              const DevTables& tb, unsigned* queue, cudaStream_t st);
 void m2l_f32(const int* dnn, int p, const uint32_t* src, const uint32_t* off,

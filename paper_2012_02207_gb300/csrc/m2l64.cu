@@ -1,7 +1,7 @@
 // Rotation-accelerated M2L (Sec. 2.4) in FP64, any order p <= 30: the steps of
 // m2l.cu,
 //     Rz(pi/2 - phi) S Rz(-theta) S  z-translation  S Rz(theta) S Rz(phi - pi/2),
-// one source per lane, a warp (or a block of four warps) per target cell.
+// one source per lane, a block of four warps per target cell.
 //
 // GB300 runs an FP64 instruction of a warp for 64 cycles of its scheduler, so
 // the FP64 operations are what bounds the kernel (about 2,860 per source at
@@ -180,33 +180,27 @@ constexpr int kM2L64Warps = 4;
 constexpr int kM2L64Blocks = 3;
 
 // PM bounds the per-thread arrays (p <= PM). A target's sources are dealt in
-// batches of 32 to kM2L64Warps parts; every part sums its batches per lane, then
-// its lanes, and the parts are added in order. share: the warps of a block take
-// a part each of one target; otherwise a warp takes all parts of a target of its
-// own, one after the other. The sums are the same either way (a forest's
-// clusters get the bits of their separate solves).
+// batches of 32 to the kM2L64Warps warps of a block; every warp sums its batches
+// per lane, then its lanes, and the warps' parts are added in order. With a target
+// to each warp, which this kernel had for larger trees, the warps of an SM gather
+// from all over the tree: beside 160 MB of per-thread arrays the multipoles no longer
+// stay in L2 (1M bodies, p = 10: 451 to 524 ms against 345, p = 12 580 against 313).
 template <int PM>
 __global__ void __launch_bounds__(32 * kM2L64Warps, kM2L64Blocks)
-    k_m2l64(const int* __restrict__ dnn, int p, bool share, const uint32_t* __restrict__ src,
+    k_m2l64(const int* __restrict__ dnn, int p, const uint32_t* __restrict__ src,
             const uint32_t* __restrict__ off, const double* __restrict__ mult, const double* __restrict__ zc,
             const double* __restrict__ hs, double* __restrict__ loc, Swap64 sw, const double* __restrict__ fact,
             const double* __restrict__ iw, unsigned* __restrict__ queue) {
-    extern __shared__ double red[];  // share: a target's sums per part
+    extern __shared__ double red[];  // the target's sums per part
     __shared__ int s_target;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nr = ncoef_real(p);
     double c[ncoef_real(PM)], acc[ncoef_real(PM)], pa[2 * (PM + 1)], pb[2 * (PM + 1)];
     for (;;) {
-        int b = 0;
-        if (!share) {
-            if (lane == 0) b = (int)atomicAdd(queue, 1u);
-            b = __shfl_sync(0xffffffffu, b, 0);
-        } else {
-            __syncthreads();  // the previous target's sums and number are consumed
-            if (threadIdx.x == 0) s_target = (int)atomicAdd(queue, 1u);
-            __syncthreads();
-            b = s_target;
-        }
+        __syncthreads();  // the previous target's sums and number are consumed
+        if (threadIdx.x == 0) s_target = (int)atomicAdd(queue, 1u);
+        __syncthreads();
+        const int b = s_target;
         if (b >= *dnn) break;
         const uint32_t q0 = off[b], q1 = off[b + 1];
         const int nbatch = (int)((q1 - q0 + 31) / 32);
@@ -214,9 +208,9 @@ __global__ void __launch_bounds__(32 * kM2L64Warps, kM2L64Blocks)
         double* out = loc + (size_t)nr * b;
         const double bx = zc[3 * b], by = zc[3 * b + 1], bz = zc[3 * b + 2];
         const double sb = hs[b];
-        for (int w = share ? wib : 0; w < nparts; w += share ? kM2L64Warps : 1) {
+        if (wib < nparts) {
             for (int j = 0; j < nr; ++j) acc[j] = 0.0;
-            for (uint32_t q = q0 + 32 * w + lane; q < q1; q += 32 * kM2L64Warps) {
+            for (uint32_t q = q0 + 32 * wib + lane; q < q1; q += 32 * kM2L64Warps) {
                 const int a = (int)src[q];
                 const double rx = zc[3 * a] - bx, ry = zc[3 * a + 1] - by, rz = zc[3 * a + 2] - bz;
                 const double sa = hs[a];
@@ -268,48 +262,35 @@ __global__ void __launch_bounds__(32 * kM2L64Warps, kM2L64Blocks)
                 halve64<8>(v, lane, 4);
                 halve64<4>(v, lane, 2);
                 halve64<2>(v, lane, 1);
-                if (j0 + lane < nr) {
-                    if (share) red[(size_t)w * nr + j0 + lane] = v[0];
-                    else out[j0 + lane] = w ? out[j0 + lane] + v[0] : v[0];
-                }
+                if (j0 + lane < nr) red[(size_t)wib * nr + j0 + lane] = v[0];
             }
         }
-        if (share) {
-            __syncthreads();
-            for (int j = threadIdx.x; j < nr; j += 32 * kM2L64Warps) {
-                double s = red[j];
-                for (int w = 1; w < nparts; ++w) s += red[(size_t)w * nr + j];
-                out[j] = s;
-            }
+        __syncthreads();
+        for (int j = threadIdx.x; j < nr; j += 32 * kM2L64Warps) {
+            double s = red[j];
+            for (int w = 1; w < nparts; ++w) s += red[(size_t)w * nr + j];
+            out[j] = s;
         }
     }
 }
 
 template <int PM>
-void launch_m2l64(bool share, const int* dnn, int p, const uint32_t* src, const uint32_t* off, const double* mult,
+void launch_m2l64(const int* dnn, int p, const uint32_t* src, const uint32_t* off, const double* mult,
                   const double* zc, const double* hs, double* loc, const DevTables& tb, unsigned* queue,
                   cudaStream_t st) {
-    const int sh = share ? kM2L64Warps * ncoef_real(p) * (int)sizeof(double) : 0;
+    const int sh = kM2L64Warps * ncoef_real(p) * (int)sizeof(double);
     (k_m2l64<PM><<<device_sm_count() * kM2L64Blocks, 32 * kM2L64Warps, sh, st>>>(
-         dnn, p, share, src, off, mult, zc, hs, loc, Swap64{tb.swap_cos, tb.swap_sin}, tb.fact, tb.iw, queue),
+         dnn, p, src, off, mult, zc, hs, loc, Swap64{tb.swap_cos, tb.swap_sin}, tb.fact, tb.iw, queue),
      note_launch());
 }
 
-// Below this many cells a target's sources are split over the four warps of a
-// block: there are too few targets to fill the SMs evenly (4096 bodies, 317
-// cells: 0.29 ms, where a warp per target would run two to six batches of
-// sources one after the other). Above it the last, partly filled round of
-// batches and the block's barriers cost more than the uneven end.
-constexpr int kM2L64FewCells = 16384;
-
 }  // namespace
 
-void m2l_f64(const int* dnn, int ncells, int p, const uint32_t* src, const uint32_t* off, const double* mult,
+void m2l_f64(const int* dnn, int p, const uint32_t* src, const uint32_t* off, const double* mult,
              const double* zc, const double* hs, double* loc, const DevTables& tb, unsigned* queue, cudaStream_t st) {
     cudaMemsetAsync(queue, 0, sizeof(unsigned), st);
-    const bool share = ncells < kM2L64FewCells;
-    if (p <= 16) launch_m2l64<16>(share, dnn, p, src, off, mult, zc, hs, loc, tb, queue, st);
-    else launch_m2l64<kMaxP>(share, dnn, p, src, off, mult, zc, hs, loc, tb, queue, st);
+    if (p <= 16) launch_m2l64<16>(dnn, p, src, off, mult, zc, hs, loc, tb, queue, st);
+    else launch_m2l64<kMaxP>(dnn, p, src, off, mult, zc, hs, loc, tb, queue, st);
 }
 
 }  // namespace gbfmm
