@@ -1021,8 +1021,13 @@ __global__ void __launch_bounds__(128, 5) k_jerk_items_f32(LeafArgs a, const flo
         const uint32_t q0 = item.q0, q1 = item.q1;
         const uint32_t slot0 = slot_first[B] + item.part * (uint32_t)nB;
         const float4 bh = a.zhi[B], bl = a.zlo[B];
-        for (int tc = item.t0; tc < item.t1; tc += 32) {
-            const int nt = item.t1 - tc < 32 ? item.t1 - tc : 32;
+        // (the FP32 sums of a target depend on G, so the targets always come in the leaf's
+        // chunks of 32: where an item is a shorter slice, slice s takes chunk s)
+        const bool sliced = a.tslice < 32;
+        const int t0 = sliced ? item.t0 / a.tslice * 32 : item.t0;
+        const int t1 = sliced ? (t0 + 32 < nB ? t0 + 32 : nB) : item.t1;
+        for (int tc = t0; tc < t1; tc += 32) {
+            const int nt = t1 - tc < 32 ? t1 - tc : 32;
             const int G = 32 / nt;
             const unsigned inv2g = ((1u << 20) + 2 * G - 1) / (2 * G);
             const int t = lane / G, sub = lane - t * G;
