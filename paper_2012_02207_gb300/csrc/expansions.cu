@@ -196,8 +196,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_p2m(TreeView t, int p, TabF64 tb
 // FP32 translations downstream add. Bound by issue (72 % of the slots). The sums over
 // the bodies took half the time with one lane to an entry, as a column has at most
 // 2(p+1) entries and the last ones few: columns of 16 entries or less give an entry
-// 2, 4 or 8 lanes. With dw_dot2 in the recurrences, P2M and M2M together: 8M bodies
-// at p = 12 20.2 -> 14.3 ms, 1M at 10 2.17 -> 1.62 ms, 4k at 8 .185 -> .164 ms.
+// 2, 4 or 8 lanes. With the M2M's swaps in one loop (translate.cu), P2M and M2M together:
+// 8M bodies at p = 12 21.1 -> 17.1 ms, 1M at 10 2.12 -> 1.77 ms, 4k at 8 .195 -> .150 ms.
 // Shared memory per warp: the tile of one chunk's harmonics, 2(p+1) rows of
 // 33 (one per body, padded), and the sums, p+1 columns of 2(p+1) entries.
 __host__ __device__ inline int p2m_dw_warp_values(int p) { return 2 * (p + 1) * 33 + (p + 1) * 2 * (p + 1); }

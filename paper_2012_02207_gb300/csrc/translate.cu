@@ -134,8 +134,7 @@ __device__ void wrotz(WarpVec<T>& w, int p, const T* pw, bool conj, int lane) {
 // v <- swap v. Real and imaginary outputs, which read the cosine and the sine
 // block, run through one loop with their own starts, so a warp with both does
 // not take the two one after the other (that left 16 of 32 lanes active; now 22.
-// With dw_add_mul the largest level of 64 clusters, 24k cells at p = 12: 518 -> 160 us;
-// the FP32 L2L of 8M bodies 3.58 -> 2.47 ms). scale: degree n also times scale[n].
+// The FP32 L2L of 8M bodies 3.58 -> 2.47 ms). scale: degree n also times scale[n].
 template <int G, bool SCALE, typename T>
 __device__ void wswap(WarpVec<T>& w, int p, const RotTables<T>& tb, int lane, const T* scale = nullptr) {
     const int nr = ncoef_real(p);
