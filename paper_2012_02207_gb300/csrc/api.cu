@@ -9,7 +9,6 @@
 // The host reads back three small things (node count, level starts, list
 // sizes); everything else stays on the device.
 #include <cmath>
-#include <cstddef>
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
@@ -325,6 +324,7 @@ int build_directed(fmm_ctx* ctx, int which, cudaStream_t st) {
     // The theta-walk's lists are sorted by (target, source), the order the
     // scalar estimate sums in.
     const int lo_bit = which >= 2 ? ctx->nb : 0;
+    const bool stall = (ctx->cfg.fault_inject & 16u) != 0;
     if (2 * ctx->nb <= 32) {
         // 32-bit keys: half the bytes per radix pass; both ping-pong halves fit in dalt
         uint32_t* ka = as<uint32_t>(ctx->dalt[which]);
@@ -332,7 +332,7 @@ int build_directed(fmm_ctx* ctx, int which, cudaStream_t st) {
         pairs_to_directed32(as<int2>(ctx->lists[which]), ctx->ds->list_cnt + which, np, ctx->nb, ka,
                             as<unsigned long long>(ctx->dcount) + 2 + which, nkeys, st);
         const int in1 = radix_sort32(ka, kb, 2 * np, 2 * ctx->nb, as<uint32_t>(ctx->hist), &ctx->ds->sort_err, st, nkeys,
-                                       lo_bit);
+                                       lo_bit, stall);
         directed_offsets_src32(in1 ? kb : ka, 2 * np, nkeys, ctx->nb, &ctx->ds->nnodes, &ctx->ds->sort_err,
                                as<uint32_t>(ctx->dsrc[which]), as<uint32_t>(ctx->doff[which]), st);
         return FMM_OK;
@@ -340,7 +340,8 @@ int build_directed(fmm_ctx* ctx, int which, cudaStream_t st) {
     pairs_to_directed(as<int2>(ctx->lists[which]), ctx->ds->list_cnt + which, np, ctx->nb,
                       as<uint64_t>(ctx->dkeys[which]), as<unsigned long long>(ctx->dcount) + 2 + which, nkeys, st);
     const int in1 = radix_sort(as<uint64_t>(ctx->dkeys[which]), nullptr, as<uint64_t>(ctx->dalt[which]), nullptr,
-                               2 * np, 2 * ctx->nb, as<uint32_t>(ctx->hist), &ctx->ds->sort_err, st, nkeys, lo_bit);
+                               2 * np, 2 * ctx->nb, as<uint32_t>(ctx->hist), &ctx->ds->sort_err, st, nkeys, lo_bit,
+                               stall);
     directed_offsets(as<uint64_t>(in1 ? ctx->dalt[which] : ctx->dkeys[which]), 2 * np, nkeys, ctx->nb,
                      &ctx->ds->nnodes, &ctx->ds->sort_err, as<uint32_t>(ctx->dsrc[which]), as<uint32_t>(ctx->doff[which]), st);
     return FMM_OK;
@@ -414,6 +415,7 @@ int run_walk(fmm_ctx* ctx, int mode, cudaStream_t st) {
         }
         if (it == kWalkBadIndex) return fail(ctx, FMM_ERR_CUDA, "dual-tree walk read an out-of-range cell index");
         if (it == FMM_ERR_TIMEOUT) return fail(ctx, it, "a bounded wait of the walk's ordered appends ran out");
+        if (it == kWalkSortFailed) return fail(ctx, FMM_ERR_TIMEOUT, "a bounded wait of a list sort ran out");
         if (it == FMM_ERR_CUDA)
             return fail(ctx, it, std::string("dual-tree walk failed: ") + cudaGetErrorString(cudaGetLastError()));
         if (it < 0) return fail(ctx, it, "dual-tree walk failed");
@@ -485,7 +487,6 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
          (rc = ensure(ctx, ctx->cid, 4 * N))))
         return rc;
     CK(rec(0));
-    static_assert(offsetof(DevScalars, sort_err) == offsetof(DevScalars, err) + sizeof(unsigned), "both words at once");
     CK(cudaMemsetAsync(&ctx->ds->err, 0, 2 * sizeof(unsigned), st));
     CK(cudaMemcpyAsync(ctx->coff.ptr, gp ? gp->h_coff : ctx->h_coff.data(), 4 * ((size_t)nclusters + 1),
                        cudaMemcpyHostToDevice, st));
@@ -503,6 +504,7 @@ int solve_device(fmm_ctx* ctx, int64_t n, int nclusters, const int64_t* offsets,
     tb.lcp = as<int8_t>(ctx->lcp); tb.win = as<int8_t>(ctx->win); tb.hi = as<uint8_t>(ctx->hi);
     tb.chunk_cnt = as<uint32_t>(ctx->chunk);
     tb.ds = ctx->ds;
+    tb.stall_sort = (ctx->cfg.fault_inject & 8u) != 0;
     int in1 = 0;
     tree_build_count(tb, &in1, st);
     ctx->sorted_in_1 = in1;

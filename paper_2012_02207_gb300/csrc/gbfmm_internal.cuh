@@ -50,6 +50,8 @@ struct DevScalars {
     int nnodes;
     int level_start[kMaxLevel + 3];
 };
+static_assert(offsetof(DevScalars, sort_err) == offsetof(DevScalars, err) + sizeof(unsigned),
+              "the two words are cleared and read at once");
 
 // Host tables of normalisation constants for hat-normalised harmonics
 // Shat_n^m = sqrt((n+m)!(n-m)!) Upsilon_n^m.
@@ -153,13 +155,14 @@ void set_global_error(const char* msg);
 // to kErrTimeout if a wait of the sort runs out (the result is then not sorted).
 // dn (device, may be NULL): the grid covers n keys but only the first
 // min(n, *dn) are sorted (a count known on the device only, in a captured solve).
+// stall (test hook): every wait of the sort runs out.
 size_t radix_hist_words(int64_t n);
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits,
                uint32_t* hist, unsigned* err, cudaStream_t st, const unsigned long long* dn = nullptr,
-               int lo_bit = 0);
+               int lo_bit = 0, bool stall = false);
 // The same for 32-bit keys without payload.
 int radix_sort32(uint32_t* k0, uint32_t* k1, int64_t n, int bits, uint32_t* hist, unsigned* err, cudaStream_t st,
-                 const unsigned long long* dn = nullptr, int lo_bit = 0);
+                 const unsigned long long* dn = nullptr, int lo_bit = 0, bool stall = false);
 // single-block exclusive scan of count uint32 values in place; total -> *total (device)
 void scan_exclusive_u32(uint32_t* data, int64_t count, uint32_t* total, cudaStream_t st);
 // the same for large tables (multi-block); scratch: scan_scratch_words(count) words
@@ -192,6 +195,7 @@ struct TreeBuffers {
     int *level, *begin, *end, *parent, *first_child, *nchild;
     int64_t node_cap;
     DevScalars* ds;
+    bool stall_sort;             // test hook: the waits of the sort by key run out
 };
 // keys -> sort -> gather -> node-start counts and their scan; the node
 // total lands at chunk_cnt[22 * nchunks]. sorted_in_1 tells where the sorted
@@ -242,6 +246,7 @@ inline int64_t walk_scan_tiles(int64_t front_cap) { return front_cap / kWalkTile
 // mode 1: the error-controlled MAC (lists m2l/p2p). Returns iterations or a
 // negative fmm_status. Counts land in ds->list_cnt.
 constexpr int kWalkBadIndex = -100;  // dual_tree_walk: a frontier entry out of range
+constexpr int kWalkSortFailed = -101;  // dual_tree_walk: a sort before the walk failed (sort_err)
 // M: cell masses, soft: Plummer softening length (0: Newtonian MAC)
 int dual_tree_walk(int mode, const TreeView& t, const double* zc, const double* r, const double* P,
                    const float* fmin, int p, double eps, const double* binom_row, const float4* zhi,

@@ -17,7 +17,8 @@
 // Waits are bounded (about a second): a block that gives up raises kErrTimeout
 // in the sort's error word and goes on with the prefix it has; its positions
 // stay inside the array, and the users of the sorted data check the word or
-// clamp what they read (the host then fails the call).
+// clamp what they read (the host then fails the call). Once the word is raised,
+// later waits last a millisecond.
 #include "gbfmm_internal.cuh"
 
 namespace gbfmm {
@@ -57,7 +58,8 @@ static_assert(kSortHeadWords % 2 == 0, "the records are 8-byte aligned");
 
 constexpr unsigned long long kRecCount = 1ull << 62, kRecPrefix = 2ull << 62;
 constexpr unsigned long long kRecValue = (1ull << 56) - 1ull;
-constexpr unsigned long long kSortWaitNs = 1000000000ull;  // one second
+constexpr unsigned long long kSortWaitNs = 1000000000ull;      // one second
+constexpr unsigned long long kSortWaitFailedNs = 1000000ull;   // when a wait before has run out
 
 __device__ __forceinline__ void rec_store(unsigned long long* p, unsigned long long v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
@@ -65,6 +67,11 @@ __device__ __forceinline__ void rec_store(unsigned long long* p, unsigned long l
 __device__ __forceinline__ unsigned long long rec_load(const unsigned long long* p) {
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned err_load(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 __device__ __forceinline__ unsigned long long sort_ns() {
@@ -145,7 +152,8 @@ __device__ __forceinline__ void rank_items(const K* key, int mine, int shift, ui
 template <typename K, bool VAL>
 __global__ void __launch_bounds__(kThreads, kPassBlocks) k_sort_pass(
     const K* __restrict__ kin, const uint32_t* __restrict__ vin, K* __restrict__ kout, uint32_t* __restrict__ vout,
-    int64_t n, const unsigned long long* __restrict__ dn, int shift, int pass, SortScratch s, unsigned* err) {
+    int64_t n, const unsigned long long* __restrict__ dn, int shift, int pass, SortScratch s, unsigned* err,
+    int stall) {
     extern __shared__ __align__(16) unsigned char sh_scatter[];
     K* skey = reinterpret_cast<K*>(sh_scatter);                                  // kTile
     uint32_t* sval = reinterpret_cast<uint32_t*>(skey + kTile);                  // kTile (VAL only)
@@ -222,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_sort_pass(
     uint32_t excl = 0;
     if (tile > 0 && d < 256) {
         constexpr int kAhead = 4;
-        const unsigned long long want = tag >> 56;
+        const unsigned long long want = (tag >> 56) + (stall ? kMaxPasses : 0);  // (stall: of no record)
         unsigned long long t0 = 0;
         bool done = false;
         for (int64_t j = tile - 1; !done; j -= kAhead) {
@@ -235,7 +243,8 @@ __global__ void __launch_bounds__(kThreads, kPassBlocks) k_sort_pass(
                     while ((w[q] >> 62) == 0ull || ((w[q] >> 56) & 63ull) != want) {
                         const unsigned long long now = sort_ns();
                         if (t0 == 0) t0 = now;
-                        if (now - t0 > kSortWaitNs) {
+                        if (now - t0 > kSortWaitNs ||
+                            (now - t0 > kSortWaitFailedNs && (err_load(err) & kErrTimeout))) {
                             atomicOr(err, kErrTimeout);
                             w[q] = kRecPrefix | tag;  // go on with what there is
                             break;
@@ -475,7 +484,7 @@ void scan_exclusive_u32(uint32_t* data, int64_t count, uint32_t* total, cudaStre
 namespace {
 template <typename K, bool VAL>
 int radix_sort_impl(K* k0, uint32_t* v0, K* k1, uint32_t* v1, int64_t n, int lo_bit, int bits, uint32_t* hist,
-                    cudaStream_t st, const unsigned long long* dn, unsigned* err) {
+                    cudaStream_t st, const unsigned long long* dn, unsigned* err, bool stall) {
     if (n <= 1 || bits <= lo_bit) return 0;
     const int npass = (bits - lo_bit + 7) / 8;
     if (n <= kTile) {
@@ -496,7 +505,7 @@ int radix_sort_impl(K* k0, uint32_t* v0, K* k1, uint32_t* v1, int64_t n, int lo_
         K* ko = cur ? k0 : k1;
         uint32_t* vo = cur ? v0 : v1;
         (k_sort_pass<K, VAL><<<nblocks, kThreads, scatter_smem<K, VAL>(), st>>>(ki, vi, ko, vo, n, dn,
-                                                                                lo_bit + 8 * pass, pass, s, err),
+                                                                                lo_bit + 8 * pass, pass, s, err, stall ? 1 : 0),
          note_launch());
         cur ^= 1;
     }
@@ -505,14 +514,14 @@ int radix_sort_impl(K* k0, uint32_t* v0, K* k1, uint32_t* v1, int64_t n, int lo_
 }  // namespace
 
 int radix_sort(uint64_t* k0, uint32_t* v0, uint64_t* k1, uint32_t* v1, int64_t n, int bits, uint32_t* hist,
-               unsigned* err, cudaStream_t st, const unsigned long long* dn, int lo_bit) {
-    return v0 ? radix_sort_impl<uint64_t, true>(k0, v0, k1, v1, n, lo_bit, bits, hist, st, dn, err)
-              : radix_sort_impl<uint64_t, false>(k0, nullptr, k1, nullptr, n, lo_bit, bits, hist, st, dn, err);
+               unsigned* err, cudaStream_t st, const unsigned long long* dn, int lo_bit, bool stall) {
+    return v0 ? radix_sort_impl<uint64_t, true>(k0, v0, k1, v1, n, lo_bit, bits, hist, st, dn, err, stall)
+              : radix_sort_impl<uint64_t, false>(k0, nullptr, k1, nullptr, n, lo_bit, bits, hist, st, dn, err, stall);
 }
 
 int radix_sort32(uint32_t* k0, uint32_t* k1, int64_t n, int bits, uint32_t* hist, unsigned* err, cudaStream_t st,
-                 const unsigned long long* dn, int lo_bit) {
-    return radix_sort_impl<uint32_t, false>(k0, nullptr, k1, nullptr, n, lo_bit, bits, hist, st, dn, err);
+                 const unsigned long long* dn, int lo_bit, bool stall) {
+    return radix_sort_impl<uint32_t, false>(k0, nullptr, k1, nullptr, n, lo_bit, bits, hist, st, dn, err, stall);
 }
 
 }  // namespace gbfmm

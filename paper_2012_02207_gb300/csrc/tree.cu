@@ -526,7 +526,7 @@ void tree_build_count(TreeBuffers& b, int* sorted_in_1, cudaStream_t st) {
      note_launch());
     (k_bbox_final<<<blocks_for((int64_t)nc * 32, 128), 128, 0, st>>>(b.bbox_part, nc, slices, b.box), note_launch());
     (k_keys<<<blocks_for(n, 256), 256, 0, st>>>(b.x, b.y, b.z, n, b.coff, nc, b.box, b.k0, b.v0), note_launch());
-    int in1 = radix_sort(b.k0, b.v0, b.k1, b.v1, n, 63, b.hist, &b.ds->sort_err, st);
+    int in1 = radix_sort(b.k0, b.v0, b.k1, b.v1, n, 63, b.hist, &b.ds->sort_err, st, nullptr, 0, b.stall_sort);
     const uint64_t* keys = in1 ? b.k1 : b.k0;
     const uint32_t* perm = in1 ? b.v1 : b.v0;
     const uint32_t* cid = nullptr;
