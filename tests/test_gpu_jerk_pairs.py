@@ -33,3 +33,30 @@ def test_mixed_near_jerk(n, leaf, soft):
         r2[np.arange(len(r2)), np.arange(i, i + len(r2))] = np.inf  # the body itself
         scale[i:i + 256] = (m[None] * np.linalg.norm(u, axis=-1) / r2**1.5).sum(1)
     assert np.max(np.linalg.norm(jerk - ref, axis=1) / scale) <= 1e-5
+
+
+def test_fp64_jerk_does_not_depend_on_the_size_of_the_tree():
+    """Work items are shorter slices of a leaf's targets below 2048 cells. Two trees with the same cluster,
+    one on each side of that: the other bodies are as good as massless and in octants of their own, where the
+    cluster sees them as one cell (or one body), so every sum over the cluster has the same terms."""
+    import torch
+
+    import paper_2012_02207_gb300 as gb
+
+    rng = np.random.default_rng(5)
+    n = 3001
+    pos = -0.5 + 0.02 * rng.standard_normal((n, 3)).clip(-2.0, 2.0)
+    vel = rng.standard_normal((n, 3))
+    corners = np.array([[-1.0, 1.0, -1.0], [1.0, -1.0, 1.0]])  # they set the cube
+    out, cells = [], []
+    for extra in (1, 9000):
+        other = 0.5 + 0.02 * rng.standard_normal((extra, 3)).clip(-2.0, 2.0)
+        q = np.concatenate([pos, corners, other])
+        u = np.concatenate([vel, np.zeros((2 + extra, 3))])
+        m = np.concatenate([np.full(n, 1.0 / n), np.full(2 + extra, 1e-300)])
+        f = gb.FMM(p=8, eps=1e-6, leaf_size=13, precision="fp64")
+        cols = [torch.tensor(np.ascontiguousarray(c), device="cuda") for c in (*q.T, *u.T, m)]
+        out.append(torch.stack(f.solve_jerk(*cols))[:, :n])
+        cells.append(f.stats()["nnodes"])
+    assert cells[0] < 2048 < cells[1]
+    assert torch.equal(out[0], out[1])
