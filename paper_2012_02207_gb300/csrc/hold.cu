@@ -119,12 +119,68 @@ struct HoldFrame {
 constexpr int kHoldThreads = 256;
 
 constexpr int kHoldPairs = 1024;  // pairs whose terms are in shared memory at a time (>= kHoldSmallMax)
+constexpr int kHoldWhole = kHoldPairs / 4;  // sets up to here always have four whole rows in a chunk
+constexpr int kHoldRows = 16;               // rows of a chunk of a larger set's pairs
 constexpr int kHoldUnsure = 256;  // pairs the bounds leave open, listed before they are evaluated
 
 // shared memory of a kick's terms or a split's FP32 members
 __host__ __device__ constexpr size_t hold_term_bytes(int k) {
     return 6 * kHoldPairs * sizeof(double) > (size_t)k * sizeof(PairBody32) ? 6 * kHoldPairs * sizeof(double)
                                                                            : (size_t)k * sizeof(PairBody32);
+}
+
+// The two terms of pair (a, b) of a set, on a and on b, to term[e].
+__device__ __forceinline__ void kick_pair(const int* ix, int a, int b, const double* px, const double* py,
+                                          const double* pz, const double* pm, double soft2, double* term, int e) {
+    const int i = ix[a], j = ix[b];
+    const double dx = px[j] - px[i], dy = py[j] - py[i], dz = pz[j] - pz[i];
+    double r2 = dx * dx + dy * dy + dz * dz;
+    if (soft2 > 0.0) r2 = r2 + soft2;
+    const double r = sqrt(r2);
+    const double r3 = r2 * r;
+    const double ma = pm[j] / r3, mb = pm[i] / r3;
+    term[e] = ma * dx;
+    term[kHoldPairs + e] = ma * dy;
+    term[2 * kHoldPairs + e] = ma * dz;
+    // (the pair seen from b: exactly the opposite offsets)
+    term[3 * kHoldPairs + e] = mb * -dx;
+    term[4 * kHoldPairs + e] = mb * -dy;
+    term[5 * kHoldPairs + e] = mb * -dz;
+}
+
+// The sums of a kick where few rows of a set fit in term: chunks of kHoldRows rows,
+// each in tiles of columns from the chunk's first row on. A body's column comes in the
+// chunks of the rows below it, then its row with the columns above it, tile by tile.
+__device__ void kick_sums_tiled(const int* ix, int n, int ns, const double* px, const double* py,
+                                             const double* pz, const double* pm, double soft2, double* acc,
+                                             double* term) {
+    const int tid = threadIdx.x;
+    const int rows = kHoldRows < ns ? kHoldRows : ns, cols = kHoldPairs / rows;  // (cols >= rows)
+    for (int a0 = 0; a0 < ns; a0 += rows) {
+        const int a1 = a0 + rows < ns ? a0 + rows : ns;
+        for (int c0 = a0; c0 < n; c0 += cols) {
+            const int c1 = c0 + cols < n ? c0 + cols : n, w = c1 - c0;
+            for (int e = tid; e < (a1 - a0) * w; e += kHoldThreads) {
+                const int a = a0 + e / w, b = c0 + e % w;
+                if (b > a) kick_pair(ix, a, b, px, py, pz, pm, soft2, term, e);
+            }
+            __syncthreads();
+            // the columns' sums and, after the first tile, where they are no longer columns, the rows'
+            const int ncol = 3 * w, nrow = c0 > a0 ? 3 * (a1 - a0) : 0;
+            for (int e = tid; e < ncol + nrow; e += kHoldThreads) {
+                const int c = e % 3, s = e < ncol ? c0 + e / 3 : a0 + (e - ncol) / 3;
+                const double* on_b = term + (3 + c) * kHoldPairs + (s - c0);
+                const double* on_a = term + c * kHoldPairs + (s - a0) * w - c0;
+                double v = acc[3 * s + c];
+                if (e < ncol)
+                    for (int a = a0; a < a1 && a < s; ++a) v += on_b[(a - a0) * w];
+                if (s < a1)
+                    for (int b = s + 1 > c0 ? s + 1 : c0; b < c1; ++b) v += on_a[b];
+                acc[3 * s + c] = v;
+            }
+            __syncthreads();
+        }
+    }
 }
 
 // Kick of the set ix[0..n), its first ns members slow: slow bodies feel
@@ -134,44 +190,40 @@ __host__ __device__ constexpr size_t hold_term_bytes(int k) {
 // body s adds its sources in order: those of the chunk's rows below s, then,
 // if s is itself a row of the chunk, those above s. acc: 3 n sums; term:
 // 6 kHoldPairs values (on a from b, then on b from a).
+//
+// A row's sum is serial, and an FP64 instruction takes the pipe as long for one lane as
+// for 32, so a chunk needs several rows: where fewer than four (and not all) fit, rows
+// come in tiles (LARGE; in a kernel of their own, as the code costs the small sets 1 to 4 %). Kicks of a whole set, ms each, one thread per body | whole rows |
+// tiles: 256 bodies 1.7 | 0.9 | -, 512 7.0 | 4.7 | 2.2, 700 13.1 | 13.6 | 4.0, 1024 27.9 | 28.4 | 8.6.
+template <bool LARGE>
 __device__ void set_kick(const int* ix, int n, int ns, const double* px, const double* py, const double* pz,
                           const double* pm, double* pvx, double* pvy, double* pvz, double G, double soft2, double h,
                           double* acc, double* term) {
     const int tid = threadIdx.x;
-    const int rows = kHoldPairs / n < ns ? kHoldPairs / n : ns;
+    const int fit = kHoldPairs / n, rows = fit < ns ? fit : ns;
     for (int e = tid; e < 3 * n; e += kHoldThreads) acc[e] = 0.0;
-    for (int a0 = 0; a0 < ns; a0 += rows) {
-        const int a1 = a0 + rows < ns ? a0 + rows : ns;
-        for (int e = tid; e < (a1 - a0) * n; e += kHoldThreads) {
-            const int a = a0 + e / n, b = e % n;
-            if (b <= a) continue;
-            const int i = ix[a], j = ix[b];
-            const double dx = px[j] - px[i], dy = py[j] - py[i], dz = pz[j] - pz[i];
-            double r2 = dx * dx + dy * dy + dz * dz;
-            if (soft2 > 0.0) r2 = r2 + soft2;
-            const double r = sqrt(r2);
-            const double r3 = r2 * r;
-            const double ma = pm[j] / r3, mb = pm[i] / r3;
-            term[e] = ma * dx;
-            term[kHoldPairs + e] = ma * dy;
-            term[2 * kHoldPairs + e] = ma * dz;
-            // (the pair seen from b: exactly the opposite offsets)
-            term[3 * kHoldPairs + e] = mb * -dx;
-            term[4 * kHoldPairs + e] = mb * -dy;
-            term[5 * kHoldPairs + e] = mb * -dz;
+    if (LARGE && fit < 4 && fit < ns) {
+        kick_sums_tiled(ix, n, ns, px, py, pz, pm, soft2, acc, term);
+    } else {
+        for (int a0 = 0; a0 < ns; a0 += rows) {
+            const int a1 = a0 + rows < ns ? a0 + rows : ns;
+            for (int e = tid; e < (a1 - a0) * n; e += kHoldThreads) {
+                const int a = a0 + e / n, b = e % n;
+                if (b > a) kick_pair(ix, a, b, px, py, pz, pm, soft2, term, e);
+            }
+            __syncthreads();
+            for (int e = a0 * 3 + tid; e < 3 * n; e += kHoldThreads) {  // bodies below a0 have all their sources
+                const int s = e / 3, c = e - 3 * s;
+                const double* on_b = term + (3 + c) * kHoldPairs + s;
+                const double* on_a = term + c * kHoldPairs + (s - a0) * n;
+                double v = acc[e];
+                for (int a = a0; a < a1 && a < s; ++a) v += on_b[(a - a0) * n];
+                if (s < a1)
+                    for (int b = s + 1; b < n; ++b) v += on_a[b];
+                acc[e] = v;
+            }
+            __syncthreads();
         }
-        __syncthreads();
-        for (int e = a0 * 3 + tid; e < 3 * n; e += kHoldThreads) {  // bodies below a0 have all their sources
-            const int s = e / 3, c = e - 3 * s;
-            const double* on_b = term + (3 + c) * kHoldPairs + s;
-            const double* on_a = term + c * kHoldPairs + (s - a0) * n;
-            double v = acc[e];
-            for (int a = a0; a < a1 && a < s; ++a) v += on_b[(a - a0) * n];
-            if (s < a1)
-                for (int b = s + 1; b < n; ++b) v += on_a[b];
-            acc[e] = v;
-        }
-        __syncthreads();
     }
     for (int s = tid; s < n; s += kHoldThreads) {
         const int i = ix[s];
@@ -236,6 +288,8 @@ __device__ void set_fast_bits(const int* ix, int n, const double* px, const doub
 }
 
 // stats: {slow-system kicks, FMM solves (none here), direct solves, deepest level, splits}
+// LARGE: k may be above kHoldWhole
+template <bool LARGE>
 __global__ void __launch_bounds__(kHoldThreads) k_hold_small(int k, const int* __restrict__ idx, double* x,
                                                              double* y, double* z, double* vx, double* vy,
                                                              double* vz, const double* __restrict__ m, double G,
@@ -323,7 +377,7 @@ __global__ void __launch_bounds__(kHoldThreads) k_hold_small(int k, const int* _
             if (f.ns > 0) {
                 // slow bodies feel all of P, fast ones the slow ones; drift the slow ones
                 const double h = 0.5 * f.dt;
-                set_kick(ix + f.lo, n, f.ns, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h, acc, term);
+                set_kick<LARGE>(ix + f.lo, n, f.ns, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h, acc, term);
                 for (int t = f.lo + tid; t < s1; t += kHoldThreads) {
                     const int i = ix[t];
                     px[i] += f.dt * pvx[i];
@@ -331,7 +385,7 @@ __global__ void __launch_bounds__(kHoldThreads) k_hold_small(int k, const int* _
                     pz[i] += f.dt * pvz[i];
                 }
                 __syncthreads();
-                set_kick(ix + f.lo, n, f.ns, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h, acc, term);
+                set_kick<LARGE>(ix + f.lo, n, f.ns, px, py, pz, pm, pvx, pvy, pvz, G, soft2, h, acc, term);
                 kicks += 2;
                 direct += (f.ns < n) ? 4 : 2;
             }
@@ -421,10 +475,14 @@ void hold_small(int k, const int* idx, double* x, double* y, double* z, double* 
                 unsigned long long* stats, cudaStream_t st) {
     if (k <= 0) return;
     const size_t sh = hold_small_smem(k);
-    ensure_dyn_smem((const void*)k_hold_small, (int)hold_small_smem(kHoldSmallMax));
-    (k_hold_small<<<1, kHoldThreads, sh, st>>>(k, idx, x, y, z, vx, vy, vz, m, G, soft * soft, eta, sym ? 1 : 0, dt,
-                                               dt_min, depth, stats),
-     note_launch());
+    auto go = [&](auto kernel, int most) {
+        ensure_dyn_smem((const void*)kernel, (int)hold_small_smem(most));
+        (kernel<<<1, kHoldThreads, sh, st>>>(k, idx, x, y, z, vx, vy, vz, m, G, soft * soft, eta, sym ? 1 : 0, dt,
+                                             dt_min, depth, stats),
+         note_launch());
+    };
+    if (k <= kHoldWhole) go(k_hold_small<false>, kHoldWhole);
+    else go(k_hold_small<true>, kHoldSmallMax);
 }
 
 }  // namespace gbfmm
