@@ -140,7 +140,7 @@ struct fmm_ctx {
     // sizes, split flags and scan, the fast count; per-depth slow/fast lists
     Buf h_all, h_gat, h_acc, h_acc2, h_tau, h_flag, h_scan, h_scr, h_nf;
     std::vector<Buf> h_S, h_F;
-    Buf step_upper;  // per-body bounds of the step sizes
+    Buf step_scratch;  // of the step sizes
     // walk and lists
     // per list: sorted directed keys, the sort's second buffer (its own, so a
     // buffer never moves to a list of another size), CSR offsets
@@ -816,6 +816,7 @@ struct HoldRun {
     int64_t direct_below;
     int64_t device_below;                   // sets of at most this many bodies evolve in one block
     unsigned long long* dstats = nullptr;   // the device-resident evolutions' counters (device)
+    bool units = false;                     // the units of the step sizes' bounds are set
     int64_t kicks = 0, fmm_solves = 0, direct_solves = 0, max_depth = 0, splits = 0;
 };
 
@@ -889,8 +890,12 @@ int hold_evolve(HoldRun& R, const int* P, int k, double dt, int depth) {
         double* g = as<double>(ctx->h_gat);
         hold_gather(k, P, R.x, R.y, R.z, R.vx, R.vy, R.vz, R.m, g, k, -1, R.st);
         const size_t K = (size_t)k;
+        if (!R.units) {  // once: the first set is the whole cluster
+            timestep_units(k, g, g + K, g + 2 * K, g + 6 * K, ctx->cfg.G, ctx->step_scratch.ptr, R.st);
+            R.units = true;
+        }
         timesteps_f64(k, g, g + K, g + 2 * K, g + 3 * K, g + 4 * K, g + 5 * K, g + 6 * K, ctx->cfg.G, R.eta, R.sym,
-                      as<double>(ctx->h_tau), as<unsigned>(ctx->step_upper), R.st);
+                      as<double>(ctx->h_tau), ctx->step_scratch.ptr, R.st);
         hold_split(k, P, as<double>(ctx->h_tau), dt, as<uint32_t>(ctx->h_flag), as<uint32_t>(ctx->h_scan),
                    as<int>(ctx->h_S[depth]), as<int>(ctx->h_F[depth]), as<uint32_t>(ctx->h_nf),
                    as<uint32_t>(ctx->h_scr), R.st);
@@ -1048,7 +1053,7 @@ void fmm_destroy(fmm_ctx* ctx) {
                   &ctx->part_lo, &ctx->work, &ctx->coff, &ctx->box, &ctx->ck0, &ctx->ck1, &ctx->cv0,
                   &ctx->cv1, &ctx->cid, &ctx->jv, &ctx->jv32, &ctx->jw, &ctx->jmom, &ctx->jmult,
                   &ctx->jmult32, &ctx->jloc, &ctx->jloc32, &ctx->h_all, &ctx->h_gat, &ctx->h_acc, &ctx->h_acc2,
-                  &ctx->h_tau, &ctx->h_flag, &ctx->h_scan, &ctx->h_scr, &ctx->h_nf, &ctx->geo, &ctx->step_upper};
+                  &ctx->h_tau, &ctx->h_flag, &ctx->h_scan, &ctx->h_scr, &ctx->h_nf, &ctx->geo, &ctx->step_scratch};
     for (Buf* b : all) release(*b);
     for (Buf& b : ctx->h_S) release(b);
     for (Buf& b : ctx->h_F) release(b);
@@ -1298,7 +1303,7 @@ int fmm_hold(fmm_ctx* ctx, int64_t n, double* x, double* y, double* z, double* v
         (rc = ensure(ctx, ctx->h_acc, 32 * N)) || (rc = ensure(ctx, ctx->h_acc2, 32 * N)) ||
         (rc = ensure(ctx, ctx->h_tau, 8 * N)) || (rc = ensure(ctx, ctx->h_flag, 4 * N)) ||
         (rc = ensure(ctx, ctx->h_scan, 4 * N)) || (rc = ensure(ctx, ctx->h_scr, 4 * scan_scratch_words((int64_t)N))) ||
-        (rc = ensure(ctx, ctx->h_nf, 64)) || (rc = ensure(ctx, ctx->step_upper, sizeof(unsigned) * N, false)))
+        (rc = ensure(ctx, ctx->h_nf, 64)) || (rc = ensure(ctx, ctx->step_scratch, timesteps_scratch_bytes(n), false)))
         return rc;
     R.dstats = as<unsigned long long>(ctx->h_nf) + 1;  // words 1..5 (word 0 holds the split's fast count)
     CK(cudaMemsetAsync(R.dstats, 0, 5 * sizeof(unsigned long long), R.st));
@@ -1332,9 +1337,10 @@ int fmm_timesteps(fmm_ctx* ctx, int64_t n, const double* x, const double* y, con
     if (!x || !y || !z || !vx || !vy || !vz || !m || !tau) return fail(ctx, FMM_ERR_ARG, "NULL pointer");
     cudaSetDevice(ctx->device);
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const int rc = ensure(ctx, ctx->step_upper, sizeof(unsigned) * (size_t)n, false);
+    const int rc = ensure(ctx, ctx->step_scratch, timesteps_scratch_bytes(n), false);
     if (rc != FMM_OK) return rc;
-    timesteps_f64((int)n, x, y, z, vx, vy, vz, m, ctx->cfg.G, eta, symmetrize != 0, tau, as<unsigned>(ctx->step_upper),
+    timestep_units((int)n, x, y, z, m, ctx->cfg.G, ctx->step_scratch.ptr, st);
+    timesteps_f64((int)n, x, y, z, vx, vy, vz, m, ctx->cfg.G, eta, symmetrize != 0, tau, ctx->step_scratch.ptr,
                   st);
     CK(cudaGetLastError());
     CK(cudaStreamSynchronize(st));

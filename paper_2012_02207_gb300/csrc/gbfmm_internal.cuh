@@ -410,10 +410,15 @@ void jerk_leaves(const LeafArgs& a, bool fp32, const void* locj, const double* v
                  unsigned* work, const int* leaf_of, double* jx, double* jy, double* jz, cudaStream_t st);
 // ------------------------------------------------------------- timestep.cu
 // HOLD step sizes: tau_i = min over j != i of the pair step (Appendix A);
-// upper: n words of scratch
+// scratch: timesteps_scratch_bytes(n), where timestep_units has put the units of the
+// FP32 bounds (any units give the same step sizes; those of other bodies of the
+// same cluster do as well)
+size_t timesteps_scratch_bytes(int64_t n);
+void timestep_units(int n, const double* x, const double* y, const double* z, const double* m, double G,
+                    void* scratch, cudaStream_t st);
 void timesteps_f64(int n, const double* x, const double* y, const double* z, const double* vx, const double* vy,
                    const double* vz, const double* m, double G, double eta, bool sym, double* tau,
-                   unsigned* upper, cudaStream_t st);
+                   void* scratch, cudaStream_t st);
 // ----------------------------------------------------------------- hold.cu
 constexpr int kHoldMaxDepth = 60;                  // no set is split below this level
 constexpr int kHoldMaxLevels = kHoldMaxDepth + 1;  // frames of the device-resident recursion

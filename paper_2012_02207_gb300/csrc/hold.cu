@@ -267,7 +267,8 @@ __device__ void set_fast_bits(const int* ix, int n, const double* px, const doub
         const int a = p - b * (b - 1) / 2;
         const PairScale32 scale(b32[a], G, eta);
         float lo, hi;
-        pair_bounds32(b32[a], b32[b], scale, sym, lo, hi);
+        // (equal velocities are rare after a first kick: such a pair is evaluated)
+        pair_bounds32(b32[a], b32[b], scale, sym, [] { return false; }, lo, hi);
         if (hi < dtf) {
             mark(a, b);
         } else if (lo < dtf) {

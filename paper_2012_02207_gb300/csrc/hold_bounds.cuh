@@ -11,9 +11,12 @@
 //   d_fl = eta S cos, S = 1 + gm / (r v^2)               below eta S 2^-18,
 // both capped at 1, so D = 1 - d/2 >= 1/2 has a relative error below 0.75 T 2^-17.4 / D
 // and eta S 2^-19 / D. The bounds take K (1 + T / D) and K (1 + eta S / D) with
-// K = 2^-16 as the relative errors of t / D. Outside the ranges that keep every
-// intermediate a normal number, and for differences too close to cancel, the
-// pair gets lo = -1 and hi = infinity: it is always evaluated exactly.
+// K = 2^-16 as the relative errors of t / D. For bodies of equal velocity (a cluster
+// starting from rest), which the caller compares, t_ff alone counts and d_ff = 0. Outside
+// the ranges that keep every intermediate a normal number, and for differences too
+// close to cancel, the pair gets lo = -1 and hi = infinity: it is always evaluated
+// exactly. The ranges are those of units in which lengths, masses times G and with them
+// speeds are of order 1 up to powers of the number of bodies (PairBody32::scale).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -33,6 +36,13 @@ struct PairBody32 {
         c.z = (float)w; c.w = (float)(w - (double)c.z);
         m = (float)mass;
     }
+    // to other units: lengths, speeds by powers of two, masses by any factor (t = eta r / v and
+    // t^2 = eta^2 r^3 / (G m) keep their order in units of length L, speed V and mass L V^2)
+    __device__ __forceinline__ void scale(float l, float v, float g) {
+        a.x *= l; a.y *= l; a.z *= l; a.w *= l; b.x *= l; b.y *= l;
+        b.z *= v; b.w *= v; c.x *= v; c.y *= v; c.z *= v; c.w *= v;
+        m *= g;
+    }
 };
 
 // the body's own constants: the smallest squared distance and speed that its
@@ -51,8 +61,17 @@ struct PairScale32 {
     }
 };
 
+// equal numbers, by integer tests (an FP64 comparison would cost an FP64 instruction)
+__device__ __forceinline__ bool same_number(double a, double b) {
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    return x == y || (x | y) << 1 == 0;  // (zeros of either sign)
+}
+
+// same_velocity(): whether the bodies' FP64 velocities are equal; asked only where the difference is
+// too close to cancel.
+template <typename Same>
 __device__ __forceinline__ void pair_bounds32(const PairBody32& p, const PairBody32& q, const PairScale32& s, bool sym,
-                                              float& lo, float& hi) {
+                                              Same same_velocity, float& lo, float& hi) {
     constexpr float K = 0x1p-16f;
     const float dx = (q.a.x - p.a.x) + (q.a.y - p.a.y), dy = (q.a.z - p.a.z) + (q.a.w - p.a.w),
                 dz = (q.b.x - p.b.x) + (q.b.y - p.b.y);
@@ -60,8 +79,8 @@ __device__ __forceinline__ void pair_bounds32(const PairBody32& p, const PairBod
                 uz = (q.c.z - p.c.z) + (q.c.w - p.c.w);
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz)), v2 = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
     const float gm = s.G * (p.m + q.m);
-    const bool ok = s.ok && r2 >= s.r2min && r2 <= 0x1p40f && v2 >= s.v2min && v2 <= 0x1p40f && gm >= 0x1p-60f &&
-                    gm <= 0x1p20f;
+    const bool ok = s.ok && r2 >= s.r2min && r2 <= 0x1p40f && gm >= 0x1p-60f && gm <= 0x1p20f;
+    const bool moving = v2 >= s.v2min && v2 <= 0x1p60f;
     const float ir = rsqrtf(r2), iv = rsqrtf(v2), r = r2 * ir;
     const float c = r2 * r * __fdividef(1.0f, gm);
     const float tff = s.eta * (c * rsqrtf(c)), tfl = s.eta * r * iv;
@@ -82,9 +101,10 @@ __device__ __forceinline__ void pair_bounds32(const PairBody32& p, const PairBod
     const float hfl = kfl <= 0.25f ? afl * fmaf(2.0f, kfl, 1.0f) : __int_as_float(0x7f800000);
     hi = fminf(hff, hfl);
     // (a NaN bound fails the comparison and counts as out of range)
-    if (!(ok && kff < 1e30f && kfl < 1e30f && hi > 0.0f)) {
-        lo = -1.0f;
-        hi = __int_as_float(0x7f800000);
+    if (!(ok && moving && kff < 1e30f && kfl < 1e30f && hi > 0.0f)) {
+        const bool rest = ok && v2 < s.v2min && same_velocity();
+        lo = rest ? tff * (1.0f - K) : -1.0f;
+        hi = rest ? tff * (1.0f + 2.0f * K) : __int_as_float(0x7f800000);
     }
 }
 

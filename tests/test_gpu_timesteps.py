@@ -68,3 +68,50 @@ def test_edges_of_the_bounds(case):
             pos[i + 1] = pos[i] + 1e-3 * d
             vel[i + 1] = vel[i] + (d if i % 4 else np.cross(d, [1.0, 0.0, 0.0])) * 10.0 ** rng.uniform(-2, 3)
     check(pos, vel, m, eta=eta, G=G)
+
+
+# lengths, speeds and masses of the caller's units (G to match), from rest, and with bodies whose exponents pull the
+# bounds' units away from the rest's: far out, heavy, at the origin or at the same place as another's first
+@pytest.mark.parametrize("length,mass,G", [(3.086e16, 1.989e30, 6.674e-11), (3.086e18, 1.989e33, 6.674e-8),
+                                           (1.0, 1.0, 4.49e-3), (1e-120, 1e-200, 1.0), (1e30, 1e-40, 1e-20)])
+@pytest.mark.parametrize("case", ["", "at rest", "common velocity", "outliers", "at the origin"])
+def test_units(length, mass, G, case):
+    rng = np.random.default_rng(4)
+    n = 300
+    pos, vel, _ = ics.plummer(n, 74, center=False)
+    m = ics.kroupa_masses(n, 75)
+    if case == "at rest":
+        vel[:] = 0.0
+        vel[::50] = rng.normal(size=(6, 3))
+    elif case == "common velocity":
+        vel[:] = [0.1, -0.2, 0.3]
+    elif case == "outliers":
+        pos[::40] *= 1e12
+        m[5::40] *= 1e15
+        vel[::9] *= 1e-14
+    elif case == "at the origin":
+        pos[0] = 0.0
+        pos[1:200] *= 1e-5
+    check(pos * length, vel * np.sqrt(G * mass / length), m * mass, G=G)
+
+
+def test_time_does_not_depend_on_the_units_or_the_velocities():
+    """SI units and a start from rest cost what N-body units do (where no bound decides, every pair is
+    evaluated exactly, which takes 18 times as long)."""
+    n = 16384
+    pos, vel, m = ics.plummer(n, 76)
+    L, M, G = 3.086e16, 1.989e30, 6.674e-11
+    ms = []
+    for p, v, w, g in ((pos, vel, m, 1.0), (pos * L, vel * np.sqrt(G * M / L), m * M, G), (pos, 0.0 * vel, m, 1.0)):
+        cols = [torch.tensor(np.ascontiguousarray(c), dtype=torch.float64, device="cuda") for c in (*p.T, *v.T, w)]
+        f = gb.FMM(G=g)
+        t = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            f.timesteps(*cols, eta=0.025)
+            b.record()
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+        ms.append(min(t[1:]))
+    assert max(ms) < 3.0 * ms[0], ms
