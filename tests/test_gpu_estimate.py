@@ -43,3 +43,26 @@ def test_estimate_outside_the_fast_range(length, mass):
     """Squared distances below 2^-80 or above 2^80, masses below 2^-40 or above 2^40."""
     pos, _, _ = ics.plummer(900, 5, center=False)
     check(pos * length, ics.kroupa_masses(900, 6) * mass, 64)
+
+
+@pytest.mark.parametrize("target", [2.0 - 2.0**-23, 1.0 + 2.0**-23, 2.0 - 2.0**-22, 1.0])
+def test_estimate_at_extreme_significands(target):
+    """Squared distances whose significand is all ones, just above one, or one, by masses of a power of two and
+    others: where a reciprocal that is off by an ulp would show in the quotient. The pair's offsets in x and y
+    are chosen so that the FP32 sum of their squares is the wanted number."""
+    def squared(x, y):
+        return np.float32(np.float32(x * x) + np.float32(y * y))
+
+    t32, found = np.float32(target), None
+    x = np.float32(np.sqrt(target))
+    while found is None:  # x * x at or below the target, the rest by y
+        rest = target - float(x) ** 2
+        for y in np.float32(np.sqrt(max(rest, 0.0))) * np.linspace(0.9, 1.1, 201, dtype=np.float32):
+            if squared(x, y) == t32:
+                found = (x, y)
+        x = np.nextafter(x, np.float32(0))
+    dx, dy = (float(v) for v in found)
+    for scale in (2.0**-30, 1.0, 2.0**20):
+        pos = 0.5 * scale * np.array([[-dx, -dy, 0.0], [dx, dy, 0.0]])
+        for mass in (1.0, 2.0**-20, 2.0**-17, 1.5, 2.0 - 2.0**-23, 1.0 + 2.0**-23, 1 / 3):
+            check(pos, np.array([mass, mass]), 64)
