@@ -68,3 +68,20 @@ def test_fp64_forest_equals_separate_solves():
         g = gb.FMM(p=5, eps=1e-6, leaf_size=4, precision="fp64")
         one = torch.stack(g.solve(*(c[a:b].contiguous() for c in cols)))
         assert torch.equal(one, out[:, a:b])
+
+
+def test_fp64_m2l_source_counts():
+    """A block takes a target; its four warps take the sources in batches of 32. Targets without sources, of one,
+    part of one, two, three, four and more batches, against the oracle."""
+    n, p, leaf, eps = 12000, 5, 8, 1e-5
+    pos, _, m = ics.plummer(n, 10)
+    f, acc, pot = solve(pos, m, p=p, eps=eps, leaf_size=leaf)
+    count = np.bincount(f.export_pairs("m2l").ravel(), minlength=f.stats()["nnodes"])
+    batches = np.bincount((count + 31) // 32)
+    assert np.all(batches[:6] > 0) and np.any((count > 0) & (count < 32)) and np.any(count % 32 == 0)
+    oacc, opot = oracle.fmm(pos, m, p=p, eps=eps, leaf_size=leaf)
+    run = oracle.OracleRun(pos, m, p=p, eps=eps, leaf_size=leaf, stage=oracle.STAGE_F)
+    fi = np.empty(n)
+    fi[run.tree()["perm"]] = run.geometry()["f"]
+    assert np.max(np.linalg.norm(acc - oacc, axis=1) / fi) <= 1e-12
+    assert np.max(np.abs(pot - opot) / np.abs(opot)) <= 1e-12
