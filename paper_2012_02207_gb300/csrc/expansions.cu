@@ -311,7 +311,9 @@ void launch_p2m_dw_split(const TreeView& t, int p, const double* xs, const doubl
 
 // A leaf's columns go to the four warps of a block where the tree has so few nodes
 // that a warp per leaf leaves most of the chip idle (the columns are independent:
-// the results are the same). N = 4096, 317 nodes, p = 8: 39 -> 20 us.
+// the results are the same). Upward pass with a warp and with four, ms: 287 cells, p = 8
+// .164 | .147; p = 10: 1237 cells .223 | .211, 1977 .234 | .230, 3234 .248 | .257, 12450 .516 |
+// .566, 62640 1.79 | 2.11.
 constexpr int kSplitCells = 2048;
 void launch_p2m_dw(const TreeView& t, int p, const double* xs, const double* ys, const double* zs, const double* w,
                    const double* zc, const double* hs, double* mult, cudaStream_t st) {
@@ -323,9 +325,10 @@ void launch_p2m_dw(const TreeView& t, int p, const double* xs, const double* ys,
 // (also the FP32 copies used by the walk's screen: Phat_n = P_n / s^n)
 // LANES threads per node, thread j the degrees n = j, j + LANES, ..: each
 // degree's sum and power of s keep their order. Four for small trees, where a
-// node's chain of operations bounds the launch (N = 4096: 28 us with one,
-// 11 us with four), one above kPnormCells, where the FP64 instructions
-// do (the degrees of unequal length leave lanes idle).
+// node's chain of operations bounds the launch, one above kPnormCells, where the FP64
+// instructions do (the degrees of unequal length leave lanes idle). Upward pass with one
+// and with four, p = 10, ms: 1237 cells .234 | .211, 6128 .373 | .355, 18888 .703 | .691,
+// 35473 1.174 | 1.165, 62640 1.791 | 1.791.
 constexpr int kPnormCells = 16384;
 template <int LANES>
 __global__ void k_pnorm(const int* __restrict__ dnn, int p, const double* __restrict__ mult,

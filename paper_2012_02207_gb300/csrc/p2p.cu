@@ -1320,11 +1320,12 @@ void upload_leaf_tables(const HostTables& h) {
 
 // Targets per work item. A slice stages the sources again, so whole leaves are
 // cheapest where there are items enough; on a small tree an item per part of a
-// leaf leaves most warps idle. FP32: up to 2048 cells slices of 8 (N = 4096:
-// leaf phase 0.232 ms whole, 0.154 by 16, 0.144 by 8; at 4282 cells 0.80 whole
-// and by 32, 0.84 by 16). FP64, where staging hides behind the arithmetic: 4 up to
-// 2048 cells (N = 4096: 3.73 ms whole, 1.21 by 8, 0.93 by 4), 8 above (N =
-// 100000: 35.5 ms whole, 33.2 by 8, 33.8 by 4).
+// leaf leaves most warps idle. Leaf phase in ms, whole leaves (256) | slices of 16 | 8:
+// FP32, leaf size 64: 287 cells .170 | .117 | .102, 684 .218 | .146 | .155, 1237 .302 | .237 |
+// .256, 1977 .364 | .319 | .360, 3234 .443 | .453 | .539, 6128 .722 | .736 | .904. FP64, where
+// staging hides behind the arithmetic, whole | 8 | 4: 287 cells 3.67 | 1.28 | 1.01, 684 5.88 |
+// 3.33 | 3.20, 1237 10.7 | 7.61 | 7.71, 3234 20.4 | 18.8 | 19.2, 6128 37.1 | 34.1 | 34.8, 62640
+// 94.3 | 92.8 | 95.3.
 constexpr int kFewCells = 2048;
 int leaf_target_slice(int ncells, bool fp32) {
     if (fp32) return ncells < kFewCells ? 8 : kMaxLeaf;
