@@ -6,7 +6,9 @@
 // counters), so equal keys keep their order, and learns where the tile's digits
 // go from a decoupled look-back over the earlier tiles' published counts: one
 // thread per digit, four records at a time. Every key is read and written once
-// per pass.
+// per pass. (Decoupled look-back: Merrill and Garland, "Single-pass parallel prefix
+// scan with decoupled look-back", 2016; one sweep per digit: Adinets and Merrill,
+// "Onesweep: a faster least significant digit radix sort for GPUs", 2022.)
 //
 // What bounds it: ranking and the scattered writes where there are many tiles;
 // the launch where there are few. With a histogram, its scan (one or three
